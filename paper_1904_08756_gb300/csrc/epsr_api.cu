@@ -166,7 +166,12 @@ struct epsr_box {
     int *gc_count = nullptr, *gc_offset = nullptr, *gc_block = nullptr;
     uint4 *gc_scaled = nullptr;
     int4 *gc_coords = nullptr;
-    std::vector<long long> tile_lo, tile_hi;
+    // clusters of 32 atoms in Hilbert order (pair histogram)
+    std::vector<ClBox> cl_box_h;
+    ClBox *cl_box = nullptr;
+    int *cl_su_box = nullptr;
+    ClScratch cl{};
+    long long n_cl = 0;
     // partner slices in global memory, for boxes whose slices do not fit in shared memory
     int4 *slice_g = nullptr;
     unsigned short *home_g = nullptr;
@@ -180,7 +185,9 @@ struct epsr_box {
                         sorted_scaled, sorted_coords, moves, mc_sort.count, mc_sort.offset,
                         mc_sort.block, mc_sort.key, mc_sort.rank, mc_sort.index, pos_of,
                         ep_F, ep_Y, ep_C, ep_Q, lambda, smear_acc, slice_g, home_g,
-                        gc_items, gc_count, gc_offset, gc_block, gc_scaled, gc_coords};
+                        gc_items, gc_count, gc_offset, gc_block, gc_scaled, gc_coords,
+                        cl_box, cl_su_box, cl.count, cl.offset, cl.block, cl.coords,
+                        cl.cl_c, cl.cl_h, cl.su_c, cl.su_h};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     }
@@ -519,14 +526,30 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         bx.gc0 = h->total_gcells;
         h->total_gcells += bx.gc_n ? bx.gc_n * bx.gc_n * bx.gc_n : 1;
         for (int c = 0; c < bx.gc_n * bx.gc_n * bx.gc_n; ++c) h->gc_items_h.push_back(GcItem{b, c});
+        // clusters: about 3 A Hilbert cells (a power of two per side, at most one cell per atom)
+        ClBox cb;
+        memset(&cb, 0, sizeof(cb));
+        while (cb.bits < 7 && (1LL << (3 * (cb.bits + 1))) <= bx.n_atoms) ++cb.bits;
+        cb.key0 = h->cl.n_keys;
+        h->cl.n_keys += 1 << (3 * cb.bits);
+        cb.cl0 = (int)h->n_cl;
+        cb.n_cl = (bx.n_atoms + 31) / 32;
+        cb.su0 = h->cl.n_su;
+        cb.n_su = (cb.n_cl + 31) / 32;
+        cb.r_fx = (int)std::min(std::ceil(std::sqrt((double)bx.tmax)) + 2.0, 1073741824.0);
+        h->n_cl += cb.n_cl;
+        h->cl.n_su += cb.n_su;
+        h->cl_box_h.push_back(cb);
     }
+    std::vector<int> su_box;
+    for (int b = 0; b < n_boxes; ++b) su_box.insert(su_box.end(), h->cl_box_h[b].n_su, b);
+    h->cl.n_keys_pad = (h->cl.n_keys + 3) & ~3;
+    h->cl.n_boxes = n_boxes;
     // g(r) work list: upper triangle of tile pairs per box
     for (int b = 0; b < n_boxes; ++b) {
         const int nt = (h->hb[b].n_atoms + kGrTile - 1) / kGrTile;
-        h->tile_lo.push_back((long long)h->tiles_h.size());
         for (int i = 0; i < nt; ++i)
             for (int j = i; j < nt; ++j) h->tiles_h.push_back(GrTile{b, i, j, 0});
-        h->tile_hi.push_back((long long)h->tiles_h.size());
     }
     // per-atom arrays
     std::vector<int4> c4(atom0);
@@ -565,10 +588,21 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         (rc = dalloc(&h->gc_count, (size_t)h->total_gcells + 1)) ||
         (rc = dalloc(&h->gc_offset, (size_t)h->total_gcells + 1)) ||
         (rc = dalloc(&h->gc_block, ((size_t)h->total_gcells + 1 + 1023) / 1024)) ||
-        (rc = dalloc(&h->gc_scaled, atom0)) || (rc = dalloc(&h->gc_coords, atom0))) {
+        (rc = dalloc(&h->gc_scaled, atom0)) || (rc = dalloc(&h->gc_coords, atom0)) ||
+        (rc = dalloc(&h->cl_box, n_boxes)) || (rc = dalloc(&h->cl_su_box, su_box.size())) ||
+        (rc = dalloc(&h->cl.count, (size_t)h->cl.n_keys_pad + n_boxes)) ||
+        (rc = dalloc(&h->cl.offset, h->cl.n_keys)) ||
+        (rc = dalloc(&h->cl.block, ((size_t)h->cl.n_keys + 1023) / 1024)) || (rc = dalloc(&h->cl.coords, atom0)) ||
+        (rc = dalloc(&h->cl.cl_c, (size_t)h->n_cl)) || (rc = dalloc(&h->cl.cl_h, (size_t)h->n_cl)) ||
+        (rc = dalloc(&h->cl.su_c, h->cl.n_su)) || (rc = dalloc(&h->cl.su_h, h->cl.n_su))) {
         delete h;
         return rc;
     }
+    h->cl.box = h->cl_box;
+    h->cl.su_box = h->cl_su_box;
+    h->cl.key = h->sort.key;             // per-atom scratch shared with the all-pairs order
+    h->cl.rank = h->sort.rank;
+    h->cl.index = h->sort.index;
 #define CKD(call)                                                            \
     do {                                                                     \
         cudaError_t e_ = (call);                                             \
@@ -583,6 +617,8 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
     CKD(cudaMemcpyAsync(h->tiles, h->tiles_h.data(), h->tiles_h.size() * sizeof(GrTile), cudaMemcpyHostToDevice, stream));
     if (!h->gc_items_h.empty())
         CKD(cudaMemcpyAsync(h->gc_items, h->gc_items_h.data(), h->gc_items_h.size() * sizeof(GcItem), cudaMemcpyHostToDevice, stream));
+    CKD(cudaMemcpyAsync(h->cl_box, h->cl_box_h.data(), n_boxes * sizeof(ClBox), cudaMemcpyHostToDevice, stream));
+    CKD(cudaMemcpyAsync(h->cl_su_box, su_box.data(), su_box.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->hist_box, h->hist_box_h.data(), n_boxes * sizeof(long long), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemsetAsync(h->stats, 0, n_boxes * sizeof(epsr_mc_stats), stream));
     CKD(cudaMemsetAsync(h->status, 0, sizeof(int), stream));
@@ -994,45 +1030,46 @@ extern "C" int epsr_partial_gr_range(epsr_box *box, int64_t tile_begin, int64_t 
     return gr_range(box, tile_begin, tile_end, hist, (cudaStream_t)stream);
 }
 
+// Traversal of every box's clusters, set up for the current coordinates.
+static ClArgs cl_args(epsr_box *box, int warps)
+{
+    ClArgs a;
+    memset(&a, 0, sizeof(a));
+    a.boxes = box->boxes;
+    a.box = box->cl_box;
+    a.coords = box->cl.coords;
+    a.cl_c = box->cl.cl_c;
+    a.cl_h = box->cl.cl_h;
+    a.su_c = box->cl.su_c;
+    a.su_h = box->cl.su_h;
+    a.next_item = box->cl.count + box->cl.n_keys_pad;
+    a.thresholds = box->thresholds;
+    a.n_cl_total = box->n_cl;
+    a.n_boxes = box->n_boxes;
+    // at least four items per warp, so that the last ones to finish idle the chip little; more
+    // shares repeat the box tests of a cluster
+    while (a.plog < 5 && (box->n_cl << a.plog) < 4LL * warps) ++a.plog;
+    for (const auto &b : box->hb) a.hist_cap = std::max(a.hist_cap, b.n_types * b.n_types * b.n_bins);
+    return a;
+}
+
+// The histogram of every box: the clusters' near pairs, or (histograms beyond shared memory) all
+// pairs tile by tile.
+static int gr_all(epsr_box *box, uint64_t *hist, cudaStream_t s)
+{
+    const int grid = box->sms * box->gr_ctas_per_sm;
+    ClArgs a = cl_args(box, grid * 8);
+    if (gr_clusters_smem(a.hist_cap) > (size_t)kClMaxSmem) return gr_range(box, 0, (long long)box->tiles_h.size(), hist, s);
+    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, s);
+    if (rc) return rc;
+    a.hist = (unsigned long long *)hist;
+    return launch_gr_clusters(a, grid, s);
+}
+
 extern "C" int epsr_partial_gr_cells(epsr_box *box, uint64_t *hist, float *g, int64_t n_configs,
                                      epsr_stream_t stream)
 {
-    if (!box || !hist) return set_error(EPSR_EINVAL, "NULL argument");
-    if (g && n_configs < 1) return set_error(EPSR_EINVAL, "n_configs must be >= 1");
-    cudaStream_t s = (cudaStream_t)stream;
-    int rc = EPSR_OK;
-    if (!box->gc_items_h.empty()) {
-        rc = launch_scale_coords(box->boxes, box->atom_box, box->coords, box->scaled, box->n_atoms, s);
-        if (rc) return rc;
-        SortScratch sc = box->sort;          // per-atom scratch shared with the all-pairs order
-        sc.count = box->gc_count;
-        sc.offset = box->gc_offset;
-        sc.block = box->gc_block;
-        rc = launch_spatial_sort(box->boxes, box->atom_box, box->scaled, box->coords, box->n_atoms,
-                                 box->total_gcells + 1, 2, sc, box->gc_scaled, box->gc_coords, nullptr, s);
-        if (rc) return rc;
-        GcArgs a;
-        a.boxes = box->boxes;
-        a.coords = box->gc_coords;
-        a.scaled = box->gc_scaled;
-        a.cell_start = box->gc_offset;
-        a.cell_count = box->gc_count;
-        a.thresholds = box->thresholds;
-        a.items = box->gc_items;
-        a.n_items = (long long)box->gc_items_h.size();
-        a.hist = (unsigned long long *)hist;
-        a.max_pairs_bins = box->ep_cap;
-        a.max_bins1 = box->tbl_cap;
-        const int grid = (int)std::min<long long>(a.n_items, (long long)box->sms * 8);
-        rc = launch_partial_gr_cells(a, std::max(grid, 1), s);
-        if (rc) return rc;
-    }
-    // boxes too small for three cells per side: the all-pairs tiles of those boxes
-    for (int b = 0; b < box->n_boxes; ++b)
-        if (box->hb[b].gc_n == 0 && (rc = gr_range(box, box->tile_lo[b], box->tile_hi[b], hist, s)))
-            return rc;
-    if (g) return epsr_normalize_g(box, hist, g, n_configs, stream);
-    return EPSR_OK;
+    return epsr_partial_gr(box, hist, g, n_configs, stream);
 }
 
 extern "C" int epsr_normalize_g(epsr_box *box, const uint64_t *hist, float *g, int64_t n_configs,
@@ -1048,7 +1085,7 @@ extern "C" int epsr_partial_gr(epsr_box *box, uint64_t *hist, float *g, int64_t 
 {
     if (!box || !hist) return set_error(EPSR_EINVAL, "NULL argument");
     if (g && n_configs < 1) return set_error(EPSR_EINVAL, "n_configs must be >= 1");
-    int rc = gr_range(box, 0, (long long)box->tiles_h.size(), hist, (cudaStream_t)stream);
+    int rc = gr_all(box, hist, (cudaStream_t)stream);
     if (rc) return rc;
     if (g) return epsr_normalize_g(box, hist, g, n_configs, stream);
     return EPSR_OK;

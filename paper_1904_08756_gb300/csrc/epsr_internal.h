@@ -123,21 +123,50 @@ struct GcItem {
     int box, cell;
 };
 
-struct GcArgs {
-    const BoxDev *boxes;
-    const int4 *coords;          // [n_atoms_total] in cell-list order
-    const uint4 *scaled;         // [n_atoms_total] in cell-list order
-    const int *cell_start;       // [total cells + 1] first sorted position of each cell
-    const int *cell_count;       // [total cells]
-    const long long *thresholds;
-    const GcItem *items;
-    long long n_items;
-    unsigned long long *hist;
-    int max_pairs_bins, max_bins1;
-};
 
-int launch_partial_gr_cells(const GcArgs &args, int grid, cudaStream_t stream);
 constexpr int kMcCells = 512;    // cells per (type, CTA) block of the Monte Carlo order
+
+// ---- clusters of 32 atoms in Hilbert order (clusters.cuh) ------------------------------------
+struct ClBox {            // one box
+    int cl0, n_cl;        // first cluster and number of clusters
+    int su0, n_su;        // the same of super-clusters (32 clusters)
+    int key0, bits;       // first sort key; bits per axis of the Hilbert cells
+    int r_fx;             // histogram range in grid units, rounded up (at most 2^30)
+    int pad;
+};
+struct ClScratch {        // device buffers of one handle
+    const ClBox *box;
+    const int *su_box;    // box of every super-cluster
+    int *count;           // [n_keys_pad], then the work counters [n_boxes]
+    int *offset, *block;  // [n_keys], [ceil(n_keys / 1024)]
+    int *key, *rank, *index;
+    int4 *coords;         // coordinates in cluster order
+    int4 *cl_c, *cl_h;    // cluster boxes: centre and atom count; half widths and first position
+    int4 *su_c, *su_h;    // super-cluster boxes
+    int n_keys, n_keys_pad, n_boxes, n_su;
+};
+struct ClArgs {           // one traversal
+    const BoxDev *boxes;
+    const ClBox *box;
+    const int4 *coords, *cl_c, *cl_h, *su_c, *su_h;
+    int *next_item;       // [n_boxes] next unclaimed work item
+    const long long *thresholds;
+    unsigned long long *hist;
+    long long n_cl_total;
+    int n_boxes;
+    int plog;             // a cluster's partners are split into 2^plog work items
+    int hist_cap;         // max over boxes of n_types^2 * n_bins
+};
+constexpr int kClMaxSmem = 200 * 1024;
+size_t gr_clusters_smem(int hist_cap);
+int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords, long long n, const ClScratch &sc,
+                    cudaStream_t stream);
+int launch_gr_clusters(const ClArgs &args, int grid, cudaStream_t stream);
+// exclusive scan of n counts (block: scratch [ceil(n / 1024)]), and the scatter of a counting sort
+int launch_scan(const int *count, int n, int *offset, int *block, cudaStream_t stream);
+int launch_scan_one(const int *count, int n, int *offset, cudaStream_t stream);
+int launch_scatter(const int *key, const int *rank, const int *offset, int *index, long long n, cudaStream_t stream);
+constexpr int kScanOneMax = 1 << 18;   // counts scanned by the one-launch form at most
 
 int launch_scale_coords(const BoxDev *boxes, const int *atom_box, const int4 *coords,
                         uint4 *scaled, long long n, cudaStream_t stream);
