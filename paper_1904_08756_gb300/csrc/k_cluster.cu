@@ -199,32 +199,39 @@ int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords
 constexpr int kClThreads = 256;
 constexpr int kClWarps = kClThreads / 32;
 
-struct GrBin {
-    const long long *T;
-    const int4 *coords;
-    unsigned *hist;
-    float inv, tmax_hi;
-    long long tmax;
-    int L, nb;
-};
-
-// Exact bin of a pair at integer separations sp (out of the main loop: about one pair in 10^3).
-__device__ __noinline__ void gr_count_exact(const GrBin &G, int4 pi, int4 pj, int row)
+// Exact bin of a pair of grid points (off the main path: about one pair in 10^3), counted in
+// the row of its ordered types.
+__device__ __noinline__ void gr_count_exact(unsigned *row, const long long *T, long long tmax, float inv, int L, int nb,
+                                            int4 pi, int4 pj)
 {
-    const Sep sp = sep(pi, pj, G.L);
+    const Sep sp = sep(pi, pj, L);
     const long long d2 = d2_of(sp);
-    if (d2 < G.tmax) atomicAdd(&G.hist[row + bin_of(d2, g2_of(sp), G.T, G.nb, G.inv)], 1u);
+    if (d2 < tmax) atomicAdd(&row[bin_of(d2, g2_of(sp), T, nb, inv)], 1u);
 }
 
-// Bin of a squared distance g2 < tmax_hi: false when it lies too close to an edge to tell.
-__device__ __forceinline__ bool gr_count(const GrBin &G, float g2, int row)
+// Two squared distances at once: the distances in bins less a half (u), rounded to integers in
+// the low bits of t; lane q of `sure` is set when the bin of distance q is certain.
+struct Bins2 {
+    int k0, k1;
+    bool sure0, sure1;
+};
+__device__ __forceinline__ Bins2 bins2(float g0, float g1, uint64_t INV)
 {
-    const float u = fmaf(sqrt_approx(g2), G.inv, -0.5f);             // distance in bins, less a half
-    const float t = u + 12582912.f;                                 // rounded to an integer in the low bits
-    const float d = u - (t - 12582912.f);
-    if (!(fabsf(d) < fmaf(u, -0x1p-20f, 0.5f - 0x1p-20f))) return false;
-    atomicAdd(&G.hist[row + (__float_as_int(t) - 0x4B400000)], 1u);
-    return true;
+    const uint64_t M = pk2(12582912.f, 12582912.f), NM = pk2(-12582912.f, -12582912.f);
+    const uint64_t U = fma2(pk2(sqrt_approx(g0), sqrt_approx(g1)), INV, pk2(-0.5f, -0.5f));
+    const uint64_t T = add2(U, M);
+    const uint64_t D = sub2(U, add2(T, NM));
+    const uint64_t E = fma2(U, pk2(-0x1p-20f, -0x1p-20f), pk2(0.5f - 0x1p-20f, 0.5f - 0x1p-20f));
+    float t0, t1, d0, d1, e0, e1;
+    upk2(T, t0, t1);
+    upk2(D, d0, d1);
+    upk2(E, e0, e1);
+    Bins2 b;
+    b.k0 = __float_as_int(t0) - 0x4B400000;
+    b.k1 = __float_as_int(t1) - 0x4B400000;
+    b.sure0 = fabsf(d0) < e0;
+    b.sure1 = fabsf(d1) < e1;
+    return b;
 }
 
 __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
@@ -241,16 +248,8 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
         const BoxDev &bx = A.boxes[b];
         const ClBox cb = A.box[b];
         const int L = bx.L, nt = bx.n_types, nb = bx.n_bins;
-        const float r2 = bx.tmax_hi * 1.0001f;
-        GrBin G;
-        G.T = A.thresholds + bx.tbl_off;
-        G.coords = A.coords;
-        G.hist = s_hist;
-        G.inv = bx.inv_dr_fx;
-        G.tmax_hi = bx.tmax_hi;
-        G.tmax = bx.tmax;
-        G.L = L;
-        G.nb = nb;
+        const float hi = bx.tmax_hi, r2 = hi * 1.0001f, inv = bx.inv_dr_fx;
+        const uint64_t INV = pk2(inv, inv);
         const int n_items = cb.n_cl << A.plog;
         for (;;) {
             int it = 0;
@@ -259,18 +258,22 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
             if (it >= n_items) break;
             const int ci = it >> A.plog, part = it & ((1 << A.plog) - 1);
             const ICluster I = load_icluster(A, cb.cl0 + ci, L, cb.r_fx, lane);
-            const int rowi = I.p.w * nt * nb;
+            unsigned *rowi = s_hist + I.p.w * nt * nb;
+            // one pair by its grid coordinates
+            auto count = [&](int4 pj, int row) {
+                const float g2 = g2_of(sep(I.p, pj, L));
+                if (g2 >= hi) return;
+                const Bins2 k = bins2(g2, g2, INV);
+                if (k.sure0) atomicAdd(&rowi[row + k.k0], 1u);
+                else gr_count_exact(rowi + row, A.thresholds + bx.tbl_off, bx.tmax, inv, L, nb, I.p, pj);
+            };
             if (part == 0) {
                 // pairs inside the cluster: lane i with lane i + o, o = 1 .. 16
                 for (int o = 1; o <= 16; ++o) {
                     const int src = (lane + o) & 31;
                     const int4 pj = make_int4(__shfl_sync(0xffffffffu, I.p.x, src), __shfl_sync(0xffffffffu, I.p.y, src),
                                               __shfl_sync(0xffffffffu, I.p.z, src), __shfl_sync(0xffffffffu, I.p.w, src));
-                    if (lane < I.c.w && src < I.c.w && (o < 16 || lane < 16)) {
-                        const float g2 = g2_of(sep(I.p, pj, L));
-                        const int row = rowi + pj.w * nb;
-                        if (g2 < G.tmax_hi && !gr_count(G, g2, row)) gr_count_exact(G, I.p, pj, row);
-                    }
+                    if (lane < I.c.w && src < I.c.w && (o < 16 || lane < 16)) count(pj, pj.w * nb);
                 }
             }
             auto value = [nb](const int4 &q) { return __int_as_float(q.w * nb); };
@@ -286,12 +289,17 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
                         const uint64_t DX = sub2(pk2(a.x, a.y), XI), DY = sub2(pk2(a.z, a.w), YI), DZ = sub2(pk2(c.x, c.y), ZI);
                         float g0, g1;
                         upk2(fma2(DX, DX, fma2(DY, DY, mul2(DZ, DZ))), g0, g1);
-                        bool e0 = false, e1 = false;
-                        const int r0 = rowi + __float_as_int(c.z), r1 = rowi + __float_as_int(c.w);
-                        if (g0 < G.tmax_hi) e0 = !gr_count(G, g0, r0);
-                        if (g1 < G.tmax_hi) e1 = !gr_count(G, g1, r1);
-                        if (e0) gr_count_exact(G, I.p, A.coords[l.idx[2 * q]], r0);
-                        if (e1) gr_count_exact(G, I.p, A.coords[l.idx[2 * q + 1]], r1);
+                        const Bins2 k = bins2(g0, g1, INV);
+                        const bool in0 = g0 < hi, in1 = g1 < hi;
+                        const int r0 = __float_as_int(c.z), r1 = __float_as_int(c.w);
+                        if (in0 && k.sure0) atomicAdd(&rowi[r0 + k.k0], 1u);
+                        if (in1 && k.sure1) atomicAdd(&rowi[r1 + k.k1], 1u);
+                        const bool x0 = in0 && !k.sure0, x1 = in1 && !k.sure1;
+                        if (x0 || x1) {
+                            const long long *T = A.thresholds + bx.tbl_off;
+                            if (x0) gr_count_exact(rowi + r0, T, bx.tmax, inv, L, nb, I.p, A.coords[l.idx[2 * q]]);
+                            if (x1) gr_count_exact(rowi + r1, T, bx.tmax, inv, L, nb, I.p, A.coords[l.idx[2 * q + 1]]);
+                        }
                     }
                 });
             } else {
@@ -300,10 +308,8 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
                     for (int s = 0; s < n; ++s) {
                         const float *pa = reinterpret_cast<const float *>(&l.a[s >> 1]) + (s & 1);
                         const float *pb = reinterpret_cast<const float *>(&l.b[s >> 1]) + (s & 1);
-                        const int4 pj = make_int4(__float_as_int(pa[0]), __float_as_int(pa[2]), __float_as_int(pb[0]), 0);
-                        const float g2 = g2_of(sep(I.p, pj, L));
-                        const int row = rowi + __float_as_int(pb[2]);
-                        if (g2 < G.tmax_hi && !gr_count(G, g2, row)) gr_count_exact(G, I.p, pj, row);
+                        count(make_int4(__float_as_int(pa[0]), __float_as_int(pa[2]), __float_as_int(pb[0]), 0),
+                              __float_as_int(pb[2]));
                     }
                 });
             }
