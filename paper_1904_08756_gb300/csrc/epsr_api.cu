@@ -117,8 +117,7 @@ struct epsr_box {
     std::vector<GrTile> tiles_h;
     int sms = 0;
     int mc_batch = 0;                         // 0: chosen per box by the kernel
-    int cell_margin = 1 << 20;                // 1 A on the 2^20 grid
-    int esc_cap = -1;                         // -1: the kernel's maximum
+    bool near_all = false;                    // no box queries: every chunk of partners is near
     int mc_ctas = 0;
     int gr_ctas_per_sm = 4;                   // persistent CTAs per SM of the all-pairs histogram
     int fault_cta = -1;
@@ -174,7 +173,6 @@ struct epsr_box {
     long long n_cl = 0;
     // partner slices in global memory, for boxes whose slices do not fit in shared memory
     int4 *slice_g = nullptr;
-    unsigned short *home_g = nullptr;
     size_t slice_g_cap = 0;
 
     ~epsr_box()
@@ -184,7 +182,7 @@ struct epsr_box {
                         sort.count, sort.offset, sort.block, sort.key, sort.rank, sort.index,
                         sorted_scaled, sorted_coords, moves, mc_sort.count, mc_sort.offset,
                         mc_sort.block, mc_sort.key, mc_sort.rank, mc_sort.index, pos_of,
-                        ep_F, ep_Y, ep_C, ep_Q, lambda, smear_acc, slice_g, home_g,
+                        ep_F, ep_Y, ep_C, ep_Q, lambda, smear_acc, slice_g,
                         gc_items, gc_count, gc_offset, gc_block, gc_scaled, gc_coords,
                         cl_box, cl_su_box, cl.count, cl.offset, cl.block, cl.coords,
                         cl.cl_c, cl.cl_h, cl.su_c, cl.su_h};
@@ -320,7 +318,8 @@ static void plan_mc_groups(epsr_box *h)
     h->total_mc_cells = 0;
     std::vector<int> G(nb, 1);
     if (nb == 1) {
-        long long want = (h->hb[0].n_atoms + 511) / 512;
+        const int least = h->mc_ctas > 0 ? 64 : 512;
+        long long want = (h->hb[0].n_atoms + least - 1) / least;
         G[0] = (int)std::max(1LL, std::min<long long>(want, budget));
     } else {
         // every box starts with one CTA; each further CTA goes to the box whose per-CTA
@@ -343,38 +342,50 @@ static void plan_mc_groups(epsr_box *h)
         BoxDev &b = h->hb[i];
         b.cta0 = c0;
         b.n_cta = G[i];
-        // slice capacity: the most atoms any CTA gets (atom j goes to CTA j mod G)
-        const long long cap = (b.n_atoms + G[i] - 1) / G[i];
-        b.chunk = (int)cap;
+        b.mc_bits = h->cl_box_h[i].bits;
         b.mc_cell0 = h->total_mc_cells;
-        h->total_mc_cells += b.n_types * G[i] * kMcCells;
+        h->total_mc_cells += b.n_types << (3 * b.mc_bits);
         c0 += G[i];
     }
     h->cta_box_len = c0;
 }
 
-// Shared-memory layout of the sweep for the current CTA split: thresholds, EP table, cell
-// index [types][513] (uint32), correction items, and, when they fit, the partner slice (int4 per
-// slot, and its copy on the 2^32-periodic grid) and the home cell of every slot (uint16); otherwise the slices and home cells live in
-// global memory and a chunk of partners is staged.
+// Shared-memory layout of the sweep for the current CTA split: thresholds, EP table, correction
+// tables, chunk boxes and near masks, and, when they fit, the partner slice (int4 per slot, and its
+// copy on the 2^32-periodic grid); otherwise the slices live in global memory, a part of the copy is
+// staged, and chunks double until their masks take at most kMcMaxWords words.
 struct McLayout {
-    int slice_cap = 0, types_cap = 1;
+    int slice_cap = 0, words_cap = 1, chunk_log = 5;
     size_t smem = 0;
     bool gslice = false;
 };
 
 static int mc_layout(const epsr_box *h, McLayout *L)
 {
-    for (auto &b : h->hb) L->slice_cap = std::max(L->slice_cap, b.chunk);
-    for (auto &b : h->hb) L->types_cap = std::max(L->types_cap, b.n_types);
-    const size_t tables = (size_t)h->tbl_cap * sizeof(long long) + (size_t)h->ep_cap * sizeof(float) +
-                          (size_t)L->types_cap * (kMcCells + 1) * sizeof(unsigned) +
-                          (size_t)kMcBatchMax * kMcBatchMax * sizeof(float) + (size_t)kMcCorrItems * sizeof(float);
-    const size_t per_slot = 2 * sizeof(int4) + sizeof(unsigned short);   // slot, its 2^32-grid copy, home cell
-    L->smem = (((size_t)L->slice_cap * per_slot + tables) + 15) & ~(size_t)15;
+    auto sizes = [&](int cs) {
+        L->chunk_log = cs;
+        L->slice_cap = 0;
+        L->words_cap = 1;
+        for (auto &b : h->hb) {
+            int slots = 0, words = 0;
+            for (int t = 0; t < b.n_types; ++t) {
+                const int n = (int)((b.count[t] + b.n_cta - 1) / b.n_cta), nc = (n + (1 << cs) - 1) >> cs;
+                slots += nc << cs;
+                words += (nc + 31) / 32;
+            }
+            L->slice_cap = std::max(L->slice_cap, slots);
+            L->words_cap = std::max(L->words_cap, words);
+        }
+        return (size_t)h->tbl_cap * sizeof(long long) + (size_t)h->ep_cap * sizeof(float) +
+               (size_t)kMcBatchMax * kMcBatchMax * sizeof(float) + (size_t)kMcCorrItems * sizeof(float) +
+               (size_t)L->words_cap * (32 * 6 * sizeof(int) + kMcBatchMax * sizeof(unsigned));
+    };
+    size_t tables = sizes(5);
+    L->smem = ((size_t)L->slice_cap * 2 * sizeof(int4) + tables + 15) & ~(size_t)15;
     L->gslice = L->smem > kMcMaxDynSmem;
     if (L->gslice) {
-        L->smem = ((tables + 15) & ~(size_t)15) + (size_t)kMcStageChunk * sizeof(int4);
+        for (int cs = 5; L->words_cap > kMcMaxWords && cs < 11; ) tables = sizes(++cs);
+        L->smem = ((size_t)kMcStageChunk * sizeof(uint4) + tables + 15) & ~(size_t)15;
         if (L->smem > kMcMaxDynSmem)
             return set_error(EPSR_EINVAL, "mc sweep: %zu bytes of tables per CTA (limit %zu)", L->smem, kMcMaxDynSmem);
     }
@@ -392,12 +403,9 @@ static int alloc_mc_slices(epsr_box *h)
     const size_t slots = (size_t)h->cta_box_len * L.slice_cap;
     if (h->slice_g_cap >= slots) return EPSR_OK;
     if (h->slice_g) cudaFree(h->slice_g);
-    if (h->home_g) cudaFree(h->home_g);
     h->slice_g = nullptr;
-    h->home_g = nullptr;
     h->slice_g_cap = 0;
     rc = dalloc(&h->slice_g, slots);
-    if (!rc) rc = dalloc(&h->home_g, slots);
     if (rc) return rc;
     h->slice_g_cap = slots;
     return EPSR_OK;
@@ -856,8 +864,7 @@ extern "C" int epsr_mc_set_cells(epsr_box *box, int32_t margin_fx, int32_t escap
     for (const auto &b : box->hb)
         if (margin_fx >= b.L / 4)
             return set_error(EPSR_EINVAL, "mc cells: margin %d not below a quarter of box side %d", margin_fx, b.L);
-    box->cell_margin = margin_fx;
-    box->esc_cap = escapee_cap;
+    box->near_all = escapee_cap == 0;
     return EPSR_OK;
 }
 
@@ -896,7 +903,7 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     McLayout lay;
     int rcl = mc_layout(box, &lay);
     if (rcl) return rcl;
-    const int slice_cap = lay.slice_cap, types_cap = lay.types_cap;
+    const int slice_cap = lay.slice_cap;
     const size_t smem = lay.smem;
     const bool gslice = lay.gslice;
     if (gslice && box->slice_g_cap < (size_t)box->cta_box_len * slice_cap)
@@ -907,14 +914,13 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     int rc0 = launch_scale_coords(box->boxes, box->atom_box, box->coords, box->scaled, box->n_atoms, s);
     if (!rc0)
         rc0 = launch_spatial_sort(box->boxes, box->atom_box, box->scaled, box->coords, box->n_atoms,
-                                  box->total_mc_cells + 1, 1, box->mc_sort, nullptr, nullptr,
+                                  box->total_mc_cells, 1, box->mc_sort, nullptr, nullptr,
                                   box->pos_of, s);
     if (rc0) return rc0;
     McArgs a;
     memset(&a, 0, sizeof(a));
-    a.sorted_index = box->mc_sort.index;
+    a.sorted_index = box->mc_sort.rank;
     a.pos_of = box->pos_of;
-    a.mc_offset = box->mc_sort.offset;
     a.boxes = box->boxes;
     a.coords = box->coords;
     a.mol_start = box->mol_start;
@@ -937,11 +943,10 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     a.slice_cap = slice_cap;
     a.tbl_cap = box->tbl_cap;
     a.ep_cap = box->ep_cap;
-    a.types_cap = types_cap;
     a.slice_g = gslice ? box->slice_g : nullptr;
-    a.home_g = gslice ? box->home_g : nullptr;
-    a.cell_margin = box->cell_margin;
-    a.esc_cap = box->esc_cap < 0 ? mc_escapee_max() : box->esc_cap;
+    a.chunk_log = lay.chunk_log;
+    a.words_cap = lay.words_cap;
+    a.near_all = box->near_all ? 1 : 0;
     a.skip_arrival_cta = box->fault_cta;
     a.moves = box->moves;
     a.chunk = chunk;
@@ -1494,7 +1499,7 @@ static SmearArgs smear_args(epsr_box *box, double sigma)
     SmearArgs a;
     memset(&a, 0, sizeof(a));
     a.boxes = box->boxes;
-    a.index = box->sort.index;
+    a.index = smear_uses_cells(box, sigma) ? box->sort.index : box->sort.rank;
     a.sigma = sigma;
     a.max_pairs_bins = box->ep_cap;
     if (smear_uses_cells(box, sigma)) {

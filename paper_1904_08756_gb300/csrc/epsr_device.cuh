@@ -41,7 +41,6 @@ struct BoxDev {
     int32_t ep_off;       // offset of the n_pairs * n_bins empirical potential
     int32_t has_ep;       // 0 while the empirical potential is identically zero
     int32_t cta0, n_cta;  // CTA group of the Monte Carlo kernel
-    int32_t chunk;        // partner atoms per CTA of the group
     double h_rot;         // tan(max_rotation / 2) / sqrt(3)
     double kT;            // kJ/mol
     double volume;        // A^3
@@ -58,6 +57,7 @@ struct BoxDev {
     int32_t cell0;        // first global cell of this box (spatial sort)
     int32_t cells_p3;     // cells per box in the sort key space (power of two cubed)
     int32_t mc_cell0;     // first key of this box in the type-major sort
+    int32_t mc_bits;      // bits per axis of its Hilbert cells
     int32_t near_fx;      // ceil(sqrt(max(rc2, tmax if an EP is set, lj2 if LJ is cut))), grid units
     int32_t lj_cut;       // 1: Lennard-Jones truncated at d2 < lj2; 0: over every pair
     int64_t lj2;          // (llround(r_lj * S))^2, grid units^2
@@ -149,6 +149,27 @@ __device__ __forceinline__ int bin_of(long long d2, float g2, const long long *T
     while (k > 0 && T[k] > d2) --k;
     while (T[k + 1] <= d2) ++k;
     return k;
+}
+
+// Empirical potential at a separation with g2 < tmax_hi: the bin from the FP32 squared distance
+// (the root with relative error 2^-23, g2 with 2^-22), the exact one only within x 2^-20 of a
+// bin edge, the table's end included.
+static __device__ __noinline__ float ep_at_exact(const float *row, float g2, Sep s, const long long *T, long long tmax, int n_bins,
+                                          float inv_dr_fx)
+{
+    const long long d2 = d2_of(s);
+    return d2 < tmax ? row[bin_of(d2, g2, T, n_bins, inv_dr_fx)] : 0.f;
+}
+
+__device__ __forceinline__ float ep_at(const float *row, float g2, Sep s, const BoxDev &bx, const long long *T)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g2));
+    const float u = fmaf(r, bx.inv_dr_fx, -0.5f);
+    const float t = u + 12582912.f;                          // u rounded to an integer in the low bits
+    const float d = u - (t - 12582912.f);
+    if (fabsf(d) < fmaf(u, -0x1p-20f, 0.5f - 0x1p-20f)) return row[__float_as_int(t) - 0x4B400000];
+    return ep_at_exact(row, g2, s, T, bx.tmax, bx.n_bins, bx.inv_dr_fx);
 }
 
 // A pair row whose Lennard-Jones term reaches every partner (LJ not cut): evaluated against
@@ -263,12 +284,10 @@ __device__ __forceinline__ float pair_du(Sep sn, Sep so, const PairRow &pr, cons
     } else if (co) {
         du = fmaf(-pr.kqq, ao, du);
     }
-    if (bx.has_ep && (g2n < bx.tmax_hi || g2o < bx.tmax_hi)) {
+    if (bx.has_ep) {
         const float *row = ep + pr.pair * bx.n_bins;
-        if (below(g2n, sn, bx.tmax, bx.tmax_lo, bx.tmax_hi))
-            du += row[bin_of(d2_of(sn), g2n, T, bx.n_bins, bx.inv_dr_fx)];
-        if (below(g2o, so, bx.tmax, bx.tmax_lo, bx.tmax_hi))
-            du -= row[bin_of(d2_of(so), g2o, T, bx.n_bins, bx.inv_dr_fx)];
+        if (g2n < bx.tmax_hi) du += ep_at(row, g2n, sn, bx, T);
+        if (g2o < bx.tmax_hi) du -= ep_at(row, g2o, so, bx, T);
     }
     return du;
 }
@@ -355,6 +374,33 @@ struct __align__(16) MoveRec {
     int kind;        // 0 translate every atom, 1 rotate (and translate), 2 translate atom `atom`
     int atom;
 };
+
+// ---- spatial order ----------------------------------------------------------------------------
+// Index of cell (x, y, z), `bits` bits per axis, along the Hilbert curve: the transpose form of
+// J. Skilling, "Programming the Hilbert curve", AIP Conf. Proc. 707 (2004) 381.
+__device__ __forceinline__ unsigned hilbert3(unsigned x, unsigned y, unsigned z, int bits)
+{
+    if (bits == 0) return 0u;
+    for (unsigned q = 1u << (bits - 1); q > 1u; q >>= 1) {       // undo the excess rotations
+        const unsigned p = q - 1u;
+        if (x & q) x ^= p;
+        unsigned t = (x ^ y) & p;
+        if (y & q) x ^= p;
+        else { x ^= t; y ^= t; }
+        t = (x ^ z) & p;
+        if (z & q) x ^= p;
+        else { x ^= t; z ^= t; }
+    }
+    y ^= x;                                                       // Gray code
+    z ^= y;
+    unsigned t = 0u;
+    for (unsigned q = 1u << (bits - 1); q > 1u; q >>= 1)
+        if (z & q) t ^= q - 1u;
+    x ^= t; y ^= t; z ^= t;
+    unsigned h = 0u;
+    for (int b = bits - 1; b >= 0; --b) h = (h << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
+    return h;
+}
 
 // ---- device status word ------------------------------------------------------------------
 constexpr int kStatusTimeout = 1;

@@ -35,7 +35,7 @@ void sq_plan_dims(const epsr_sq_plan *p, int *nQ, int *n_bins, int *max_cols);
 int sq_plan_stages(const epsr_sq_plan *p);
 
 // ---- Monte Carlo kernel ----------------------------------------------------------------------
-constexpr size_t kMcMaxDynSmem = 176 * 1024;   // with about 44 KB of static shared memory, under the 227 KB per CTA
+constexpr size_t kMcMaxDynSmem = 182 * 1024;   // with about 44 KB of static shared memory, under the 227 KB per CTA
 // exchange buffer of the sweep, per parity: the partial dU of every move of a batch from every
 // CTA ([kMcBatchMax][grid]), then kMcSlotStride - kMcBatchMax = kMcCorrPerCta floats per CTA of
 // which a box group uses its first CTA's share onwards for the batch-pair corrections
@@ -45,8 +45,9 @@ constexpr int kMcSlotStride = kMcBatchMax + kMcCorrPerCta;
 // correction items of one batch in shared memory (>= 496 pairs x 8 atoms: batches above 32 moves
 // need 8 or more CTAs per box)
 constexpr int kMcCorrItems = 4096;
-// partners staged per chunk in shared memory when the slices live in global memory
+// partners staged at once in shared memory when the slices live in global memory
 constexpr int kMcStageChunk = 2048;
+constexpr int kMcMaxWords = 24;           // chunk mask words per CTA of such a slice, at most
 
 struct McArgs {
     const BoxDev *boxes;
@@ -63,7 +64,6 @@ struct McArgs {
     const MoveRec *moves;         // [n_boxes][chunk] this launch's moves
     const int *sorted_index;      // [n_atoms_total] atom at each type-major sorted position
     const int *pos_of;            // [n_atoms_total] sorted position of each atom
-    const int *mc_offset;         // [total keys + 1] first sorted position of each key
     long long chunk;              // move-table stride per box
     long long log_off;            // log index of this launch's first move
     int *status;                  // device status word
@@ -78,11 +78,10 @@ struct McArgs {
     int slice_cap;                // int4 capacity of the shared partner slice
     int tbl_cap;                  // capacity (entries) of the shared threshold table
     int ep_cap;                   // capacity (entries) of the shared empirical-potential table
-    int types_cap;                // largest number of atom types of the handle's boxes
     int4 *slice_g;                // [grid][slice_cap] partner slices in global memory, or NULL
-    unsigned short *home_g;       // [grid][slice_cap] home cells of those slots, or NULL
-    int cell_margin;              // drift (grid units) before a partner leaves its cell's queries
-    int esc_cap;                  // escapee list capacity (0: no cell queries)
+    int chunk_log;                // log2 of the slots per chunk (5; more for slices in global memory)
+    int words_cap;                // chunk mask words per CTA, at most
+    int near_all;                 // 1: every chunk is near (no box queries)
     int skip_arrival_cta;         // test hook: this CTA never arrives (-1: none)
 };
 
@@ -123,8 +122,6 @@ struct GcItem {
     int box, cell;
 };
 
-
-constexpr int kMcCells = 512;    // cells per (type, CTA) block of the Monte Carlo order
 
 // ---- clusters of 32 atoms in Hilbert order (clusters.cuh) ------------------------------------
 struct ClBox {            // one box

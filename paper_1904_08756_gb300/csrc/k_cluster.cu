@@ -8,32 +8,6 @@
 
 namespace epsr {
 
-// Index of cell (x, y, z), `bits` bits per axis, along the Hilbert curve: the transpose form of
-// J. Skilling, "Programming the Hilbert curve", AIP Conf. Proc. 707 (2004) 381.
-__device__ __forceinline__ unsigned hilbert3(unsigned x, unsigned y, unsigned z, int bits)
-{
-    if (bits == 0) return 0u;
-    for (unsigned q = 1u << (bits - 1); q > 1u; q >>= 1) {       // undo the excess rotations
-        const unsigned p = q - 1u;
-        if (x & q) x ^= p;
-        unsigned t = (x ^ y) & p;
-        if (y & q) x ^= p;
-        else { x ^= t; y ^= t; }
-        t = (x ^ z) & p;
-        if (z & q) x ^= p;
-        else { x ^= t; z ^= t; }
-    }
-    y ^= x;                                                       // Gray code
-    z ^= y;
-    unsigned t = 0u;
-    for (unsigned q = 1u << (bits - 1); q > 1u; q >>= 1)
-        if (z & q) t ^= q - 1u;
-    x ^= t; y ^= t; z ^= t;
-    unsigned h = 0u;
-    for (int b = bits - 1; b >= 0; --b) h = (h << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
-    return h;
-}
-
 __global__ void cluster_key_kernel(const BoxDev *boxes, const ClBox *cbox, const int *atom_box, const int4 *coords,
                                    int *key, int *rank, int *count, long long n)
 {

@@ -85,12 +85,10 @@ __global__ void cell_key_kernel(const BoxDev *boxes, const int *atom_box, const 
             const unsigned n = (unsigned)(b.gc_n > 0 ? b.gc_n : 1);
             k = b.gc0 + (int)((__umulhi(s.z, n) * n + __umulhi(s.y, n)) * n + __umulhi(s.x, n));
         } else if (type_major) {
-            // Monte Carlo partition: atom i of the box goes to CTA (i mod G) of its group;
-            // inside a CTA's share of a type, atoms are ordered by an 8^3 Morton cell.
-            const unsigned c8x = __umulhi(s.x, 8u), c8y = __umulhi(s.y, 8u), c8z = __umulhi(s.z, 8u);
-            const int code8 = (int)(spread5(c8x) | (spread5(c8y) << 1) | (spread5(c8z) << 2));
-            const int r = (int)((i - b.atom0) % b.n_cta);
-            k = b.mc_cell0 + ((int)s.w * b.n_cta + r) * kMcCells + code8;
+            // Monte Carlo partition: type by type, each along the Hilbert curve of its cells
+            const unsigned m = 1u << b.mc_bits;
+            k = b.mc_cell0 + ((int)s.w << (3 * b.mc_bits)) +
+                (int)hilbert3(__umulhi(s.x, m), __umulhi(s.y, m), __umulhi(s.z, m), b.mc_bits);
         } else {
             k = b.cell0 + (int)(spread5(cx) | (spread5(cy) << 1) | (spread5(cz) << 2));
         }
@@ -185,31 +183,21 @@ __global__ void scatter_index_kernel(const int *key, const int *rank, const int 
         sorted_index[offset[key[i]] + rank[i]] = (int)i;
 }
 
-// Makes the order deterministic: each cell's segment (a few atoms) is put in atom-index
-// order, then (optionally) the coordinates are gathered in that order and the inverse map
-// atom -> sorted position is written. Ranks from the counting pass depend on atomic timing;
-// the final order depends only on the coordinates.
-__global__ void cell_order_kernel(const int *count, const int *offset, int total_cells,
-                                  int *idx, const uint4 *scaled, const int4 *coords,
-                                  uint4 *s_scaled, int4 *s_coords, int *pos_of, int in_order)
+// Makes the order deterministic: each cell's segment is put in atom-index order (the ranks of the
+// counting pass depend on atomic timing), the coordinates are gathered in that order and the
+// inverse map atom -> sorted position is written, each optionally. One thread per atom counts the
+// atoms of its cell with a smaller index, which stays parallel for crowded cells.
+__global__ void cell_order_kernel(const int *key, const int *count, const int *offset, const int *idx, const uint4 *scaled,
+                                  const int4 *coords, int *out, uint4 *s_scaled, int4 *s_coords, int *pos_of, long long n)
 {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < total_cells; c += gridDim.x * blockDim.x) {
-        const int b = offset[c], n = in_order ? count[c] : 0;
-        for (int a = 1; a < n; ++a) {
-            const int v = idx[b + a];
-            int k = a - 1;
-            while (k >= 0 && idx[b + k] > v) {
-                idx[b + k + 1] = idx[b + k];
-                --k;
-            }
-            idx[b + k + 1] = v;
-        }
-        for (int a = 0, na = count[c]; a < na; ++a) {
-            const int i = idx[b + a];
-            if (s_scaled) s_scaled[b + a] = scaled[i];
-            if (s_coords) s_coords[b + a] = coords[i];
-            if (pos_of) pos_of[i] = b + a;
-        }
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
+        const int i = idx[p], c = key[i], b = offset[c], m = count[c];
+        int at = b;
+        for (int q = 0; q < m; ++q) at += idx[b + q] < i ? 1 : 0;
+        out[at] = i;
+        if (s_scaled) s_scaled[at] = scaled[i];
+        if (s_coords) s_coords[at] = coords[i];
+        if (pos_of) pos_of[i] = at;
     }
 }
 
@@ -265,15 +253,14 @@ int launch_spatial_sort(const BoxDev *boxes, const int *atom_box, const uint4 *s
     int rc = launch_scan(sc.count, total_cells, sc.offset, sc.block, stream);
     if (rc) return rc;
     if ((rc = launch_scatter(sc.key, sc.rank, sc.offset, sc.index, n, stream))) return rc;
-    const int cgrid = (total_cells + 255) / 256 < 4096 ? (total_cells + 255) / 256 : 4096;
     if (type_major == 2) {
         // the cell-list order only feeds integer counts: the order inside a cell does not
         // matter there and its cells are large, so the scatter's order is kept and the
         // coordinates are gathered by position, in parallel
         gather_sorted_kernel<<<grid, 256, 0, stream>>>(sc.index, scaled, coords, s_scaled, s_coords, n);
     } else {
-        cell_order_kernel<<<cgrid, 256, 0, stream>>>(sc.count, sc.offset, total_cells, sc.index, scaled,
-                                                     coords, s_scaled, s_coords, pos_of, 1);
+        cell_order_kernel<<<grid, 256, 0, stream>>>(sc.key, sc.count, sc.offset, sc.index, scaled, coords, sc.rank,
+                                                    s_scaled, s_coords, pos_of, n);
     }
     note_launch();
     e = cudaGetLastError();

@@ -10,12 +10,13 @@
 //     GPU instead of once per move in every CTA.
 //  2. mc_sweep_kernel, a cooperative persistent kernel: every box of the handle owns a
 //     contiguous group of CTAs; each CTA keeps a slice of its box's atoms (the partners)
-//     resident in shared memory for the whole sweep.
+//     resident in shared memory for the whole sweep: a contiguous run of every type's Hilbert
+//     order, so a compact region, in chunks of 32 slots with bounding boxes.
 //
 // Batching without changing the chain: moves are taken in batches of up to K
 // consecutive moves with distinct molecules (a batch ends before the first molecule that
-// repeats; K <= 64). Warp w computes the partial dU of moves w, w + 16, w + 32 and w + 48
-// against the slice as it stood at the start of the batch. One grid barrier per batch gathers the per-CTA partials; every
+// repeats; K <= 64). The CTA computes the partial dU of every move against its slice as it
+// stood at the start of the batch. One grid barrier per batch gathers the per-CTA partials; every
 // CTA sums them in the same fixed order and resolves the batch in order: move k's dU is
 // its batch-start value plus, for every earlier accepted move k' of the batch, the exact
 // change of the pair energies between the two moved molecules,
@@ -35,9 +36,9 @@ constexpr int kBatchMax = kMcBatchMax;         // moves per batch: warp w takes 
 constexpr int kPerWarp = kBatchMax / kMcWarps;  // moves per warp and batch
 constexpr int kMoveBlock = 128;                // move records staged in shared memory at once
 constexpr int kCorrItems = kMcCorrItems;       // >= 496 pairs x 8 atoms (coarse items at G = 1)
-constexpr int kStageChunk = kMcStageChunk;     // partners per staged chunk (slices in global memory)
-constexpr int kEscMax = 256;                   // escapee list capacity per CTA (at most)
-constexpr int kEscFlag = (int)0x80000000u;     // bit 31 of a slice entry's .w: escapee
+constexpr int kStage = kMcStageChunk;          // partners staged at once (slices in global memory)
+constexpr int kQueue = kBatchMax * kBatchMax / 2;   // near items of one round (in the corrections' buffer)
+constexpr int kEscMax = 256;                   // largest escapee_cap that epsr_mc_set_cells accepts
 static_assert(kMcCorrPerCta == kBatchMax * (kBatchMax - 1) / 2 && kMcSlotStride == kBatchMax + kMcCorrPerCta,
               "barrier slot layout");
 static_assert(kMcThreads == 8 * kBatchMax, "gather: 8 threads per move");
@@ -124,15 +125,17 @@ struct McShared {
     int natoms[kBatchMax];
     int a0[kBatchMax];
     int spos[kBatchMax][kMaxMolAtoms];   // type-major sorted position of each moved atom
-    int hw[kBatchMax];                   // half width of the near cube around old atom 0
-    // first three atoms of each move on the 2^32-periodic grid, new and old: [move][atom][axis]
-    unsigned scn[kBatchMax][3][3];
-    unsigned sco[kBatchMax][3][3];
+    float hw2[kBatchMax];                // square of the near radius around old atom 0 (grid units)
+    // per move and partner type: bit a of the low (high) byte set when moved atom a has a
+    // Lennard-Jones (near-only) row with the type
+    unsigned short rows[kBatchMax][kMaxTypes];
+    int n_near[kBatchMax];               // near chunks of each move
     // this CTA's partners: per type t, sorted positions [rs[t], rs[t] + rl[t]) held at
-    // slice slots [blk[t], blk[t + 1])
+    // slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
     int rs[kMaxTypes];
     int rl[kMaxTypes];
     int blk[kMaxTypes + 1];
+    int wd[kMaxTypes + 1];
     float thr[kBatchMax];
     double u_acc[kBatchMax];
     float part[kBatchMax];
@@ -143,9 +146,6 @@ struct McShared {
     float acc_du[kMoveBlock];                // rank 0: dU of each decided move if accepted, else 0
     float dU[kBatchMax];
     int abort_flag;
-    int cb[9];                               // cell boundaries ceil(j L / 8)
-    int n_esc, cells_on;
-    int esc[kEscMax];                        // escapee slots
     // leader-only running statistics
     long long st_att, st_acc, st_nonfinite;
     double st_sum;
@@ -211,67 +211,6 @@ __device__ __forceinline__ int floordiv32(int a, int b)   // b > 0
     return q;
 }
 
-// ---- near-partner cells -------------------------------------------------------------------------
-// A CTA's partners of each type are ordered by the cell of an 8^3 grid (cell k on an axis
-// holds ceil(k L / 8) <= x < ceil((k + 1) L / 8)) as the sweep starts, so the partners
-// inside a cube around a moved molecule lie in the slice ranges of the few cells the cube
-// meets. Atoms move during the sweep: a partner that leaves its home cell widened by
-// the cell margin is an escapee; it keeps its slot (flagged in bit 31 of .w) and joins a
-// per-CTA list that every cell query scans in full. Cell queries cover the cube widened by
-// the margin, so together with the escapees every partner inside the cube is found.
-
-struct CellIndex {
-    const unsigned *cst;         // [n_types][kMcCells + 1] first slot of each cell, relative to blk[t]
-    const int *cb;               // [9] cell boundaries ceil(j L / 8), cb[8] = L
-    const int *esc;              // escapee slots
-    int n_esc;
-    int margin;                  // drift (grid units) allowed before an atom becomes an escapee
-    bool on;                     // cell queries allowed (escapee list not overflowed)
-};
-
-__device__ __forceinline__ int cell_of(int x, const int *cb)   // x in [0, L)
-{
-    int k = 0;
-#pragma unroll
-    for (int j = 1; j < 8; ++j) k += x >= cb[j] ? 1 : 0;
-    return k;
-}
-
-// Cyclic run of cells [k0, k0 + n) (mod 8) meeting [c - w, c + w] on one axis.
-__device__ __forceinline__ void cell_run(int c, long long w, int L, const int *cb, int &k0, int &n)
-{
-    if (8 * (2 * w + 1) >= 7LL * L) { k0 = 0; n = 8; return; }
-    long long lo = c - w, hi = c + w;
-    if (lo < 0) lo += L;
-    if (hi >= L) hi -= L;
-    k0 = cell_of((int)lo, cb);
-    n = ((cell_of((int)hi, cb) - k0) & 7) + 1;
-}
-
-__device__ __forceinline__ unsigned spread3(unsigned v)   // bits 0..2 -> 0, 3, 6
-{
-    return (v & 1u) | ((v & 2u) << 2) | ((v & 4u) << 4);
-}
-
-__device__ __forceinline__ unsigned compact3(unsigned v)  // bits 0, 3, 6 -> 0..2
-{
-    return (v & 1u) | ((v >> 2) & 2u) | ((v >> 4) & 4u);
-}
-
-__device__ __forceinline__ unsigned cell_code(int cx, int cy, int cz)
-{
-    return spread3((unsigned)cx) | (spread3((unsigned)cy) << 1) | (spread3((unsigned)cz) << 2);
-}
-
-// Is grid point x (one axis) within `margin` of cell k's interval (cyclically)?
-__device__ __forceinline__ bool near_cell(int x, int k, const int *cb, int L, int margin)
-{
-    long long d = (long long)x - ((long long)cb[k] - margin);
-    if (d < 0) d += L;
-    if (d >= L) d -= L;
-    return d < (long long)(cb[k + 1] - cb[k]) + 2LL * margin;
-}
-
 // Out-of-line copy of pair_du for code that runs once per batch (keeps the kernel small).
 template <bool CUT>
 __device__ __noinline__ float pair_du_cold(Sep sn, Sep so, const PairRow &pr, const BoxDev &bx,
@@ -311,405 +250,80 @@ __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b)
     return d;
 }
 
-// Lennard-Jones change of two far partners (one f32x2 lane pair) from their packed separation
-// components against a moved atom's new (XN, YN, ZN) and old (XO, YO, ZO) position, in units whose
-// square S2 converts to A^2: the direct difference u(r') - u(r), and both squared distances of
-// each partner in those units.
-struct FarLJ {
-    float d0, d1, g2n0, g2n1, g2o0, g2o1;
+// Lennard-Jones change u(r') - u(r) of two far partners p and q (one f32x2 lane pair) on the
+// 2^32-periodic grid, against a moved atom's new and old position there: a 32-bit difference
+// wraps to the minimum image, so a separation component costs one subtraction and one
+// conversion, and the two partners share every FP32 instruction. Taken directly: its rounding
+// is a few ulp of |u|, which is small beyond the near radius.
+struct LjSource {
+    unsigned nx, ny, nz, ox, oy, oz;
+    float c12, nc6;
 };
-__device__ __forceinline__ FarLJ far_lj2_xyz(uint64_t XN, uint64_t YN, uint64_t ZN, uint64_t XO, uint64_t YO,
-                                            uint64_t ZO, uint64_t S2, uint64_t C12, uint64_t NC6)
+__device__ __forceinline__ uint64_t far_du2(uint4 p, uint4 q, const LjSource &s, uint64_t S2)
 {
-    const uint64_t G2N = f2_fma(XN, XN, f2_fma(YN, YN, f2_mul(ZN, ZN)));
-    const uint64_t G2O = f2_fma(XO, XO, f2_fma(YO, YO, f2_mul(ZO, ZO)));
-    FarLJ f;
-    f2_unpack(G2N, f.g2n0, f.g2n1);
-    f2_unpack(G2O, f.g2o0, f.g2o1);
+    const uint64_t XN = f2_pack((float)(int)(p.x - s.nx), (float)(int)(q.x - s.nx));
+    const uint64_t YN = f2_pack((float)(int)(p.y - s.ny), (float)(int)(q.y - s.ny));
+    const uint64_t ZN = f2_pack((float)(int)(p.z - s.nz), (float)(int)(q.z - s.nz));
+    const uint64_t XO = f2_pack((float)(int)(p.x - s.ox), (float)(int)(q.x - s.ox));
+    const uint64_t YO = f2_pack((float)(int)(p.y - s.oy), (float)(int)(q.y - s.oy));
+    const uint64_t ZO = f2_pack((float)(int)(p.z - s.oz), (float)(int)(q.z - s.oz));
     float r2n0, r2n1, r2o0, r2o1;
-    f2_unpack(f2_mul(G2N, S2), r2n0, r2n1);
-    f2_unpack(f2_mul(G2O, S2), r2o0, r2o1);
+    f2_unpack(f2_mul(f2_fma(XN, XN, f2_fma(YN, YN, f2_mul(ZN, ZN))), S2), r2n0, r2n1);
+    f2_unpack(f2_mul(f2_fma(XO, XO, f2_fma(YO, YO, f2_mul(ZO, ZO))), S2), r2o0, r2o1);
     const uint64_t AN = f2_pack(rsqrtf(r2n0), rsqrtf(r2n1)), AO = f2_pack(rsqrtf(r2o0), rsqrtf(r2o1));
     const uint64_t IN = f2_mul(AN, AN), IO = f2_mul(AO, AO);
     const uint64_t S6N = f2_mul(f2_mul(IN, IN), IN), S6O = f2_mul(f2_mul(IO, IO), IO);
-    const uint64_t D = f2_sub(f2_mul(f2_fma(C12, S6N, NC6), S6N), f2_mul(f2_fma(C12, S6O, NC6), S6O));
-    f2_unpack(D, f.d0, f.d1);
-    return f;
+    const uint64_t C12 = f2_pack(s.c12, s.c12), NC6 = f2_pack(s.nc6, s.nc6);
+    return f2_sub(f2_mul(f2_fma(C12, S6N, NC6), S6N), f2_mul(f2_fma(C12, S6O, NC6), S6O));
 }
 
-// The same for two partners p and q on the 2^32-periodic grid (signed 32-bit differences).
-__device__ __forceinline__ FarLJ far_lj2(uint4 p, uint4 q, unsigned nx, unsigned ny, unsigned nz, unsigned ox,
-                                        unsigned oy, unsigned oz, uint64_t S2, uint64_t C12, uint64_t NC6)
+// Lennard-Jones terms of one moved atom each of two moves (s0, s1) with the groups of 32 slots
+// g0 .. g0 + ng - 1 of a run of n slots (sx: their 2^32-periodic copy, from its slot 0), group
+// g taken by a move unless bit g of its mask (near: left to the items) is set. A lane takes two
+// partners per step and both moves share their loads: four independent packed chains.
+__device__ __forceinline__ void far_groups(float &acc0, float &acc1, const LjSource &s0, const LjSource &s1,
+                                           unsigned near0, unsigned near1, const uint4 *sx, int ng, int n, uint64_t S2,
+                                           int lane)
 {
-    return far_lj2_xyz(f2_pack((float)(int)(p.x - nx), (float)(int)(q.x - nx)),
-                       f2_pack((float)(int)(p.y - ny), (float)(int)(q.y - ny)),
-                       f2_pack((float)(int)(p.z - nz), (float)(int)(q.z - nz)),
-                       f2_pack((float)(int)(p.x - ox), (float)(int)(q.x - ox)),
-                       f2_pack((float)(int)(p.y - oy), (float)(int)(q.y - oy)),
-                       f2_pack((float)(int)(p.z - oz), (float)(int)(q.z - oz)), S2, C12, NC6);
+    const unsigned both = near0 & near1;
+    for (int g = 0; g < ng; g += 2) {
+        if (((both >> g) & 3u) == 3u) continue;
+        const int j0 = g * 32 + lane, j1 = j0 + 32;
+        const uint4 p = sx[j0], q = sx[g + 1 < ng ? j1 : j0];
+        float a0, a1, b0, b1;
+        f2_unpack(far_du2(p, q, s0, S2), a0, a1);
+        f2_unpack(far_du2(p, q, s1, S2), b0, b1);
+        const bool v0 = j0 < n, v1 = j1 < n;             // the second group past ng has v1 false or its bit set
+        if (v0 && !((near0 >> g) & 1u)) acc0 += a0;
+        if (v1 && !((near0 >> (g + 1)) & 1u)) acc0 += a1;
+        if (v0 && !((near1 >> g) & 1u)) acc1 += b0;
+        if (v1 && !((near1 >> (g + 1)) & 1u)) acc1 += b1;
+    }
 }
 
-// Lennard-Jones rows (bit a of lj: atom a of the move) against partners [j0, j1) of type t,
-// added to acc in the order of a lane-strided scan, on the grid coordinates (integer minimum
-// image). A lane takes two partners, j and j + 32, per step. A pair whose squared distances both
-// exceed far2 has no Coulomb and no EP term, so its dU is the Lennard-Jones change alone, the
-// direct difference computed for both partners at once in packed f32x2 arithmetic; a pair that
-// is not that far takes the full pair_du (the cancellation-free form).
+// Near item: the change of one move's energy with one partner of every lane (grid point pj, of a
+// type t; valid: a partner, not an atom of the move), over the moved atoms in `todo`.
 template <int M, bool CUT>
-__device__ __forceinline__ float lj_rows(float acc, const int4 (&pn)[M], const int4 (&po)[M], unsigned lj, int a0,
-                                         int m, const int4 *part, int j0, int j1, int t, const BoxDev &bx,
-                                         const long long *T, const float *ep, int lane)
+__device__ __forceinline__ float near_du(const int4 *np, const int4 *op, int m, unsigned todo, int4 pj, int t, bool valid,
+                                         const BoxDev &bx, const long long *T, const float *ep)
 {
-    const int L = bx.L;
-    const float far2 = fmaxf(bx.rc2_hi, bx.has_ep ? bx.tmax_hi : 0.f);
-    const uint64_t S2 = f2_pack(bx.inv_s2, bx.inv_s2);
-    for (int j = j0 + lane; j < j1; j += 64) {
-        const bool in1 = j + 32 < j1;
-        const int4 p0 = part[j];
-        const int4 p1 = part[in1 ? j + 32 : j];
-        const int i0 = (p0.w & 0x7fffffff) >> 3, i1 = (p1.w & 0x7fffffff) >> 3;
-        const bool v0 = !(i0 >= a0 && i0 < a0 + m);
-        const bool v1 = in1 && !(i1 >= a0 && i1 < a0 + m);
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            if (a >= m || !((lj >> a) & 1u)) continue;
-            const PairRow &r = bx.row[pn[a].w * kMaxTypes + t];
-            const Sep n0 = sep(pn[a], p0, L), o0 = sep(po[a], p0, L);
-            const Sep n1 = sep(pn[a], p1, L), o1 = sep(po[a], p1, L);
-            const FarLJ f = far_lj2_xyz(f2_pack((float)n0.x, (float)n1.x), f2_pack((float)n0.y, (float)n1.y),
-                                        f2_pack((float)n0.z, (float)n1.z), f2_pack((float)o0.x, (float)o1.x),
-                                        f2_pack((float)o0.y, (float)o1.y), f2_pack((float)o0.z, (float)o1.z), S2,
-                                        f2_pack(r.c12, r.c12), f2_pack(-r.c6, -r.c6));
-            float d0 = f.d0, d1 = f.d1;
-            const bool s0 = v0 && !(f.g2n0 > far2 && f.g2o0 > far2);
-            const bool s1 = v1 && !(f.g2n1 > far2 && f.g2o1 > far2);
-            if (s0 || s1) {
-                if (s0) d0 = pair_du<CUT>(n0, o0, r, bx, T, ep);
-                if (s1) d1 = pair_du<CUT>(n1, o1, r, bx, T, ep);
-            }
-            if (v0) acc += d0;
-            if (v1) acc += d1;
-        }
-    }
-    return acc;
-}
-
-// The Lennard-Jones rows of lj_rows on the 2^32-periodic copy of the slice (sx: {X, Y, Z,
-// atom}, the moved atoms at qn/qo, [atom][axis]): a 32-bit difference wraps to the minimum
-// image, so a separation component costs one subtraction and one conversion, and two
-// partners share every FP32 instruction (f32x2). For single-atom moves a lane takes four
-// partners per step (two independent packed pairs: the scan is latency-bound at 16 warps per
-// SM), then two in the tail; for molecules (whose larger partner_sum the four-partner body
-// slowed) two per step throughout. A far pair (both squared distances beyond the Coulomb
-// cutoff and the EP table) has only the Lennard-Jones term, taken as the direct difference
-// u(r') - u(r): its rounding is a few ulp of |u| there, where |u| is small. A pair that is not
-// far takes pair_du on the exact grid slots (the cancellation-free form), one such partner of
-// the lane after the other. The moved atoms with a Lennard-Jones row take the slice one after
-// the other (water and single atoms have one such atom).
-template <int M, bool CUT>
-__device__ __forceinline__ float lj_rows_sc(float acc, const int4 *np, const int4 *op, const unsigned *qnp,
-                                            const unsigned *qop, unsigned lj, int a0, int m, const int4 *slice,
-                                            const uint4 *sx, int j0, int j1, int t, const BoxDev &bx,
-                                            const long long *T, const float *ep, int lane)
-{
-    const int L = bx.L;
-    const float far2 = fmaxf(bx.rc2_hi, bx.has_ep ? bx.tmax_hi : 0.f) * bx.sc_k2;
-    const uint64_t S2 = f2_pack(bx.sc_s2, bx.sc_s2);
-    for (int a = 0; a < m; ++a) {
-        if (!((lj >> a) & 1u)) continue;
-        const unsigned nx = qnp[3 * a], ny = qnp[3 * a + 1], nz = qnp[3 * a + 2];
-        const unsigned ox = qop[3 * a], oy = qop[3 * a + 1], oz = qop[3 * a + 2];
-        const PairRow &r = bx.row[np[a].w * kMaxTypes + t];
-        const uint64_t C12 = f2_pack(r.c12, r.c12), NC6 = f2_pack(-r.c6, -r.c6);
-        int j = j0 + lane;
-        for (; M == 1 && j + 96 < j1; j += 128) {        // four partners: j, j + 32, j + 64, j + 96
-            const uint4 p0 = sx[j], p1 = sx[j + 32], p2 = sx[j + 64], p3 = sx[j + 96];
-            const FarLJ f = far_lj2(p0, p1, nx, ny, nz, ox, oy, oz, S2, C12, NC6);
-            const FarLJ g = far_lj2(p2, p3, nx, ny, nz, ox, oy, oz, S2, C12, NC6);
-            float d[4] = {f.d0, f.d1, g.d0, g.d1};
-            const bool v0 = (unsigned)((int)p0.w - a0) >= (unsigned)m, v1 = (unsigned)((int)p1.w - a0) >= (unsigned)m;
-            const bool v2 = (unsigned)((int)p2.w - a0) >= (unsigned)m, v3 = (unsigned)((int)p3.w - a0) >= (unsigned)m;
-            unsigned nm = (v0 && !(f.g2n0 > far2 && f.g2o0 > far2) ? 1u : 0u) |
-                          (v1 && !(f.g2n1 > far2 && f.g2o1 > far2) ? 2u : 0u) |
-                          (v2 && !(g.g2n0 > far2 && g.g2o0 > far2) ? 4u : 0u) |
-                          (v3 && !(g.g2n1 > far2 && g.g2o1 > far2) ? 8u : 0u);
-            if (nm) {                                    // per lane: the loop's trip count differs by lane
-                const int4 pn = np[a], po = op[a];
-                while (nm) {
-                    const int q = __ffs(nm) - 1;
-                    nm &= nm - 1u;
-                    const int4 pj = slice[j + 32 * q];
-                    const float v = pair_du<CUT>(sep(pn, pj, L), sep(po, pj, L), r, bx, T, ep);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (u == q) d[u] = v;
-                }
-            }
-            if (v0) acc += d[0];
-            if (v1) acc += d[1];
-            if (v2) acc += d[2];
-            if (v3) acc += d[3];
-        }
-        for (; j < j1; j += 64) {                        // tail: two partners, j and j + 32
-            const bool in1 = j + 32 < j1;
-            const int jb = in1 ? j + 32 : j;
-            const uint4 p0 = sx[j];
-            const uint4 p1 = sx[jb];
-            const bool v0 = (unsigned)((int)p0.w - a0) >= (unsigned)m;
-            const bool v1 = in1 && (unsigned)((int)p1.w - a0) >= (unsigned)m;
-            const FarLJ f = far_lj2(p0, p1, nx, ny, nz, ox, oy, oz, S2, C12, NC6);
-            float d0 = f.d0, d1 = f.d1;
-            const bool s0 = v0 && !(f.g2n0 > far2 && f.g2o0 > far2);
-            const bool s1 = v1 && !(f.g2n1 > far2 && f.g2o1 > far2);
-            if (s0 || s1) {
-                const int4 pn = np[a], po = op[a];
-                if (s0) {
-                    const int4 pj = slice[j];
-                    d0 = pair_du<CUT>(sep(pn, pj, L), sep(po, pj, L), r, bx, T, ep);
-                }
-                if (s1) {
-                    const int4 pj = slice[jb];
-                    d1 = pair_du<CUT>(sep(pn, pj, L), sep(po, pj, L), r, bx, T, ep);
-                }
-            }
-            if (v0) acc += d0;
-            if (v1) acc += d1;
-        }
-    }
-    return acc;
-}
-
-// Near rows of one move against the partners of types ta (rows nra) and tb (rows nrb; tb < 0:
-// none) found by a cell query: the ncell cells of the CTA's 8^3 grid that meet the cube around
-// old atom 0 are taken one per lane, their runs for both types prefix-summed together (two
-// independent shuffle chains), and the candidates of type ta, then of type tb, dealt out to the
-// lanes; each candidate inside the cube (half width hw) adds its pair changes to acc.
-template <int M, bool CUT>
-__device__ __forceinline__ float cell_pairs(float acc, const int4 (&pn)[M], const int4 (&po)[M], int m, int a0,
-                                            int hw, int4 o0, int ta, unsigned nra, int tb, unsigned nrb,
-                                            const int4 *slice, const int *blk, const CellIndex &ci, int k0x, int nx,
-                                            int k0y, int ny, int k0z, int ncell, const BoxDev &bx,
-                                            const long long *T, const float *ep, int lane)
-{
-    const int L = bx.L;
-    int fa = 0, na = 0, fb = 0, nb = 0;
-    if (lane < ncell) {
-        const int ix = lane % nx, iy = (lane / nx) % ny, iz = lane / (nx * ny);
-        const unsigned code = cell_code((k0x + ix) & 7, (k0y + iy) & 7, (k0z + iz) & 7);
-        const unsigned *ca = ci.cst + ta * (kMcCells + 1);
-        fa = ca[code];
-        na = ca[code + 1] - fa;
-        if (tb >= 0) {
-            const unsigned *cb = ci.cst + tb * (kMcCells + 1);
-            fb = cb[code];
-            nb = cb[code + 1] - fb;
-        }
-    }
-    int ia = na, ib = nb;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int ya = __shfl_up_sync(0xffffffffu, ia, o);
-        const int yb = __shfl_up_sync(0xffffffffu, ib, o);
-        if (lane >= o) {
-            ia += ya;
-            ib += yb;
-        }
-    }
-    const int ea = ia - na, eb = ib - nb;
-    const int tota = __shfl_sync(0xffffffffu, ia, 31), totb = __shfl_sync(0xffffffffu, ib, 31);
-    const int total = tota + totb;
-    for (int q0 = 0; q0 < total; q0 += 32) {
-        const int q = q0 + lane;
-        const bool isb = q >= tota;
-        const int qq = isb ? q - tota : q;
-        int c = 0;                                       // last cell whose run starts at or before qq
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1) {
-            const int xa = __shfl_sync(0xffffffffu, ea, c + step);
-            const int xb = __shfl_sync(0xffffffffu, eb, c + step);
-            if (c + step < ncell && (isb ? xb : xa) <= qq) c += step;
-        }
-        const int cfa = __shfl_sync(0xffffffffu, fa, c), cea = __shfl_sync(0xffffffffu, ea, c);
-        const int cfb = __shfl_sync(0xffffffffu, fb, c), ceb = __shfl_sync(0xffffffffu, eb, c);
-        if (q < total) {
-            const int t = isb ? tb : ta;
-            const unsigned nr = isb ? nrb : nra;
-            const int4 pj = slice[blk[t] + (isb ? cfb + (qq - ceb) : cfa + (qq - cea))];
-            const int jatom = (pj.w & 0x7fffffff) >> 3;
-            const bool take = pj.w >= 0 && !(jatom >= a0 && jatom < a0 + m) && mi_abs(pj.x - o0.x, L) < hw &&
-                              mi_abs(pj.y - o0.y, L) < hw && mi_abs(pj.z - o0.z, L) < hw;
-            if (take) {
-#pragma unroll
-                for (int a = 0; a < M; ++a)
-                    if (a < m && ((nr >> a) & 1u))
-                        acc += pair_du<CUT>(sep(pn[a], pj, L), sep(po[a], pj, L), bx.row[pn[a].w * kMaxTypes + t], bx,
-                                            T, ep);
-            }
-        }
-    }
-    return acc;
-}
-
-// Partial dU of one move (atoms np/op, m <= M) against the partners of this CTA, lane-
-// strided. Per partner type the kind of each moved atom's pair row is uniform across the
-// warp: a Lennard-Jones row (LJ is not cut) is evaluated against every partner of the type;
-// a row without LJ has Coulomb or empirical-potential terms only inside the near cube
-// around old atom 0 (half width hw), so its partners come from a cell query when the cube
-// meets at most 32 cells, else from the full scan with the cube test. M is a compile-time
-// bound so the atom loop unrolls into independent dependency chains. SC: the slice has its
-// 2^32-periodic copy sx and the moved atoms theirs (qn, qo), used by the Lennard-Jones rows.
-template <int M, bool CELLS, bool CUT, bool SKIP_LJ = false, bool SC = false>
-__device__ __forceinline__ float partner_sum(const int4 *np, const int4 *op, int m, int a0, int hw,
-                                             const int4 *slice, const int *blk, const CellIndex &ci,
-                                             const BoxDev &bx, const long long *T, const float *ep,
-                                             int lane, const uint4 *sx = nullptr, const unsigned *qn = nullptr,
-                                             const unsigned *qo = nullptr)
-{
-    const int L = bx.L;
-    const int4 o0 = op[0];
-    int4 pn[M], po[M];
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-        pn[a] = a < m ? np[a] : make_int4(0, 0, 0, 0);
-        po[a] = a < m ? op[a] : make_int4(0, 0, 0, 0);
-    }
-    int k0x = 0, nx = 8, k0y = 0, ny = 8, k0z = 0, nz = 8;
-    if (CELLS && ci.on) {
-        const long long w = (long long)hw + ci.margin;
-        cell_run(o0.x, w, L, ci.cb, k0x, nx);
-        cell_run(o0.y, w, L, ci.cb, k0y, ny);
-        cell_run(o0.z, w, L, ci.cb, k0z, nz);
-    }
-    const int ncell = nx * ny * nz;
-    const bool use_cells = CELLS && ci.on && ncell <= 32;
-    unsigned cell_types = 0u;
-    int pend_t = -1;                                     // a type whose cell query waits for a second
-    unsigned pend_nr = 0u;
     float acc = 0.f;
-    for (int t = 0; t < bx.n_types; ++t) {
-        unsigned lj = 0u, nr = 0u;
-        const PairRow *pr[M];
-#pragma unroll
-        for (int a = 0; a < M; ++a) {
-            pr[a] = &bx.row[pn[a].w * kMaxTypes + t];
-            if (a >= m) continue;
-            if (lj_full_row<CUT>(*pr[a], bx)) lj |= 1u << a;
-            else if (near_row<CUT>(*pr[a], bx)) nr |= 1u << a;
-        }
-        if (SKIP_LJ) lj = 0u;                            // Lennard-Jones rows done by the caller
-        if (!(lj | nr)) continue;
-        const bool cells = nr && use_cells;
-        const unsigned scan_nr = cells ? 0u : nr;
-        if (lj && !scan_nr) {
-            if (SC)
-                acc = lj_rows_sc<M, CUT>(acc, np, op, qn, qo, lj, a0, m, slice, sx, blk[t], blk[t + 1], t, bx, T, ep,
-                                         lane);
-            else
-                acc = lj_rows<M, CUT>(acc, pn, po, lj, a0, m, slice, blk[t], blk[t + 1], t, bx, T, ep, lane);
-        } else if (lj | scan_nr) {
-            const int jb = blk[t + 1];
-#pragma unroll 2
-            for (int j = blk[t] + lane; j < jb; j += 32) {
-                int4 pj = slice[j];
-                const int jatom = (pj.w & 0x7fffffff) >> 3;
-                const bool self = jatom >= a0 && jatom < a0 + m;
-                const bool near = scan_nr && mi_abs(pj.x - o0.x, L) < hw &&
-                                  mi_abs(pj.y - o0.y, L) < hw && mi_abs(pj.z - o0.z, L) < hw;
-#pragma unroll
-                for (int a = 0; a < M; ++a) {
-                    if (a < m && !self && (((lj >> a) & 1u) || (((scan_nr >> a) & 1u) && near)))
-                        acc += pair_du<CUT>(sep(pn[a], pj, L), sep(po[a], pj, L), *pr[a], bx, T, ep);
-                }
-            }
-        }
-        if (CELLS && cells) {
-            // cell queries of two partner types share one enumeration of the cells
-            cell_types |= 1u << t;
-            if (pend_t < 0) {
-                pend_t = t;
-                pend_nr = nr;
-            } else {
-                acc = cell_pairs<M, CUT>(acc, pn, po, m, a0, hw, o0, pend_t, pend_nr, t, nr, slice, blk, ci, k0x, nx,
-                                         k0y, ny, k0z, ncell, bx, T, ep, lane);
-                pend_t = -1;
-            }
-        }
-    }
-    if (CELLS && pend_t >= 0)
-        acc = cell_pairs<M, CUT>(acc, pn, po, m, a0, hw, o0, pend_t, pend_nr, -1, 0u, slice, blk, ci, k0x, nx, k0y,
-                                 ny, k0z, ncell, bx, T, ep, lane);
-    // escapees of the types answered by cell queries (their LJ rows were in the full scans)
-    if (CELLS && cell_types)
-        for (int e = lane; e < ci.n_esc; e += 32) {
-            const int4 pj = slice[ci.esc[e]];
-            const int t = pj.w & 7;
-            const int jatom = (pj.w & 0x7fffffff) >> 3;
-            if (!((cell_types >> t) & 1u) || (jatom >= a0 && jatom < a0 + m)) continue;
-            if (!(mi_abs(pj.x - o0.x, L) < hw && mi_abs(pj.y - o0.y, L) < hw && mi_abs(pj.z - o0.z, L) < hw))
-                continue;
-            for (int a = 0; a < m; ++a) {
-                const PairRow &r = bx.row[np[a].w * kMaxTypes + t];
-                if (near_row<CUT>(r, bx))
-                    acc += pair_du_cold<CUT>(sep(np[a], pj, L), sep(op[a], pj, L), r, bx, T, ep);
-            }
-        }
-    return acc;
-}
-
-// Lennard-Jones rows of one move against a staged chunk of partners of type t (the chunk
-// is shared by all warps of the CTA; used when the slices live in global memory).
-template <int M, bool CUT>
-__device__ __forceinline__ float lj_chunk(const int4 *np, const int4 *op, int m, int a0, const int4 *stage,
-                                          int nc, int t, const BoxDev &bx, const long long *T, const float *ep,
-                                          int lane)
-{
-    unsigned lj = 0u;
-    int4 pn[M], po[M];
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-        pn[a] = a < m ? np[a] : make_int4(0, 0, 0, 0);
-        po[a] = a < m ? op[a] : make_int4(0, 0, 0, 0);
-        if (a < m) {
-            const PairRow &r = bx.row[pn[a].w * kMaxTypes + t];
-            if (lj_full_row<CUT>(r, bx)) lj |= 1u << a;
-        }
-    }
-    if (!lj) return 0.f;
-    return lj_rows<M, CUT>(0.f, pn, po, lj, a0, m, stage, 0, nc, t, bx, T, ep, lane);
-}
-
-// The same for any molecule size (atoms read from shared memory; out-of-line pair function).
-template <bool CUT>
-__device__ __noinline__ float partner_sum_any(const int4 *np, const int4 *op, int m, int a0, int hw,
-                                              const int4 *slice, const int *blk, const BoxDev &bx,
-                                              const long long *T, const float *ep, int lane)
-{
     const int L = bx.L;
-    const int4 o0 = op[0];
-    float acc = 0.f;
-    for (int t = 0; t < bx.n_types; ++t) {
-        unsigned lj = 0u, nr = 0u;
-        for (int a = 0; a < m; ++a) {
-            const PairRow &pr = bx.row[np[a].w * kMaxTypes + t];
-            if (lj_full_row<CUT>(pr, bx)) lj |= 1u << a;
-            else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
-        }
-        if (!(lj | nr)) continue;
-        for (int j = blk[t] + lane; j < blk[t + 1]; j += 32) {
-            int4 pj = slice[j];
-            const int jatom = (pj.w & 0x7fffffff) >> 3;
-            if (jatom >= a0 && jatom < a0 + m) continue;
-            pj.w = t;
-            const bool near = nr && mi_abs(pj.x - o0.x, L) < hw && mi_abs(pj.y - o0.y, L) < hw &&
-                              mi_abs(pj.z - o0.z, L) < hw;
-            const unsigned todo = lj | (near ? nr : 0u);
-            for (int a = 0; a < m; ++a) {
-                if ((todo >> a) & 1u) {
-                    const int4 pn = np[a], po = op[a];
-                    acc += pair_du_cold<CUT>(sep(pn, pj, L), sep(po, pj, L), bx.row[pn.w * kMaxTypes + t], bx, T, ep);
-                }
+    if (M > 0) {
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+            if ((todo >> a) & 1u) {
+                const int4 n = np[a], o = op[a];
+                const float v = pair_du<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, T, ep);
+                if (valid) acc += v;
             }
-        }
+    } else {
+        for (int a = 0; a < m; ++a)
+            if ((todo >> a) & 1u) {
+                const int4 n = np[a], o = op[a];
+                const float v = pair_du_cold<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, T, ep);
+                if (valid) acc += v;
+            }
     }
     return acc;
 }
@@ -741,29 +355,41 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     const int rank = cta - bx.cta0;
     const int L = bx.L;
     const int nt = bx.n_types;
-    // Partners of this CTA: the atoms i of the box with i mod G == rank (an even share of
-    // every region and type), grouped by type and ordered in space within each type.
+    // Partners of this CTA: of every type the run [n_t rank / G, n_t (rank + 1) / G) of its Hilbert
+    // order (an even share of every type, a compact region), each run on a chunk boundary.
+    const int cs = A.chunk_log;
     if (tid == 0) {
-        int b = 0;
+        int b = 0, w = 0;
         for (int t = 0; t < nt; ++t) {
-            const int key0 = bx.mc_cell0 + (t * G + rank) * kMcCells;
-            const int s0 = A.mc_offset[key0] - (int)bx.atom0;
-            const int s1 = A.mc_offset[key0 + kMcCells] - (int)bx.atom0;
-            sh.rs[t] = s0;
+            const int s0 = (int)(bx.count[t] * rank / G), s1 = (int)(bx.count[t] * (rank + 1) / G);
+            sh.rs[t] = bx.type_start[t] + s0;
             sh.rl[t] = s1 - s0;
             sh.blk[t] = b;
-            b += s1 - s0;
+            sh.wd[t] = w;
+            const int nc = (s1 - s0 + (1 << cs) - 1) >> cs;
+            b += nc << cs;
+            w += (nc + 31) >> 5;
         }
         sh.blk[nt] = b;
+        sh.wd[nt] = w;
     }
     __syncthreads();
 
-    // shared memory: partner slice {x, y, z, type | atom << 3}, thresholds, empirical potential
-    // (shared-memory slices: the slice, then its 2^32-periodic copy {X, Y, Z, atom})
+    // shared memory: partner slice {x, y, z, type | atom << 3} and its 2^32-periodic copy {X, Y, Z,
+    // atom} (or, with the slice in global memory, a staged part of the copy), thresholds, empirical
+    // potential, correction tables, chunk boxes (centre and half width per axis, one column per mask
+    // bit) and near masks
     int4 *slice = GSLICE ? A.slice_g + (size_t)cta * A.slice_cap : reinterpret_cast<int4 *>(dyn);
-    uint4 *sx = GSLICE ? nullptr : reinterpret_cast<uint4 *>(slice + A.slice_cap);
-    long long *T = GSLICE ? reinterpret_cast<long long *>(dyn) : reinterpret_cast<long long *>(sx + A.slice_cap);
+    uint4 *sx = GSLICE ? reinterpret_cast<uint4 *>(dyn) : reinterpret_cast<uint4 *>(slice + A.slice_cap);
+    long long *T = reinterpret_cast<long long *>(sx + (GSLICE ? kStage : A.slice_cap));
     float *ep = reinterpret_cast<float *>(T + A.tbl_cap);
+    float (*corr)[kBatchMax] = reinterpret_cast<float (*)[kBatchMax]>(ep + A.ep_cap);
+    float *corr_part = &corr[kBatchMax][0];                                              // [kCorrItems]
+    int *queue = reinterpret_cast<int *>(&corr[0][0]);                                  // [kQueue], during phase C
+    float *q_res = reinterpret_cast<float *>(queue + kQueue);                           // [kQueue]
+    const int cols = A.words_cap * 32;
+    int *cb = reinterpret_cast<int *>(corr_part + kCorrItems);                         // [6][cols]
+    unsigned *near = reinterpret_cast<unsigned *>(cb + 6 * cols);                      // [kBatchMax][words_cap]
     for (int t = 0; t < nt; ++t)
         for (int i = tid; i < sh.rl[t]; i += kMcThreads) {
             const int atom = A.sorted_index[bx.atom0 + sh.rs[t] + i] - (int)bx.atom0;
@@ -777,44 +403,28 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     for (int k = tid; k <= bx.n_bins; k += kMcThreads) T[k] = A.thresholds[bx.tbl_off + k];
     if (bx.has_ep)
         for (int k = tid; k < bx.n_pairs * bx.n_bins; k += kMcThreads) ep[k] = A.ep[bx.ep_off + k];
-    // cell index: first slot of each cell per type (relative to the type's block), the
-    // home cell of every slot, cell boundaries; cell queries only where some pair row has
-    // no Lennard-Jones term but a Coulomb or empirical-potential one
-    unsigned *cst = reinterpret_cast<unsigned *>(ep + A.ep_cap);
-    float (*corr)[kBatchMax] = reinterpret_cast<float (*)[kBatchMax]>(cst + A.types_cap * (kMcCells + 1));
-    float *corr_part = &corr[kBatchMax][0];                                              // [kCorrItems]
-    // GSLICE: staged chunk of partners [kStageChunk], on the next 16-byte boundary (the host
-    // sizes the dynamic shared memory as the 16-byte-rounded tables plus the chunk)
-    int4 *stage = reinterpret_cast<int4 *>((reinterpret_cast<uintptr_t>(corr_part + kCorrItems) + 15) &
-                                           ~static_cast<uintptr_t>(15));
-    unsigned short *home = GSLICE ? A.home_g + (size_t)cta * A.slice_cap
-                                  : reinterpret_cast<unsigned short *>(corr_part + kCorrItems);
-    for (int t = 0; t < nt; ++t) {
-        const int key0 = bx.mc_cell0 + (t * G + rank) * kMcCells;
-        for (int c = tid; c <= kMcCells; c += kMcThreads)
-            cst[t * (kMcCells + 1) + c] = (unsigned)(A.mc_offset[key0 + c] - A.mc_offset[key0]);
-    }
-    if (tid <= 8) sh.cb[tid] = (int)(((long long)tid * L + 7) / 8);
-    if (tid == 0) {
-        bool near_rows = false;
-        for (int a = 0; a < nt; ++a)
-            for (int b = 0; b < nt; ++b) {
-                const PairRow &r = bx.row[a * kMaxTypes + b];
-                near_rows |= near_row<CUT>(r, bx);
-            }
-        sh.n_esc = 0;
-        sh.cells_on = near_rows && A.esc_cap > 0 ? 1 : 0;
-    }
     __syncthreads();
-    for (int t = 0; t < nt; ++t) {
-        const unsigned *ct = cst + t * (kMcCells + 1);
-        for (int i = tid; i < sh.rl[t]; i += kMcThreads) {
-            int c = 0;                                   // last cell starting at or before i
-            for (int step = kMcCells / 2; step > 0; step >>= 1)
-                if (ct[c + step] <= (unsigned)i) c += step;
-            home[sh.blk[t] + i] = (unsigned short)c;
+    // boxes of the chunks (coordinates in [0, L); a chunk of Hilbert neighbours seldom meets the
+    // seam, and its box is then merely wide)
+    for (int t = 0; t < nt; ++t)
+        for (int c = warp; c < ((sh.rl[t] + (1 << cs) - 1) >> cs); c += kMcWarps) {
+            int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-1, -1, -1};
+            for (int i = (c << cs) + lane; i < min(sh.rl[t], (c + 1) << cs); i += 32) {
+                const int4 p = slice[sh.blk[t] + i];
+                lo[0] = min(lo[0], p.x); hi[0] = max(hi[0], p.x);
+                lo[1] = min(lo[1], p.y); hi[1] = max(hi[1], p.y);
+                lo[2] = min(lo[2], p.z); hi[2] = max(hi[2], p.z);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int l = __reduce_min_sync(0xffffffffu, lo[a]), u = __reduce_max_sync(0xffffffffu, hi[a]);
+                if (lane == 0) {
+                    const int col = sh.wd[t] * 32 + c, ce = l + ((u - l) >> 1);
+                    cb[a * cols + col] = ce;
+                    cb[(3 + a) * cols + col] = u - ce;
+                }
+            }
         }
-    }
     __syncthreads();
 
     // moves per batch: as set, else 64 for large CTA groups (the per-batch phases amortise
@@ -942,14 +552,6 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 }
                 np4 = make_int4(nx, ny, nz, op4.w);
                 sh.newp[par][k][kk] = np4;
-                if (!GSLICE && kk < 3) {
-                    sh.scn[k][kk][0] = scale32(nx, L, bx.sc_rcp);
-                    sh.scn[k][kk][1] = scale32(ny, L, bx.sc_rcp);
-                    sh.scn[k][kk][2] = scale32(nz, L, bx.sc_rcp);
-                    sh.sco[k][kk][0] = scale32(op4.x, L, bx.sc_rcp);
-                    sh.sco[k][kk][1] = scale32(op4.y, L, bx.sc_rcp);
-                    sh.sco[k][kk][2] = scale32(op4.z, L, bx.sc_rcp);
-                }
             }
             __syncwarp();
             if (act && kk == 0) {
@@ -976,16 +578,31 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 sh.thr[k] = mr.thr;
                 sh.u_acc[k] = mr.u_acc;
             }
-            // near cube: every old and new atom position lies within `reach` of old atom 0
-            int reach = 0;
+            // near sphere: every old and new atom position lies within `reach` of old atom 0 (a bound in
+            // FP32, rounded up by the margin), so a partner beyond near_fx + reach of it has no near term
+            float reach2 = 0.f;
             if (kk < m) {
                 const int4 o = sh.oldp[k][0];
-                reach = max(max(mi_abs(op4.x - o.x, L), max(mi_abs(op4.y - o.y, L), mi_abs(op4.z - o.z, L))),
-                            max(mi_abs(np4.x - o.x, L), max(mi_abs(np4.y - o.y, L), mi_abs(np4.z - o.z, L))));
+                reach2 = fmaxf(g2_of(sep(op4, o, L)), g2_of(sep(np4, o, L)));
             }
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) reach = max(reach, __shfl_xor_sync(0xffffffffu, reach, o));
-            if (act && kk == 0) sh.hw[k] = bx.near_fx + reach + 2;
+            for (int o = 4; o > 0; o >>= 1) reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
+            if (act && kk == 0) {
+                const float r = ((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f;
+                sh.hw2[k] = r * r;
+            }
+            // rows of the moved atoms with partner type kk (an atom that stays where it is has none)
+            if (act) {
+                unsigned lj = 0u, nr = 0u;
+                for (int a = 0; a < m && kk < nt; ++a) {
+                    const int4 n = sh.newp[par][k][a], o = sh.oldp[k][a];
+                    if (n.x == o.x && n.y == o.y && n.z == o.z) continue;
+                    const PairRow &pr = bx.row[n.w * kMaxTypes + kk];
+                    if (lj_full_row<CUT>(pr, bx)) lj |= 1u << a;
+                    else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
+                }
+                sh.rows[k][kk] = (unsigned short)(lj | (nr << 8));
+            }
         }
         __syncthreads();
         // ---- E. pair-energy corrections between the batch's moved molecules -----------------
@@ -1032,87 +649,191 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             }
         }
         const bool fine = n_items <= kCorrItems;
-        // ---- C. partial dU of move `warp` against this CTA's slice ---------------------------
-        if (GSLICE && sh.mm <= 3) {
-            // slices in global memory: the Lennard-Jones partners are staged chunk by chunk in
-            // shared memory and every warp scans each chunk for its moves, so a batch reads the
-            // slice once instead of once per move; then each move's near-only rows
-            float accL[kPerWarp];
+        // ---- C. partial dU of the batch's moves against this CTA's slice ---------------------
+        // Near chunks: those whose box meets the near sphere of the move. A (move, chunk) item
+        // takes all pairs of the moved atoms with the chunk's partners in the cancellation-free form,
+        // and the items of the CTA are spread over its warps: in a large box the few moves near this
+        // CTA's region would otherwise keep single warps busy. The other chunks have at most
+        // Lennard-Jones terms, scanned by the move's warp without any test per pair.
+        const int n_words = sh.wd[nt];
+        const unsigned ltm = (1u << lane) - 1u;
 #pragma unroll
-            for (int q = 0; q < kPerWarp; ++q) accL[q] = 0.f;
+        for (int q = 0; q < kPerWarp; ++q) {
+            const int k = warp + q * kMcWarps;
+            if (k >= nb) continue;
+            const int4 o0 = sh.oldp[k][0];
+            const float hw2 = sh.hw2[k];
+            int cnt = 0;
             for (int t = 0; t < nt; ++t) {
-                for (int c0 = sh.blk[t]; c0 < sh.blk[t + 1]; c0 += kStageChunk) {
-                    const int nc = min(kStageChunk, sh.blk[t + 1] - c0);
-                    __syncthreads();
-                    for (int i = tid; i < nc; i += kMcThreads) stage[i] = __ldcg(&slice[c0 + i]);
-                    __syncthreads();
+                const int nc = (sh.rl[t] + (1 << cs) - 1) >> cs;
+                const bool any = sh.rows[k][t] != 0;
+                for (int w = sh.wd[t]; w < sh.wd[t + 1]; ++w) {
+                    const int c = (w - sh.wd[t]) * 32 + lane, col = w * 32 + lane;
+                    bool hit = any && c < nc;
+                    if (hit && A.near_all == 0) {
+                        const float x = (float)max(0, mi_abs(o0.x - cb[col], L) - cb[3 * cols + col]);
+                        const float y = (float)max(0, mi_abs(o0.y - cb[cols + col], L) - cb[4 * cols + col]);
+                        const float z = (float)max(0, mi_abs(o0.z - cb[2 * cols + col], L) - cb[5 * cols + col]);
+                        hit = fmaf(x, x, fmaf(y, y, z * z)) < hw2;
+                    }
+                    const unsigned mk = __ballot_sync(0xffffffffu, hit);
+                    if (lane == 0) near[k * A.words_cap + w] = mk;
+                    cnt += __popc(mk);
+                }
+            }
+            if (lane == 0) sh.n_near[k] = cnt;
+        }
+        __syncthreads();
+        // first item of each move (lane l holds moves l and l + 32), and this warp's items of a round
+        int n_all;
+        int base[kPerWarp];
+        {
+            const int c0 = lane < nb ? sh.n_near[lane] : 0, c1 = lane + 32 < nb ? sh.n_near[lane + 32] : 0;
+            int x0 = c0, x1 = c1;
 #pragma unroll
-                    for (int q = 0; q < kPerWarp; ++q) {
-                        const int k = warp + q * kMcWarps;
-                        if (k >= nb) continue;
-                        const int m = sh.natoms[k];
-                        accL[q] += m == 1 ? lj_chunk<1, CUT>(sh.newp[par][k], sh.oldp[k], 1, sh.a0[k], stage, nc, t, bx, T, ep, lane)
-                                          : lj_chunk<3, CUT>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k], stage, nc, t, bx, T, ep, lane);
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
+                if (lane >= o) {
+                    x0 += y0;
+                    x1 += y1;
+                }
+            }
+            const int t0n = __shfl_sync(0xffffffffu, x0, 31);
+            n_all = t0n + __shfl_sync(0xffffffffu, x1, 31);
+#pragma unroll
+            for (int q = 0; q < kPerWarp; ++q) {
+                const int k = warp + q * kMcWarps;
+                const int b0 = __shfl_sync(0xffffffffu, x0 - c0, k & 31), b1 = __shfl_sync(0xffffffffu, x1 - c1, k & 31);
+                base[q] = k < 32 ? b0 : t0n + b1;
+            }
+        }
+        float acc[kPerWarp];
+#pragma unroll
+        for (int q = 0; q < kPerWarp; ++q) acc[q] = 0.f;
+        for (int r0 = 0; r0 == 0 || r0 < n_all; r0 += kQueue) {
+#pragma unroll
+            for (int q = 0; q < kPerWarp; ++q) {
+                const int k = warp + q * kMcWarps;
+                if (k >= nb || sh.n_near[k] == 0) continue;
+                int at = base[q] - r0;
+                for (int w = 0; w < n_words; ++w) {
+                    const unsigned mk = near[k * A.words_cap + w];
+                    const int i = at + __popc(mk & ltm);
+                    if (((mk >> lane) & 1u) && i >= 0 && i < kQueue) queue[i] = k | ((w * 32 + lane) << 8);
+                    at += __popc(mk);
+                }
+            }
+            if (r0 == 0 && !(CUT && bx.lj_cut)) {
+                // Lennard-Jones terms with the far chunks, atom by atom for two moves at a time
+                const uint64_t S2 = f2_pack(bx.sc_s2, bx.sc_s2);
+                for (int t = 0; t < nt; ++t) {
+                    const int rl = sh.rl[t];
+                    for (int c0 = 0; c0 < rl; c0 += GSLICE ? kStage : rl) {
+                        const int nst = GSLICE ? min(kStage, rl - c0) : rl;
+                        if (GSLICE) {
+                            // stage the copy of the next partners, read once for the whole batch
+                            __syncthreads();
+                            for (int i = tid; i < nst; i += kMcThreads) {
+                                const int4 p = __ldcg(&slice[sh.blk[t] + c0 + i]);
+                                sx[i] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
+                                                   scale32(p.z, L, bx.sc_rcp), 0u);
+                            }
+                            __syncthreads();
+                        }
+                        const uint4 *src = GSLICE ? sx : sx + sh.blk[t];
+#pragma unroll
+                        for (int h = 0; h < kPerWarp; h += 2) {
+                            const int k0 = warp + h * kMcWarps, k1 = k0 + kMcWarps;
+                            if (k0 >= nb) continue;
+                            const bool two = k1 < nb;
+                            const unsigned l0 = sh.rows[k0][t] & 0xFFu, l1 = two ? sh.rows[k1][t] & 0xFFu : 0u;
+                            for (unsigned todo = l0 | l1; todo; todo &= todo - 1u) {
+                                const int a = __ffs(todo) - 1;
+                                const bool on0 = (l0 >> a) & 1u, on1 = (l1 >> a) & 1u;
+                                LjSource s0, s1;
+                                {
+                                    const int kx = on0 ? k0 : k1, ky = on1 ? k1 : k0;
+                                    // lanes 0..5 convert the coordinates of one move, 8..13 of the other
+                                    const int4 *pp = (lane & 7) < 3 ? sh.newp[par][lane & 8 ? ky : kx] : sh.oldp[lane & 8 ? ky : kx];
+                                    const int ax = (lane & 7) % 3;
+                                    const int xc = ax == 0 ? pp[a].x : ax == 1 ? pp[a].y : pp[a].z;
+                                    const unsigned sc = scale32(xc, L, bx.sc_rcp);
+                                    s0.nx = __shfl_sync(0xffffffffu, sc, 0); s0.ny = __shfl_sync(0xffffffffu, sc, 1);
+                                    s0.nz = __shfl_sync(0xffffffffu, sc, 2); s0.ox = __shfl_sync(0xffffffffu, sc, 3);
+                                    s0.oy = __shfl_sync(0xffffffffu, sc, 4); s0.oz = __shfl_sync(0xffffffffu, sc, 5);
+                                    s1.nx = __shfl_sync(0xffffffffu, sc, 8); s1.ny = __shfl_sync(0xffffffffu, sc, 9);
+                                    s1.nz = __shfl_sync(0xffffffffu, sc, 10); s1.ox = __shfl_sync(0xffffffffu, sc, 11);
+                                    s1.oy = __shfl_sync(0xffffffffu, sc, 12); s1.oz = __shfl_sync(0xffffffffu, sc, 13);
+                                    const PairRow &ra = bx.row[sh.oldp[kx][a].w * kMaxTypes + t];
+                                    const PairRow &rb = bx.row[sh.oldp[ky][a].w * kMaxTypes + t];
+                                    s0.c12 = ra.c12; s0.nc6 = -ra.c6;
+                                    s1.c12 = rb.c12; s1.nc6 = -rb.c6;
+                                }
+                                for (int g0 = 0; g0 < nst; g0 += 32 * 32) {
+                                    unsigned n0, n1;
+                                    if (!GSLICE) {
+                                        n0 = near[k0 * A.words_cap + sh.wd[t] + (g0 >> 10)];
+                                        n1 = two ? near[k1 * A.words_cap + sh.wd[t] + (g0 >> 10)] : 0u;
+                                    } else {
+                                        // group g of the stage lies in chunk (c0 + g0) / 32 + g, cs - 5 bits coarser
+                                        const int c = (c0 + g0 + 32 * lane) >> cs;
+                                        const int w = min(sh.wd[t] + (c >> 5), n_words - 1);
+                                        n0 = __ballot_sync(0xffffffffu, (near[k0 * A.words_cap + w] >> (c & 31)) & 1u);
+                                        n1 = __ballot_sync(0xffffffffu, two && ((near[k1 * A.words_cap + w] >> (c & 31)) & 1u));
+                                    }
+                                    if (!on0) n0 = 0xFFFFFFFFu;
+                                    if (!on1) n1 = 0xFFFFFFFFu;
+                                    const int left = nst - g0;
+                                    far_groups(acc[h], acc[h + 1], s0, s1, n0, n1, src + g0, min(32, (left + 31) >> 5), left, S2,
+                                               lane);
+                                }
+                            }
+                        }
                     }
                 }
             }
-            CellIndex ci;
-            ci.cst = cst;
-            ci.cb = sh.cb;
-            ci.esc = sh.esc;
-            ci.n_esc = min(sh.n_esc, A.esc_cap);
-            ci.margin = A.cell_margin;
-            ci.on = sh.cells_on != 0;
+            __syncthreads();
+            // near items, one per warp at a time
+            for (int i = warp; i < min(kQueue, n_all - r0); i += kMcWarps) {
+                const int e = queue[i], k = e & 0xFF, col = e >> 8;
+                int t = 0;
+                while (sh.wd[t + 1] * 32 <= col) ++t;
+                const int c = col - sh.wd[t] * 32, m = sh.natoms[k], a0 = sh.a0[k];
+                const unsigned rw = sh.rows[k][t], todo = (rw | (rw >> 8)) & 0xFFu;
+                const int4 *np = sh.newp[par][k], *op = sh.oldp[k];
+                float v = 0.f;
+                for (int o = c << cs; o < ((c + 1) << cs); o += 32) {
+                    const int s_ = o + lane;
+                    bool valid = s_ < sh.rl[t];
+                    if (!__any_sync(0xffffffffu, valid)) break;
+                    const int4 pj = slice[sh.blk[t] + (valid ? s_ : 0)];
+                    const int ja = pj.w >> 3;
+                    valid = valid && !(ja >= a0 && ja < a0 + m);
+                    v += m == 1 ? near_du<1, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep)
+                         : m <= 3 ? near_du<3, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep)
+                                  : near_du<0, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep);
+                }
+                v = warp_sum(v);
+                if (lane == 0) q_res[i] = v;
+            }
+            __syncthreads();
+            // each move's items of the round, in order (lane-strided, then the warp's sum below)
 #pragma unroll
             for (int q = 0; q < kPerWarp; ++q) {
                 const int k = warp + q * kMcWarps;
                 if (k >= nb) continue;
-                const int m = sh.natoms[k];
-                float acc = accL[q];
-                if (m == 1)
-                    acc += ci.on ? partner_sum<1, true, CUT, true>(sh.newp[par][k], sh.oldp[k], 1, sh.a0[k], sh.hw[k],
-                                                              slice, sh.blk, ci, bx, T, ep, lane)
-                                 : partner_sum<1, false, CUT, true>(sh.newp[par][k], sh.oldp[k], 1, sh.a0[k], sh.hw[k],
-                                                               slice, sh.blk, ci, bx, T, ep, lane);
-                else
-                    acc += ci.on ? partner_sum<3, true, CUT, true>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k], sh.hw[k],
-                                                              slice, sh.blk, ci, bx, T, ep, lane)
-                                 : partner_sum<3, false, CUT, true>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k], sh.hw[k],
-                                                               slice, sh.blk, ci, bx, T, ep, lane);
-                acc = warp_sum(acc);
-                if (lane == 0) sh.part[k] = acc;
+                for (int i = lane; i < sh.n_near[k]; i += 32) {
+                    const int at = base[q] + i - r0;
+                    if (at >= 0 && at < kQueue) acc[q] += q_res[at];
+                }
             }
-        } else
-        for (int k = warp; k < nb; k += kMcWarps) {
-            const int m = sh.natoms[k];
-            float acc;
-            CellIndex ci;
-            ci.cst = cst;
-            ci.cb = sh.cb;
-            ci.esc = sh.esc;
-            ci.n_esc = min(sh.n_esc, A.esc_cap);
-            ci.margin = A.cell_margin;
-            ci.on = sh.cells_on != 0;
-            const unsigned *qn = &sh.scn[k][0][0], *qo = &sh.sco[k][0][0];
-            if (m == 1)
-                acc = ci.on ? partner_sum<1, true, CUT, false, !GSLICE>(sh.newp[par][k], sh.oldp[k], 1, sh.a0[k],
-                                                                      sh.hw[k], slice, sh.blk, ci, bx, T, ep, lane,
-                                                                      sx, qn, qo)
-                            : partner_sum<1, false, CUT, false, !GSLICE>(sh.newp[par][k], sh.oldp[k], 1, sh.a0[k],
-                                                                       sh.hw[k], slice, sh.blk, ci, bx, T, ep, lane,
-                                                                       sx, qn, qo);
-            else if (m <= 3)
-                acc = ci.on ? partner_sum<3, true, CUT, false, !GSLICE>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k],
-                                                                      sh.hw[k], slice, sh.blk, ci, bx, T, ep, lane,
-                                                                      sx, qn, qo)
-                            : partner_sum<3, false, CUT, false, !GSLICE>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k],
-                                                                       sh.hw[k], slice, sh.blk, ci, bx, T, ep, lane,
-                                                                       sx, qn, qo);
-            else
-                acc = partner_sum_any<CUT>(sh.newp[par][k], sh.oldp[k], m, sh.a0[k], sh.hw[k],
-                                      slice, sh.blk, bx, T, ep, lane);
-            acc = warp_sum(acc);
-            if (lane == 0) sh.part[k] = acc;
+        }
+#pragma unroll
+        for (int q = 0; q < kPerWarp; ++q) {
+            const int k = warp + q * kMcWarps;
+            if (k >= nb) continue;
+            const float v = warp_sum(acc[q]);
+            if (lane == 0) sh.part[k] = v;
         }
         __syncthreads();
         // ---- D. gather the partials of the box's CTA group (one bounded grid barrier) -------
@@ -1290,24 +1011,12 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             const int4 p = sh.newp[par][k][a];
             const int t = p.w, sp = sh.spos[k][a] - sh.rs[t];
             if (sp >= 0 && sp < sh.rl[t]) {
-                const int slot = sh.blk[t] + sp;
-                int w = t | (ja << 3);
-                if (sh.cells_on) {
-                    bool esc = slice[slot].w < 0;
-                    if (!esc) {
-                        const unsigned h = home[slot];
-                        esc = !(near_cell(p.x, (int)compact3(h), sh.cb, L, A.cell_margin) &&
-                                near_cell(p.y, (int)compact3(h >> 1), sh.cb, L, A.cell_margin) &&
-                                near_cell(p.z, (int)compact3(h >> 2), sh.cb, L, A.cell_margin));
-                        if (esc) {
-                            const int e = atomicAdd(&sh.n_esc, 1);
-                            if (e < A.esc_cap) sh.esc[e] = slot;
-                            else sh.cells_on = 0;            // too many: full scans from now on
-                        }
-                    }
-                    if (esc) w |= kEscFlag;
-                }
-                slice[slot] = make_int4(p.x, p.y, p.z, w);
+                const int slot = sh.blk[t] + sp, col = sh.wd[t] * 32 + (sp >> cs);
+                slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
+                // the chunk's box grows to hold the new position
+                atomicMax(&cb[3 * cols + col], mi_abs(p.x - cb[col], L));
+                atomicMax(&cb[4 * cols + col], mi_abs(p.y - cb[cols + col], L));
+                atomicMax(&cb[5 * cols + col], mi_abs(p.z - cb[2 * cols + col], L));
                 if (!GSLICE)
                     sx[slot] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
                                           scale32(p.z, L, bx.sc_rcp), (unsigned)ja);
