@@ -369,7 +369,7 @@ static int mc_layout(const epsr_box *h, McLayout *L)
         for (auto &b : h->hb) {
             int slots = 0, words = 0;
             for (int t = 0; t < b.n_types; ++t) {
-                const int n = (int)((b.count[t] + b.n_cta - 1) / b.n_cta), nc = (n + (1 << cs) - 1) >> cs;
+                const int nch = (int)((b.count[t] + (1 << cs) - 1) >> cs), nc = (nch + b.n_cta - 1) / b.n_cta;
                 slots += nc << cs;
                 words += (nc + 31) / 32;
             }

@@ -130,9 +130,9 @@ struct McShared {
     // Lennard-Jones (near-only) row with the type
     unsigned short rows[kBatchMax][kMaxTypes];
     int n_near[kBatchMax];               // near chunks of each move
-    // this CTA's partners: per type t, sorted positions [rs[t], rs[t] + rl[t]) held at
-    // slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
-    int rs[kMaxTypes];
+    // this CTA's partners: per type t, the chunks first[t], first[t] + G, .. of its sorted order, rl[t]
+    // atoms in slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
+    int first[kMaxTypes];
     int rl[kMaxTypes];
     int blk[kMaxTypes + 1];
     int wd[kMaxTypes + 1];
@@ -301,6 +301,55 @@ __device__ __forceinline__ void far_groups(float &acc0, float &acc1, const LjSou
     }
 }
 
+// u(r') - u(r) for one partner as pair_du takes it, without branches, so that the atoms of a
+// molecule run side by side: every term is formed and selected. Sets `rare` where a squared
+// distance lies within its FP32 error of a cutoff, of the table's end or of a bin edge, or the new
+// distance is zero; the caller then takes pair_du.
+template <bool CUT>
+__device__ __forceinline__ float near_pair(Sep sn, Sep so, const PairRow &pr, const BoxDev &bx, const float *ep, bool &rare)
+{
+    const DuCore c = du_core(sn, so, bx.inv_s2);
+    float du = 0.f;
+    rare |= c.g2n == 0.f;
+    if (pr.c12 != 0.f || pr.c6 != 0.f) {                         // one row for the whole warp
+        const float lj = lj_du(c, pr.c12, pr.c6);
+        if (!CUT || !bx.lj_cut) {
+            du = lj;
+        } else {
+            const bool ln = c.g2n < bx.lj2_lo, lo = c.g2o < bx.lj2_lo;
+            rare |= (!ln && c.g2n <= bx.lj2_hi) || (!lo && c.g2o <= bx.lj2_hi);
+            const float a2 = ln ? c.an * c.an : c.ao * c.ao;
+            const float s6 = a2 * a2 * a2;
+            const float u = fmaf(pr.c12, s6, -pr.c6) * s6;
+            du = ln && lo ? lj : ln ? u : lo ? -u : 0.f;
+        }
+    }
+    if (pr.kqq != 0.f) {
+        const bool cn = c.g2n < bx.rc2_lo, co = c.g2o < bx.rc2_lo;
+        rare |= (!cn && c.g2n <= bx.rc2_hi) || (!co && c.g2o <= bx.rc2_hi);
+        const float p = c.an * c.ao;
+        const float both = c.dr2 * __fdividef(p * p, c.an + c.ao);       // 2 ulp; an + ao ~ 0.1..10
+        du = fmaf(pr.kqq, cn && co ? both : cn ? c.an : co ? -c.ao : 0.f, du);
+    }
+    if (bx.has_ep) {
+        const float *row = ep + pr.pair * bx.n_bins;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float g2 = h ? c.g2o : c.g2n;
+            float r;
+            asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g2));
+            const float u = fmaf(r, bx.inv_dr_fx, -0.5f);
+            const float t = u + 12582912.f;                      // u rounded to an integer in the low bits
+            const float d = u - (t - 12582912.f);
+            const bool in = g2 < bx.tmax_lo;
+            rare |= (!in && g2 <= bx.tmax_hi) || (in && !(fabsf(d) < fmaf(u, -0x1p-20f, 0.5f - 0x1p-20f)));
+            const float e = row[in ? min(max(__float_as_int(t) - 0x4B400000, 0), bx.n_bins - 1) : 0];
+            du += in ? (h ? -e : e) : 0.f;
+        }
+    }
+    return du;
+}
+
 // Near item: the change of one move's energy with one partner of every lane (grid point pj, of a
 // type t; valid: a partner, not an atom of the move), over the moved atoms in `todo`.
 template <int M, bool CUT>
@@ -309,23 +358,24 @@ __device__ __forceinline__ float near_du(const int4 *np, const int4 *op, int m, 
 {
     float acc = 0.f;
     const int L = bx.L;
+    bool rare = M == 0;
     if (M > 0) {
 #pragma unroll
-        for (int a = 0; a < M; ++a)
-            if ((todo >> a) & 1u) {
-                const int4 n = np[a], o = op[a];
-                const float v = pair_du<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, T, ep);
-                if (valid) acc += v;
-            }
-    } else {
+        for (int a = 0; a < M; ++a) {
+            if (!((todo >> a) & 1u)) continue;
+            const int4 n = np[a], o = op[a];
+            acc += near_pair<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, ep, rare);
+        }
+    }
+    if (rare && valid) {
+        acc = 0.f;
         for (int a = 0; a < m; ++a)
             if ((todo >> a) & 1u) {
                 const int4 n = np[a], o = op[a];
-                const float v = pair_du_cold<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, T, ep);
-                if (valid) acc += v;
+                acc += pair_du_cold<CUT>(sep(n, pj, L), sep(o, pj, L), bx.row[n.w * kMaxTypes + t], bx, T, ep);
             }
     }
-    return acc;
+    return valid ? acc : 0.f;
 }
 
 // GSLICE: the partner slices live in global memory ([grid][slice_cap], read through L1/L2)
@@ -355,20 +405,25 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     const int rank = cta - bx.cta0;
     const int L = bx.L;
     const int nt = bx.n_types;
-    // Partners of this CTA: of every type the run [n_t rank / G, n_t (rank + 1) / G) of its Hilbert
-    // order (an even share of every type, a compact region), each run on a chunk boundary.
+    // Partners of this CTA: every type's Hilbert order is cut into chunks of 2^cs atoms (compact
+    // regions), dealt out in turn: chunk c of a type that follows f chunks of earlier types goes to
+    // CTA (f + c) mod G of the group. A move's near chunks so fall on as many CTAs as there are
+    // chunks, instead of all on the one that owns the region (the barrier waits for the busiest).
     const int cs = A.chunk_log;
     if (tid == 0) {
         int b = 0, w = 0;
+        long long f = 0;
         for (int t = 0; t < nt; ++t) {
-            const int s0 = (int)(bx.count[t] * rank / G), s1 = (int)(bx.count[t] * (rank + 1) / G);
-            sh.rs[t] = bx.type_start[t] + s0;
-            sh.rl[t] = s1 - s0;
+            const int n = (int)bx.count[t], nch = (n + (1 << cs) - 1) >> cs;      // chunks of the type
+            const int first = (int)(((long long)rank - f % G + G) % G);           // this CTA's first chunk
+            const int nc = first < nch ? (nch - first + G - 1) / G : 0;
+            sh.first[t] = first;
+            sh.rl[t] = nc == 0 ? 0 : first + (nc - 1) * G == nch - 1 ? ((nc - 1) << cs) + n - ((nch - 1) << cs) : nc << cs;
             sh.blk[t] = b;
             sh.wd[t] = w;
-            const int nc = (s1 - s0 + (1 << cs) - 1) >> cs;
             b += nc << cs;
             w += (nc + 31) >> 5;
+            f += nch;
         }
         sh.blk[nt] = b;
         sh.wd[nt] = w;
@@ -392,7 +447,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     unsigned *near = reinterpret_cast<unsigned *>(cb + 6 * cols);                      // [kBatchMax][words_cap]
     for (int t = 0; t < nt; ++t)
         for (int i = tid; i < sh.rl[t]; i += kMcThreads) {
-            const int atom = A.sorted_index[bx.atom0 + sh.rs[t] + i] - (int)bx.atom0;
+            const int pos = bx.type_start[t] + ((sh.first[t] + (i >> cs) * G) << cs) + (i & ((1 << cs) - 1));
+            const int atom = A.sorted_index[bx.atom0 + pos] - (int)bx.atom0;
             int4 c = A.coords[bx.atom0 + atom];
             c.w = c.w | (atom << 3);
             slice[sh.blk[t] + i] = c;
@@ -657,31 +713,39 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // Lennard-Jones terms, scanned by the move's warp without any test per pair.
         const int n_words = sh.wd[nt];
         const unsigned ltm = (1u << lane) - 1u;
+        {
+            int4 o0[kPerWarp];
+            float hw2[kPerWarp];
+            int cnt[kPerWarp];
 #pragma unroll
-        for (int q = 0; q < kPerWarp; ++q) {
-            const int k = warp + q * kMcWarps;
-            if (k >= nb) continue;
-            const int4 o0 = sh.oldp[k][0];
-            const float hw2 = sh.hw2[k];
-            int cnt = 0;
+            for (int q = 0; q < kPerWarp; ++q) {
+                const int k = min(warp + q * kMcWarps, nb - 1);
+                o0[q] = sh.oldp[k][0];
+                hw2[q] = A.near_all ? 3e38f : sh.hw2[k];
+                cnt[q] = 0;
+            }
             for (int t = 0; t < nt; ++t) {
                 const int nc = (sh.rl[t] + (1 << cs) - 1) >> cs;
-                const bool any = sh.rows[k][t] != 0;
                 for (int w = sh.wd[t]; w < sh.wd[t + 1]; ++w) {
-                    const int c = (w - sh.wd[t]) * 32 + lane, col = w * 32 + lane;
-                    bool hit = any && c < nc;
-                    if (hit && A.near_all == 0) {
-                        const float x = (float)max(0, mi_abs(o0.x - cb[col], L) - cb[3 * cols + col]);
-                        const float y = (float)max(0, mi_abs(o0.y - cb[cols + col], L) - cb[4 * cols + col]);
-                        const float z = (float)max(0, mi_abs(o0.z - cb[2 * cols + col], L) - cb[5 * cols + col]);
-                        hit = fmaf(x, x, fmaf(y, y, z * z)) < hw2;
+                    const int c = (w - sh.wd[t]) * 32 + lane, col = w * 32 + min(lane, nc - 1 - (w - sh.wd[t]) * 32);
+                    const int cx = cb[col], cy = cb[cols + col], cz = cb[2 * cols + col];
+                    const int hx = cb[3 * cols + col], hy = cb[4 * cols + col], hz = cb[5 * cols + col];
+#pragma unroll
+                    for (int q = 0; q < kPerWarp; ++q) {
+                        const int k = warp + q * kMcWarps;
+                        const float x = (float)max(0, mi_abs(o0[q].x - cx, L) - hx);
+                        const float y = (float)max(0, mi_abs(o0[q].y - cy, L) - hy);
+                        const float z = (float)max(0, mi_abs(o0[q].z - cz, L) - hz);
+                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && k < nb && sh.rows[k][t] != 0;
+                        const unsigned mk = __ballot_sync(0xffffffffu, hit);
+                        if (lane == 0 && k < nb) near[k * A.words_cap + w] = mk;
+                        cnt[q] += __popc(mk);
                     }
-                    const unsigned mk = __ballot_sync(0xffffffffu, hit);
-                    if (lane == 0) near[k * A.words_cap + w] = mk;
-                    cnt += __popc(mk);
                 }
             }
-            if (lane == 0) sh.n_near[k] = cnt;
+#pragma unroll
+            for (int q = 0; q < kPerWarp; ++q)
+                if (lane == 0 && warp + q * kMcWarps < nb) sh.n_near[warp + q * kMcWarps] = cnt[q];
         }
         __syncthreads();
         // first item of each move (lane l holds moves l and l + 32), and this warp's items of a round
@@ -1009,9 +1073,9 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             if (!sh.acc[par][k] || a >= sh.natoms[k]) continue;
             const int ja = sh.a0[k] + a;
             const int4 p = sh.newp[par][k][a];
-            const int t = p.w, sp = sh.spos[k][a] - sh.rs[t];
-            if (sp >= 0 && sp < sh.rl[t]) {
-                const int slot = sh.blk[t] + sp, col = sh.wd[t] * 32 + (sp >> cs);
+            const int t = p.w, sp = sh.spos[k][a] - bx.type_start[t], ch = (sp >> cs) - sh.first[t];
+            if (ch >= 0 && ch % G == 0) {
+                const int lc = ch / G, col = sh.wd[t] * 32 + lc, slot = sh.blk[t] + (lc << cs) + (sp & ((1 << cs) - 1));
                 slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
                 // the chunk's box grows to hold the new position
                 atomicMax(&cb[3 * cols + col], mi_abs(p.x - cb[col], L));
