@@ -384,7 +384,7 @@ static int mc_layout(const epsr_box *h, McLayout *L)
     L->smem = ((size_t)L->slice_cap * 2 * sizeof(int4) + tables + 15) & ~(size_t)15;
     L->gslice = L->smem > kMcMaxDynSmem;
     if (L->gslice) {
-        for (int cs = 5; L->words_cap > kMcMaxWords && cs < 11; ) tables = sizes(++cs);
+        for (int cs = 5; L->words_cap > kMcMaxWords; ) tables = sizes(++cs);
         L->smem = ((size_t)kMcStageChunk * sizeof(uint4) + tables + 15) & ~(size_t)15;
         if (L->smem > kMcMaxDynSmem)
             return set_error(EPSR_EINVAL, "mc sweep: %zu bytes of tables per CTA (limit %zu)", L->smem, kMcMaxDynSmem);

@@ -35,7 +35,7 @@ void sq_plan_dims(const epsr_sq_plan *p, int *nQ, int *n_bins, int *max_cols);
 int sq_plan_stages(const epsr_sq_plan *p);
 
 // ---- Monte Carlo kernel ----------------------------------------------------------------------
-constexpr size_t kMcMaxDynSmem = 182 * 1024;   // with about 44 KB of static shared memory, under the 227 KB per CTA
+constexpr size_t kMcMaxDynSmem = 156 * 1024;   // with about 69 KB of static shared memory, under the 227 KB per CTA
 // exchange buffer of the sweep, per parity: the partial dU of every move of a batch from every
 // CTA ([kMcBatchMax][grid]), then kMcSlotStride - kMcBatchMax = kMcCorrPerCta floats per CTA of
 // which a box group uses its first CTA's share onwards for the batch-pair corrections

@@ -34,7 +34,7 @@ constexpr int kMcThreads = 512;
 constexpr int kMcWarps = kMcThreads / 32;
 constexpr int kBatchMax = kMcBatchMax;         // moves per batch: warp w takes moves w, w + 16, w + 32, w + 48
 constexpr int kPerWarp = kBatchMax / kMcWarps;  // moves per warp and batch
-constexpr int kMoveBlock = 128;                // move records staged in shared memory at once
+constexpr int kMoveRing = 2 * kBatchMax;        // move records held: a batch and the 64 moves after it
 constexpr int kCorrItems = kMcCorrItems;       // >= 496 pairs x 8 atoms (coarse items at G = 1)
 constexpr int kStage = kMcStageChunk;          // partners staged at once (slices in global memory)
 constexpr int kQueue = kBatchMax * kBatchMax / 2;   // near items of one round (in the corrections' buffer)
@@ -111,16 +111,14 @@ int launch_mc_moves(const BoxDev *boxes, const int *mol_start, int n_boxes, long
 }
 
 // ---- 2. persistent sweep ----------------------------------------------------------------------
-struct McShared {
-    BoxDev bx;
-    // batch records, double buffered by batch parity: the previous batch's accepted moves
-    // are the "pending" updates whose global writes may not yet be visible
-    int nb[2];
-    int nb_min;                              // first move of the batch that repeats a molecule
-    int mol[2][kBatchMax];
-    int acc[2][kBatchMax];
-    int4 newp[2][kBatchMax][kMaxMolAtoms];
-    // current batch
+// One batch of moves. Two are held: the next one is prepared while the grid barrier of the
+// current one is on its way.
+struct McBatch {
+    int nb;                                  // moves
+    int mm;                                  // largest molecule
+    int mol[kBatchMax];
+    int acc[kBatchMax];
+    int4 newp[kBatchMax][kMaxMolAtoms];
     int4 oldp[kBatchMax][kMaxMolAtoms];
     int natoms[kBatchMax];
     int a0[kBatchMax];
@@ -129,22 +127,30 @@ struct McShared {
     // per move and partner type: bit a of the low (high) byte set when moved atom a has a
     // Lennard-Jones (near-only) row with the type
     unsigned short rows[kBatchMax][kMaxTypes];
-    int n_near[kBatchMax];               // near chunks of each move
+    // first three atoms of each move on the 2^32-periodic grid, new and old: [move][atom][axis]
+    unsigned scn[kBatchMax][3][3];
+    unsigned sco[kBatchMax][3][3];
+    float thr[kBatchMax];
+    double u_acc[kBatchMax];
+    float intra[kBatchMax];                 // flexible molecules: change of the springs
+};
+
+struct McShared {
+    BoxDev bx;
+    McBatch b[2];
+    MoveRec ring[kMoveRing];                 // move t at t mod kMoveRing, copied in ahead of use
+    int nb_min;                              // first move of the next batch that repeats a molecule
+    int n_near[kBatchMax];                  // near chunks of each move
     // this CTA's partners: per type t, the chunks first[t], first[t] + G, .. of its sorted order, rl[t]
     // atoms in slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
     int first[kMaxTypes];
     int rl[kMaxTypes];
     int blk[kMaxTypes + 1];
     int wd[kMaxTypes + 1];
-    float thr[kBatchMax];
-    double u_acc[kBatchMax];
     float part[kBatchMax];
     float base[kBatchMax];
-    float intra[kBatchMax];                 // flexible molecules: change of the springs
-    int mm;                                  // largest molecule of the batch
-    MoveRec mv[kMoveBlock];                  // staged move records [mv_base, mv_base + kMoveBlock)
-    float acc_du[kMoveBlock];                // rank 0: dU of each decided move if accepted, else 0
     float dU[kBatchMax];
+    float acc_du[2 * kBatchMax];            // rank 0: dU of the decided moves if accepted, else 0
     int abort_flag;
     // leader-only running statistics
     long long st_att, st_acc, st_nonfinite;
@@ -277,6 +283,24 @@ __device__ __forceinline__ uint64_t far_du2(uint4 p, uint4 q, const LjSource &s,
     return f2_sub(f2_mul(f2_fma(C12, S6N, NC6), S6N), f2_mul(f2_fma(C12, S6O, NC6), S6O));
 }
 
+// Moved atom a of move k against partners of type t.
+__device__ __forceinline__ LjSource lj_source(const McBatch &b, int k, int a, int t, const BoxDev &bx)
+{
+    LjSource s;
+    if (a < 3) {
+        s.nx = b.scn[k][a][0]; s.ny = b.scn[k][a][1]; s.nz = b.scn[k][a][2];
+        s.ox = b.sco[k][a][0]; s.oy = b.sco[k][a][1]; s.oz = b.sco[k][a][2];
+    } else {
+        const int4 n = b.newp[k][a], o = b.oldp[k][a];
+        s.nx = scale32(n.x, bx.L, bx.sc_rcp); s.ny = scale32(n.y, bx.L, bx.sc_rcp); s.nz = scale32(n.z, bx.L, bx.sc_rcp);
+        s.ox = scale32(o.x, bx.L, bx.sc_rcp); s.oy = scale32(o.y, bx.L, bx.sc_rcp); s.oz = scale32(o.z, bx.L, bx.sc_rcp);
+    }
+    const PairRow &r = bx.row[b.oldp[k][a].w * kMaxTypes + t];
+    s.c12 = r.c12;
+    s.nc6 = -r.c6;
+    return s;
+}
+
 // Lennard-Jones terms of one moved atom each of two moves (s0, s1) with the groups of 32 slots
 // g0 .. g0 + ng - 1 of a run of n slots (sx: their 2^32-periodic copy, from its slot 0), group
 // g taken by a move unless bit g of its mask (near: left to the items) is set. A lane takes two
@@ -378,6 +402,137 @@ __device__ __forceinline__ float near_du(const int4 *np, const int4 *op, int m, 
     return valid ? acc : 0.f;
 }
 
+// Trial coordinates and what follows from them alone, for the moves of batch b (from move record
+// tn on): four moves of the warp at once, one per 8-lane group, one lane per atom of the molecule
+// (all three axes in the lane). oldp holds the current coordinates.
+template <bool CUT>
+__device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long long tn, int nb, const BoxDev &bx)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int L = bx.L, nt = bx.n_types;
+    const int k = warp + (lane >> 3) * kMcWarps;
+    const int kk = lane & 7;
+    const bool act = k < nb;
+    const MoveRec &mr = ring[(tn + (act ? k : 0)) & (kMoveRing - 1)];
+    const int a0 = mr.a0, m = act ? mr.m : 0;
+    int4 np4 = make_int4(0, 0, 0, 0), op4 = make_int4(0, 0, 0, 0);
+    if (kk < m) {
+        const int4 *op = b.oldp[k];
+        op4 = op[kk];
+        int nx, ny, nz;
+        if (mr.kind == 1) {
+            // minimum-image offsets from atom 0, summed over the molecule, and this atom's own
+            const int4 b0 = op[0];
+            long long sx = 0, sy = 0, sz = 0, ox = 0, oy = 0, oz = 0;
+            for (int i = 0; i < m; ++i) {
+                const int4 c = op[i];
+                const long long dx = mi_signed((long long)c.x - b0.x, L);
+                const long long dy = mi_signed((long long)c.y - b0.y, L);
+                const long long dz = mi_signed((long long)c.z - b0.z, L);
+                sx += dx; sy += dy; sz += dz;
+                if (i == kk) { ox = dx; oy = dy; oz = dz; }
+            }
+            const long long ux = (long long)m * ox - sx, uy = (long long)m * oy - sy,
+                            uz = (long long)m * oz - sz;
+            const int *R = mr.R;
+            // per axis: s 2^30 + R (m o - s), then floor((. + m 2^29) / 2^30) (32 bits) and
+            // floor division by m
+            const long long numx = sx * 1073741824LL + (long long)R[0] * ux + (long long)R[1] * uy +
+                                   (long long)R[2] * uz;
+            const long long numy = sy * 1073741824LL + (long long)R[3] * ux + (long long)R[4] * uy +
+                                   (long long)R[5] * uz;
+            const long long numz = sz * 1073741824LL + (long long)R[6] * ux + (long long)R[7] * uy +
+                                   (long long)R[8] * uz;
+            const long long half = (long long)m * 536870912LL;
+            nx = wrap_coord((long long)b0.x + floordiv32((int)((numx + half) >> 30), m) + mr.shift[0], L);
+            ny = wrap_coord((long long)b0.y + floordiv32((int)((numy + half) >> 30), m) + mr.shift[1], L);
+            nz = wrap_coord((long long)b0.z + floordiv32((int)((numz + half) >> 30), m) + mr.shift[2], L);
+        } else {
+            const bool moved = mr.kind != 2 || kk == mr.atom;
+            nx = wrap_coord((long long)op4.x + (moved ? mr.shift[0] : 0), L);
+            ny = wrap_coord((long long)op4.y + (moved ? mr.shift[1] : 0), L);
+            nz = wrap_coord((long long)op4.z + (moved ? mr.shift[2] : 0), L);
+        }
+        np4 = make_int4(nx, ny, nz, op4.w);
+        b.newp[k][kk] = np4;
+        if (kk < 3) {
+            b.scn[k][kk][0] = scale32(nx, L, bx.sc_rcp);
+            b.scn[k][kk][1] = scale32(ny, L, bx.sc_rcp);
+            b.scn[k][kk][2] = scale32(nz, L, bx.sc_rcp);
+            b.sco[k][kk][0] = scale32(op4.x, L, bx.sc_rcp);
+            b.sco[k][kk][1] = scale32(op4.y, L, bx.sc_rcp);
+            b.sco[k][kk][2] = scale32(op4.z, L, bx.sc_rcp);
+        }
+    }
+    __syncwarp();
+    if (act && kk == 0) {
+        // flexible molecules: change of the intra-molecular springs, written without
+        // cancellation: k[(r' - d)^2 - (r - d)^2] = k (r' - r)(r' + r - 2d), with
+        // r' - r = (r'^2 - r^2) / (r' + r) from the exact integer squared distances
+        float di = 0.f;
+        if (bx.move_kind == EPSR_MOVE_FLEXIBLE_MOLECULE)
+            for (int i = 0; i < m; ++i)
+                for (int j = i + 1; j < m; ++j) {
+                    const int4 ni = b.newp[k][i], nj = b.newp[k][j];
+                    const int t = ni.w * kMaxTypes + nj.w;
+                    if (bx.bond_k[t] == 0.0) continue;
+                    const long long d2n = dist2(ni, nj, L), d2o = dist2(b.oldp[k][i], b.oldp[k][j], L);
+                    if (d2n == d2o) continue;
+                    const float rn = sqrtf((float)d2n * bx.inv_s2), ro = sqrtf((float)d2o * bx.inv_s2);
+                    const float dr = (float)(d2n - d2o) * bx.inv_s2 / (rn + ro);
+                    di = fmaf((float)bx.bond_k[t] * dr, rn + ro - 2.f * (float)bx.bond_d[t], di);
+                }
+        b.intra[k] = di;
+        atomicMax(&b.mm, m);
+        b.natoms[k] = m;
+        b.a0[k] = a0;
+        b.thr[k] = mr.thr;
+        b.u_acc[k] = mr.u_acc;
+    }
+    // near sphere: every old and new atom position lies within `reach` of old atom 0 (a bound in
+    // FP32, rounded up by the margin), so a partner beyond near_fx + reach of it has no near term
+    float reach2 = 0.f;
+    if (kk < m) {
+        const int4 o = b.oldp[k][0];
+        reach2 = fmaxf(g2_of(sep(op4, o, L)), g2_of(sep(np4, o, L)));
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
+    if (act && kk == 0) {
+        const float r = ((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f;
+        b.hw2[k] = r * r;
+    }
+    // rows of the moved atoms with partner type kk (an atom that stays where it is has none)
+    if (act) {
+        unsigned lj = 0u, nr = 0u;
+        for (int a = 0; a < m && kk < nt; ++a) {
+            const int4 n = b.newp[k][a], o = b.oldp[k][a];
+            if (n.x == o.x && n.y == o.y && n.z == o.z) continue;
+            const PairRow &pr = bx.row[n.w * kMaxTypes + kk];
+            if (lj_full_row<CUT>(pr, bx)) lj |= 1u << a;
+            else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
+        }
+        b.rows[k][kk] = (unsigned short)(lj | (nr << 8));
+    }
+    __syncwarp();
+}
+
+// Index in batch b of an accepted move of molecule mol, or -1 (whole warp; the molecules of a
+// batch are distinct).
+__device__ __forceinline__ int accepted_index(const McBatch &b, int mol, int lane)
+{
+    const bool hit0 = lane < b.nb && b.acc[lane] && b.mol[lane] == mol;
+    const bool hit1 = lane + 32 < b.nb && b.acc[lane + 32] && b.mol[lane + 32] == mol;
+    const unsigned h0 = __ballot_sync(0xffffffffu, hit0), h1 = __ballot_sync(0xffffffffu, hit1);
+    return h1 ? 63 - __clz(h1) : h0 ? 31 - __clz(h0) : -1;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // GSLICE: the partner slices live in global memory ([grid][slice_cap], read through L1/L2)
 // because they do not fit in shared memory; the thresholds, EP table and cell index stay
 // in shared memory either way.
@@ -392,7 +547,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
 
     if (tid == 0) {
         sh.bx = A.boxes[box];
-        sh.nb[0] = sh.nb[1] = 0;
+        sh.b[0].nb = sh.b[1].nb = 0;
+        sh.b[0].mm = sh.b[1].mm = 0;
         sh.nb_min = 1 << 30;
         sh.abort_flag = 0;
         sh.st_att = sh.st_acc = sh.st_nonfinite = 0;
@@ -488,179 +644,309 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     // square of the batch); above 32 only with 8 or more CTAs per box, so that a CTA's share
     // of the batch-pair corrections fits its item buffer
     const int batch_k = min(A.batch_k > 0 ? A.batch_k : (G >= 64 ? 64 : G >= 32 ? 32 : 16), G >= 8 ? kBatchMax : 32);
-    const MoveRec *moves = A.moves + (size_t)box * A.chunk;
-    unsigned seq = 0;
-    int par = 0;
+    const int4 *moves = reinterpret_cast<const int4 *>(A.moves + (size_t)box * A.chunk);
+    constexpr int kRecI4 = (int)(sizeof(MoveRec) / sizeof(int4));
+    // copies the records of moves [m0, m1) into the ring (asynchronously, 16 bytes a thread)
+    auto copy_records = [&](long long m0, long long m1) {
+        for (int i = tid; i < (int)(m1 - m0) * kRecI4; i += kMcThreads) {
+            const long long t = m0 + i / kRecI4;
+            cp_async16(reinterpret_cast<int4 *>(&sh.ring[t & (kMoveRing - 1)]) + i % kRecI4, moves + t * kRecI4 + i % kRecI4);
+        }
+    };
+    long long held = min(A.n_moves, (long long)kMoveRing);      // records copied so far
+    copy_records(0, held);
+    cp_async_wait();
+    __syncthreads();
 
-    long long mv_base = 0, mv_end = 0;
-    for (long long t0 = 0; t0 < A.n_moves; par ^= 1) {
-        const int kmax = (int)min((long long)batch_k, A.n_moves - t0);
-        if (t0 + kmax > mv_end) {           // stage the next block of move records
-            if (rank == 0 && warp == 0) block_sum_du(sh.acc_du, (int)(t0 - mv_base), lane, sh.st_sum);
-            mv_base = t0;
-            mv_end = min(A.n_moves, t0 + kMoveBlock);
-            const int4 *src = reinterpret_cast<const int4 *>(moves + mv_base);
-            int4 *dst = reinterpret_cast<int4 *>(sh.mv);
-            const int n4 = (int)(mv_end - mv_base) * (int)(sizeof(MoveRec) / sizeof(int4));
-            for (int i = tid; i < n4; i += kMcThreads) dst[i] = src[i];
-            __syncthreads();
-        }
-        // ---- A. molecules of the batch; it ends before the first repeated molecule -----------
-        // (every pair of the batch's candidate moves tested once, across the CTA)
-        {
-            const MoveRec *mv = sh.mv + (t0 - mv_base);
-            for (int pq = tid; pq < kmax * (kmax - 1) / 2; pq += kMcThreads) {
-                const int k = pair_hi(pq), k1 = pq - k * (k - 1) / 2;
-                if (mv[k].mol == mv[k1].mol) atomicMin(&sh.nb_min, k);
+    unsigned seq = 0;
+    int par = 0, nb = 0;             // the current batch: b[par], moves [t0, t0 + nb)
+    int n_du = 0;                    // entries of acc_du (rank 0)
+    const int gk = tid >> 3, gsub = tid & 7;   // gather group: move gk, member gsub
+    int n_local = 0, mm = 0;         // this CTA's share of the current batch's corrections
+    bool fine = false;
+    long long t0 = 0;
+    for (;;) {
+        McBatch &cur = sh.b[par], &nxt = sh.b[par ^ 1];
+        const long long tn = t0 + nb;
+        int nb_next = 0;
+        // ---- A, B. the next batch, while the partials of the current one reach the other CTAs --------
+        // Its molecules and end, the current coordinates of its molecules and the trial coordinates
+        // (integer arithmetic). The decisions of the current batch are not known yet: the few
+        // molecules that they move are taken up again after them. Coordinates come from the previous
+        // batch's accepted moves (b[par ^ 1], about to be replaced; their global update may not be
+        // visible yet), else from the global array, whose value for a molecule that the current batch
+        // moves is dropped later.
+        if (tn < A.n_moves) {
+            const int kmax = (int)min((long long)batch_k, A.n_moves - tn);
+            if (gk < kmax) {                // the batch ends before the first repeated molecule
+                const int mol = sh.ring[(tn + gk) & (kMoveRing - 1)].mol;
+                bool dup = false;
+                for (int j = gsub; j < gk; j += 8) dup |= sh.ring[(tn + j) & (kMoveRing - 1)].mol == mol;
+                if (dup) atomicMin(&sh.nb_min, gk);
             }
-            if (tid < kBatchMax) sh.mol[par][tid] = tid < kmax ? mv[tid].mol : -1 - tid;
-            if (tid == 0) sh.mm = 0;
-        }
-        __syncthreads();
-        const int nb = min(kmax, sh.nb_min);
-        if (tid == 0) sh.nb[par] = nb;
-        // ---- B. current and trial coordinates of each moved molecule (integer arithmetic) ----
-        // Current coordinates of a warp's four molecules: from the previous batch's accepted move
-        // of the molecule if there is one (its global update may not be visible yet), else from
-        // the global coordinates. The global loads of all four go out first (one round trip;
-        // a value that a pending move replaces is loaded and dropped).
-        {
             int4 gc[kPerWarp];
             int gp[kPerWarp];
-            const int q = par ^ 1;
 #pragma unroll
             for (int h = 0; h < kPerWarp; ++h) {
                 const int k = warp + h * kMcWarps;
                 gc[h] = make_int4(0, 0, 0, 0);
                 gp[h] = 0;
-                if (k < nb) {
-                    const MoveRec &mr = sh.mv[t0 + k - mv_base];
+                if (k < kmax) {
+                    const MoveRec &mr = sh.ring[(tn + k) & (kMoveRing - 1)];
                     if (lane < mr.m) {
                         gc[h] = __ldcg(&A.coords[bx.atom0 + mr.a0 + lane]);
                         gp[h] = A.pos_of[bx.atom0 + mr.a0 + lane];
                     }
                 }
             }
+            const long long want = min(A.n_moves, tn + kMoveRing);
+            copy_records(held, want);
+            held = want;
+            int mol[kPerWarp];
 #pragma unroll
             for (int h = 0; h < kPerWarp; ++h) {
                 const int k = warp + h * kMcWarps;
-                if (k < nb) {
-                    const MoveRec &mr = sh.mv[t0 + k - mv_base];
-                    const int mol = sh.mol[par][k];
-                    const bool hit0 = lane < sh.nb[q] && sh.acc[q][lane] && sh.mol[q][lane] == mol;
-                    const bool hit1 = lane + 32 < sh.nb[q] && sh.acc[q][lane + 32] && sh.mol[q][lane + 32] == mol;
-                    const unsigned h0 = __ballot_sync(0xffffffffu, hit0), h1 = __ballot_sync(0xffffffffu, hit1);
-                    // molecules of a batch are distinct: at most one hit
-                    const int pidx = h1 ? 63 - __clz(h1) : h0 ? 31 - __clz(h0) : -1;
-                    if (lane < mr.m) {
-                        sh.oldp[k][lane] = pidx >= 0 ? sh.newp[q][pidx][lane] : gc[h];
-                        sh.spos[k][lane] = gp[h] - (int)bx.atom0;
+                mol[h] = -1;
+                if (k < kmax) {
+                    mol[h] = sh.ring[(tn + k) & (kMoveRing - 1)].mol;
+                    const int idx = accepted_index(nxt, mol[h], lane);
+                    if (idx >= 0 && lane < kMaxMolAtoms) gc[h] = nxt.newp[idx][lane];
+                }
+            }
+            __syncthreads();                // the previous batch is no longer needed
+            nb_next = min(kmax, sh.nb_min);
+            if (tid == 0) nxt.nb = nb_next;
+#pragma unroll
+            for (int h = 0; h < kPerWarp; ++h) {
+                const int k = warp + h * kMcWarps;
+                if (k < nb_next) {
+                    if (lane < sh.ring[(tn + k) & (kMoveRing - 1)].m) {
+                        nxt.oldp[k][lane] = gc[h];
+                        nxt.spos[k][lane] = gp[h] - (int)bx.atom0;
                     }
+                    if (lane == 0) nxt.mol[k] = mol[h];
                 }
             }
             __syncwarp();
+            trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
         }
-        // Trial coordinates: the four moves of a warp at once, one per 8-lane group, one lane per
-        // atom of the molecule (all three axes in the lane).
-        {
-            const int k = warp + (lane >> 3) * kMcWarps;
-            const int kk = lane & 7;
-            const bool act = k < nb;
-            const MoveRec &mr = sh.mv[t0 + (act ? k : 0) - mv_base];
-            const int a0 = mr.a0, m = act ? mr.m : 0;
-            int4 np4 = make_int4(0, 0, 0, 0), op4 = make_int4(0, 0, 0, 0);
-            if (kk < m) {
-                const int4 *op = sh.oldp[k];
-                op4 = op[kk];
-                int nx, ny, nz;
-                if (mr.kind == 1) {
-                    // minimum-image offsets from atom 0, summed over the molecule, and this atom's own
-                    const int4 b0 = op[0];
-                    long long sx = 0, sy = 0, sz = 0, ox = 0, oy = 0, oz = 0;
-                    for (int i = 0; i < m; ++i) {
-                        const int4 c = op[i];
-                        const long long dx = mi_signed((long long)c.x - b0.x, L);
-                        const long long dy = mi_signed((long long)c.y - b0.y, L);
-                        const long long dz = mi_signed((long long)c.z - b0.z, L);
-                        sx += dx; sy += dy; sz += dz;
-                        if (i == kk) { ox = dx; oy = dy; oz = dz; }
-                    }
-                    const long long ux = (long long)m * ox - sx, uy = (long long)m * oy - sy,
-                                    uz = (long long)m * oz - sz;
-                    const int *R = mr.R;
-                    // per axis: s 2^30 + R (m o - s), then floor((. + m 2^29) / 2^30) (32 bits) and
-                    // floor division by m
-                    const long long numx = sx * 1073741824LL + (long long)R[0] * ux + (long long)R[1] * uy +
-                                           (long long)R[2] * uz;
-                    const long long numy = sy * 1073741824LL + (long long)R[3] * ux + (long long)R[4] * uy +
-                                           (long long)R[5] * uz;
-                    const long long numz = sz * 1073741824LL + (long long)R[6] * ux + (long long)R[7] * uy +
-                                           (long long)R[8] * uz;
-                    const long long half = (long long)m * 536870912LL;
-                    nx = wrap_coord((long long)b0.x + floordiv32((int)((numx + half) >> 30), m) + mr.shift[0], L);
-                    ny = wrap_coord((long long)b0.y + floordiv32((int)((numy + half) >> 30), m) + mr.shift[1], L);
-                    nz = wrap_coord((long long)b0.z + floordiv32((int)((numz + half) >> 30), m) + mr.shift[2], L);
-                } else {
-                    const bool moved = mr.kind != 2 || kk == mr.atom;
-                    nx = wrap_coord((long long)op4.x + (moved ? mr.shift[0] : 0), L);
-                    ny = wrap_coord((long long)op4.y + (moved ? mr.shift[1] : 0), L);
-                    nz = wrap_coord((long long)op4.z + (moved ? mr.shift[2] : 0), L);
-                }
-                np4 = make_int4(nx, ny, nz, op4.w);
-                sh.newp[par][k][kk] = np4;
-            }
-            __syncwarp();
-            if (act && kk == 0) {
-                // flexible molecules: change of the intra-molecular springs, written without
-                // cancellation: k[(r' - d)^2 - (r - d)^2] = k (r' - r)(r' + r - 2d), with
-                // r' - r = (r'^2 - r^2) / (r' + r) from the exact integer squared distances
-                float di = 0.f;
-                if (bx.move_kind == EPSR_MOVE_FLEXIBLE_MOLECULE)
-                    for (int i = 0; i < m; ++i)
-                        for (int j = i + 1; j < m; ++j) {
-                            const int4 ni = sh.newp[par][k][i], nj = sh.newp[par][k][j];
-                            const int t = ni.w * kMaxTypes + nj.w;
-                            if (bx.bond_k[t] == 0.0) continue;
-                            const long long d2n = dist2(ni, nj, L), d2o = dist2(sh.oldp[k][i], sh.oldp[k][j], L);
-                            if (d2n == d2o) continue;
-                            const float rn = sqrtf((float)d2n * bx.inv_s2), ro = sqrtf((float)d2o * bx.inv_s2);
-                            const float dr = (float)(d2n - d2o) * bx.inv_s2 / (rn + ro);
-                            di = fmaf((float)bx.bond_k[t] * dr, rn + ro - 2.f * (float)bx.bond_d[t], di);
+        if (nb > 0) {
+            // ---- D. gather the partials of the box's CTA group (one bounded grid barrier) -------
+            // Lane 0 of warp 0 polls the group's counter with acquire loads; the CTA barrier after it
+            // orders every thread's reads after the acquire.
+            const bool gin = gk < nb;
+            float cv[8];                          // corrections (j, gk), j = gsub + 8 i < gk
+            float gv = 0.f, gw = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) cv[i] = 0.f;
+            if (G > 1) {
+                const float *ps = A.slots + (size_t)(seq & 1u) * A.grid * kMcSlotStride;
+                const float *pc = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
+                if (tid == 0) {
+                    const unsigned target = seq * (unsigned)G;
+                    const uint64_t t_start = globaltimer_ns();
+                    long long it = 0;
+                    bool timed_out = false;
+                    while (ld_acquire_gpu(&A.flags[box]) < target) {
+                        if ((++it & 255) == 0 &&
+                            ((globaltimer_ns() - t_start > A.timeout_ns) || it > A.max_spin ||
+                             ld_relaxed_gpu(A.status) != 0)) {
+                            timed_out = true;
+                            break;
                         }
-                sh.intra[k] = di;
-                atomicMax(&sh.mm, m);
-                sh.natoms[k] = m;
-                sh.a0[k] = a0;
-                sh.thr[k] = mr.thr;
-                sh.u_acc[k] = mr.u_acc;
+                    }
+                    if (timed_out) {
+                        atomicOr(A.status, kStatusTimeout);
+                        sh.abort_flag = 1;
+                    }
+                }
+                __syncthreads();
+                if (sh.abort_flag) {
+                    cp_async_wait();
+                    return;
+                }
+                // 8 threads per move k: every 8th CTA's partial and every 8th correction (j, k),
+                // j < k, all loads in flight at once (one L2 round trip)
+                if (gin) {
+                    const float *pk = ps + (size_t)gk * A.grid + bx.cta0;
+                    const float *ck = pc + gk * (gk - 1) / 2;
+                    float pv[kGatherLoads];
+#pragma unroll
+                    for (int i = 0; i < kGatherLoads; ++i) {
+                        const int r = gsub + 8 * i;
+                        pv[i] = r < G ? __ldcg(&pk[r]) : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int j = gsub + 8 * i;
+                        cv[i] = j < gk ? __ldcg(&ck[j]) : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < kGatherLoads; ++i) gv += pv[i];
+                    for (int r = gsub + 8 * kGatherLoads; r < G; r += 8) gv += __ldcg(&pk[r]);
+                }
+            } else if (gin) {
+                gv = gsub == 0 ? sh.part[gk] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int j = gsub + 8 * i;
+                    cv[i] = j < gk ? corr_sum(corr_part, gk * (gk - 1) / 2 + j, mm, fine) : 0.f;
+                }
             }
-            // near sphere: every old and new atom position lies within `reach` of old atom 0 (a bound in
-            // FP32, rounded up by the margin), so a partner beyond near_fx + reach of it has no near term
-            float reach2 = 0.f;
-            if (kk < m) {
-                const int4 o = sh.oldp[k][0];
-                reach2 = fmaxf(g2_of(sep(op4, o, L)), g2_of(sep(np4, o, L)));
+            // the group's sums in a fixed shuffle tree (the same order in every run): the move's
+            // partial dU and the magnitude sum of its corrections
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int j = gsub + 8 * i;
+                if (gin && j < gk) corr[j][gk] = cv[i];
+                gw += fabsf(cv[i]);
             }
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
-            if (act && kk == 0) {
-                const float r = ((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f;
-                sh.hw2[k] = r * r;
+            for (int o = 4; o > 0; o >>= 1) {
+                gv += __shfl_xor_sync(0xffffffffu, gv, o);
+                gw += __shfl_xor_sync(0xffffffffu, gw, o);
             }
-            // rows of the moved atoms with partner type kk (an atom that stays where it is has none)
-            if (act) {
-                unsigned lj = 0u, nr = 0u;
-                for (int a = 0; a < m && kk < nt; ++a) {
-                    const int4 n = sh.newp[par][k][a], o = sh.oldp[k][a];
-                    if (n.x == o.x && n.y == o.y && n.z == o.z) continue;
-                    const PairRow &pr = bx.row[n.w * kMaxTypes + kk];
-                    if (lj_full_row<CUT>(pr, bx)) lj |= 1u << a;
-                    else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
+            // ---- F. Metropolis decisions of the batch, in order: move k's dU includes the
+            // corrections of every earlier accepted move. Fast path: when no move's decision can
+            // change with any subset of its earlier corrections (|dU - threshold| beyond the sum of
+            // their magnitudes plus the FP32 rounding of that many additions), every group decides
+            // its move at once and then adds its accepted corrections (fixed tree order); otherwise
+            // warp 0 decides one move after the other (lane l holds moves l and l + 32) and adds
+            // the corrections in the chain's order. Both give the same decisions.
+            {
+                const float d = gin ? gv + cur.intra[gk] : 0.f;
+                const float thr = gin ? cur.thr[gk] : 0.f;
+                const float wv = gw + (fabsf(d) + gw) * 0x1p-16f;
+                const bool sure = !gin || metropolis(d + wv, thr) || !metropolis(d - wv, thr);
+                if (gin && gsub == 0) sh.base[gk] = gv;
+                if (__syncthreads_and(sure)) {
+                    const bool acc = gin && metropolis(d, thr);
+                    if (gin && gsub == 0) cur.acc[gk] = acc;
+                    __syncthreads();
+                    float c = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int j = gsub + 8 * i;
+                        if (j < gk && cur.acc[j]) c += cv[i];
+                    }
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                    if (gin && gsub == 0) sh.dU[gk] = d + c;
+                } else if (warp == 0) {
+                    const bool in0 = lane < nb, in1 = lane + 32 < nb;
+                    float d0 = in0 ? sh.base[lane] + cur.intra[lane] : 0.f;
+                    float d1 = in1 ? sh.base[lane + 32] + cur.intra[lane + 32] : 0.f;
+                    const float thr0 = in0 ? cur.thr[lane] : 0.f, thr1 = in1 ? cur.thr[lane + 32] : 0.f;
+                    int acc0 = 0, acc1 = 0;
+#pragma unroll 8
+                    for (int j = 0; j < 32; ++j) {
+                        if (j < nb) {
+                            const float c0 = corr[j][lane], c1 = corr[j][lane + 32];
+                            const int aj = __shfl_sync(0xffffffffu, metropolis(d0, thr0), j);
+                            if (lane == j) acc0 = aj;
+                            if (aj) {
+                                if (lane > j) d0 += c0;
+                                d1 += c1;
+                            }
+                        }
+                    }
+#pragma unroll 8
+                    for (int j = 32; j < kBatchMax; ++j) {
+                        if (j < nb) {
+                            const float c1 = corr[j][lane + 32];
+                            const int aj = __shfl_sync(0xffffffffu, metropolis(d1, thr1), j - 32);
+                            if (lane == j - 32) acc1 = aj;
+                            if (aj && lane + 32 > j) d1 += c1;
+                        }
+                    }
+                    if (in0) {
+                        sh.dU[lane] = d0;
+                        cur.acc[lane] = acc0;
+                    }
+                    if (in1) {
+                        sh.dU[lane + 32] = d1;
+                        cur.acc[lane + 32] = acc1;
+                    }
                 }
-                sh.rows[k][kk] = (unsigned short)(lj | (nr << 8));
+            }
+            __syncthreads();
+            if (rank == 0 && warp == 0) {
+                // counts now; the FP64 sum of accepted dU over a few batches at once
+                const bool in0 = lane < nb, in1 = lane + 32 < nb;
+                const bool acc0 = in0 && cur.acc[lane], acc1 = in1 && cur.acc[lane + 32];
+                const float d0 = in0 ? sh.dU[lane] : 0.f, d1 = in1 ? sh.dU[lane + 32] : 0.f;
+                const unsigned b_acc = __ballot_sync(0xffffffffu, acc0), b_acc1 = __ballot_sync(0xffffffffu, acc1);
+                const unsigned b_nf = __ballot_sync(0xffffffffu, in0 && !isfinite(d0)),
+                               b_nf1 = __ballot_sync(0xffffffffu, in1 && !isfinite(d1));
+                if (in0) sh.acc_du[n_du + lane] = acc0 ? d0 : 0.f;
+                if (in1) sh.acc_du[n_du + lane + 32] = acc1 ? d1 : 0.f;
+                if (lane == 0) {
+                    sh.st_att += nb;
+                    sh.st_acc += __popc(b_acc) + __popc(b_acc1);
+                    sh.st_nonfinite += __popc(b_nf) + __popc(b_nf1);
+                }
+                __syncwarp();
+                if (n_du + nb > kBatchMax) block_sum_du(sh.acc_du, n_du + nb, lane, sh.st_sum);
+            }
+            n_du = n_du + nb > kBatchMax ? 0 : n_du + nb;
+            // ---- G. apply accepted moves: shared slice, global coordinates, log ------------------
+            for (int it = tid; it < nb * kMaxMolAtoms; it += kMcThreads) {
+                const int k = it / kMaxMolAtoms, a = it % kMaxMolAtoms;
+                if (!cur.acc[k] || a >= cur.natoms[k]) continue;
+                const int ja = cur.a0[k] + a;
+                const int4 p = cur.newp[k][a];
+                const int t = p.w, sp = cur.spos[k][a] - bx.type_start[t], ch = (sp >> cs) - sh.first[t];
+                if (ch >= 0 && ch % G == 0) {
+                    const int lc = ch / G, col = sh.wd[t] * 32 + lc, slot = sh.blk[t] + (lc << cs) + (sp & ((1 << cs) - 1));
+                    slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
+                    // the chunk's box grows to hold the new position
+                    atomicMax(&cb[3 * cols + col], mi_abs(p.x - cb[col], L));
+                    atomicMax(&cb[4 * cols + col], mi_abs(p.y - cb[cols + col], L));
+                    atomicMax(&cb[5 * cols + col], mi_abs(p.z - cb[2 * cols + col], L));
+                    if (!GSLICE)
+                        sx[slot] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
+                                              scale32(p.z, L, bx.sc_rcp), (unsigned)ja);
+                }
+                if (rank == 0) A.coords[bx.atom0 + ja] = p;
+            }
+            if (rank == 0 && A.log && tid < nb) {
+                epsr_move_log *lg = A.log + (size_t)box * A.log_stride + (size_t)(A.log_off + t0 + tid);
+                lg->mol = cur.mol[tid];
+                lg->accepted = cur.acc[tid];
+                lg->dU = sh.dU[tid];
+                lg->n_atoms = cur.natoms[tid];
+                lg->u_acc = cur.u_acc[tid];
+                for (int a = 0; a < kMaxMolAtoms; ++a) {
+                    const int4 p = a < cur.natoms[tid] ? cur.newp[tid][a] : make_int4(0, 0, 0, 0);
+                    lg->trial[a][0] = p.x; lg->trial[a][1] = p.y; lg->trial[a][2] = p.z;
+                }
+            }
+            // ---- the moves of the next batch whose molecules the current one has moved --------------
+            if (nb_next > 0) {
+                bool again = false;
+#pragma unroll
+                for (int h = 0; h < kPerWarp; ++h) {
+                    const int k = warp + h * kMcWarps;
+                    if (k >= nb_next) continue;
+                    const int idx = accepted_index(cur, nxt.mol[k], lane);
+                    if (idx < 0) continue;
+                    again = true;
+                    if (lane < cur.natoms[idx]) nxt.oldp[k][lane] = cur.newp[idx][lane];
+                }
+                __syncwarp();
+                if (again) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
             }
         }
+        if (nb_next == 0) break;
+        par ^= 1;
+        t0 = tn;
+        nb = nb_next;
         __syncthreads();
+        McBatch &now = sh.b[par];
+        if (tid == 0) {
+            sh.nb_min = 1 << 30;
+            sh.b[par ^ 1].mm = 0;
+        }
         // ---- E. pair-energy corrections between the batch's moved molecules -----------------
         // Pair pq = (k1 < k) is computed by CTA pq mod G of the box's group, as items (pq, atom
         // a of move k) against the whole molecule of move k1, spread one per warp before the
@@ -669,8 +955,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // move k1 at its new (side 0) or old (side 1) position, one pair_du each, so a CTA's
         // share (18 items for water with G >= 120) runs as one warp's lanes in parallel.
         const int npq = nb * (nb - 1) / 2;
-        const int mm = sh.mm;
-        const int n_local = npq > rank ? (npq - rank + G - 1) / G : 0;
+        mm = now.mm;
+        n_local = npq > rank ? (npq - rank + G - 1) / G : 0;
         const int n_items = n_local * mm * mm * 2;
         if (n_items <= kCorrItems) {
             for (int it = tid; it < n_items; it += kMcThreads) {
@@ -679,9 +965,9 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 const int k = pair_hi(pq);
                 const int k1 = pq - k * (k - 1) / 2;
                 float v = 0.f;
-                if (a < sh.natoms[k] && b < sh.natoms[k1]) {
-                    const int4 na = sh.newp[par][k][a], oa = sh.oldp[k][a];
-                    const int4 p1 = side ? sh.oldp[k1][b] : sh.newp[par][k1][b];
+                if (a < now.natoms[k] && b < now.natoms[k1]) {
+                    const int4 na = now.newp[k][a], oa = now.oldp[k][a];
+                    const int4 p1 = side ? now.oldp[k1][b] : now.newp[k1][b];
                     v = pair_du<CUT>(sep(na, p1, L), sep(oa, p1, L), bx.row[na.w * kMaxTypes + p1.w], bx, T, ep);
                 }
                 corr_part[it] = v;
@@ -692,10 +978,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 const int k = pair_hi(pq);
                 const int k1 = pq - k * (k - 1) / 2;
                 float ca = 0.f;
-                if (a < sh.natoms[k]) {
-                    const int4 na = sh.newp[par][k][a], oa = sh.oldp[k][a];
-                    for (int b = 0; b < sh.natoms[k1]; ++b) {
-                        const int4 nb1 = sh.newp[par][k1][b], ob1 = sh.oldp[k1][b];
+                if (a < now.natoms[k]) {
+                    const int4 na = now.newp[k][a], oa = now.oldp[k][a];
+                    for (int b = 0; b < now.natoms[k1]; ++b) {
+                        const int4 nb1 = now.newp[k1][b], ob1 = now.oldp[k1][b];
                         const PairRow &pr = bx.row[na.w * kMaxTypes + nb1.w];
                         ca += pair_du_cold<CUT>(sep(na, nb1, L), sep(oa, nb1, L), pr, bx, T, ep) -
                               pair_du_cold<CUT>(sep(na, ob1, L), sep(oa, ob1, L), pr, bx, T, ep);
@@ -704,7 +990,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 corr_part[it] = ca;
             }
         }
-        const bool fine = n_items <= kCorrItems;
+        fine = n_items <= kCorrItems;
         // ---- C. partial dU of the batch's moves against this CTA's slice ---------------------
         // Near chunks: those whose box meets the near sphere of the move. A (move, chunk) item
         // takes all pairs of the moved atoms with the chunk's partners in the cancellation-free form,
@@ -720,8 +1006,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
 #pragma unroll
             for (int q = 0; q < kPerWarp; ++q) {
                 const int k = min(warp + q * kMcWarps, nb - 1);
-                o0[q] = sh.oldp[k][0];
-                hw2[q] = A.near_all ? 3e38f : sh.hw2[k];
+                o0[q] = now.oldp[k][0];
+                hw2[q] = A.near_all ? 3e38f : now.hw2[k];
                 cnt[q] = 0;
             }
             for (int t = 0; t < nt; ++t) {
@@ -736,7 +1022,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                         const float x = (float)max(0, mi_abs(o0[q].x - cx, L) - hx);
                         const float y = (float)max(0, mi_abs(o0[q].y - cy, L) - hy);
                         const float z = (float)max(0, mi_abs(o0[q].z - cz, L) - hz);
-                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && k < nb && sh.rows[k][t] != 0;
+                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && k < nb && now.rows[k][t] != 0;
                         const unsigned mk = __ballot_sync(0xffffffffu, hit);
                         if (lane == 0 && k < nb) near[k * A.words_cap + w] = mk;
                         cnt[q] += __popc(mk);
@@ -748,6 +1034,14 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 if (lane == 0 && warp + q * kMcWarps < nb) sh.n_near[warp + q * kMcWarps] = cnt[q];
         }
         __syncthreads();
+        // the CTA's corrections go out now; the partials of every move from its own warp below
+        ++seq;
+        float *ps = A.slots + (size_t)(seq & 1u) * A.grid * kMcSlotStride;
+        const bool arrive = G > 1 && cta != A.skip_arrival_cta;
+        if (arrive) {
+            float *pc = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
+            for (int u = kMcThreads - 1 - tid; u < n_local; u += kMcThreads) pc[rank + u * G] = corr_sum(corr_part, u, mm, fine);
+        }
         // first item of each move (lane l holds moves l and l + 32), and this warp's items of a round
         int n_all;
         int base[kPerWarp];
@@ -810,29 +1104,12 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                             const int k0 = warp + h * kMcWarps, k1 = k0 + kMcWarps;
                             if (k0 >= nb) continue;
                             const bool two = k1 < nb;
-                            const unsigned l0 = sh.rows[k0][t] & 0xFFu, l1 = two ? sh.rows[k1][t] & 0xFFu : 0u;
+                            const unsigned l0 = now.rows[k0][t] & 0xFFu, l1 = two ? now.rows[k1][t] & 0xFFu : 0u;
                             for (unsigned todo = l0 | l1; todo; todo &= todo - 1u) {
                                 const int a = __ffs(todo) - 1;
                                 const bool on0 = (l0 >> a) & 1u, on1 = (l1 >> a) & 1u;
-                                LjSource s0, s1;
-                                {
-                                    const int kx = on0 ? k0 : k1, ky = on1 ? k1 : k0;
-                                    // lanes 0..5 convert the coordinates of one move, 8..13 of the other
-                                    const int4 *pp = (lane & 7) < 3 ? sh.newp[par][lane & 8 ? ky : kx] : sh.oldp[lane & 8 ? ky : kx];
-                                    const int ax = (lane & 7) % 3;
-                                    const int xc = ax == 0 ? pp[a].x : ax == 1 ? pp[a].y : pp[a].z;
-                                    const unsigned sc = scale32(xc, L, bx.sc_rcp);
-                                    s0.nx = __shfl_sync(0xffffffffu, sc, 0); s0.ny = __shfl_sync(0xffffffffu, sc, 1);
-                                    s0.nz = __shfl_sync(0xffffffffu, sc, 2); s0.ox = __shfl_sync(0xffffffffu, sc, 3);
-                                    s0.oy = __shfl_sync(0xffffffffu, sc, 4); s0.oz = __shfl_sync(0xffffffffu, sc, 5);
-                                    s1.nx = __shfl_sync(0xffffffffu, sc, 8); s1.ny = __shfl_sync(0xffffffffu, sc, 9);
-                                    s1.nz = __shfl_sync(0xffffffffu, sc, 10); s1.ox = __shfl_sync(0xffffffffu, sc, 11);
-                                    s1.oy = __shfl_sync(0xffffffffu, sc, 12); s1.oz = __shfl_sync(0xffffffffu, sc, 13);
-                                    const PairRow &ra = bx.row[sh.oldp[kx][a].w * kMaxTypes + t];
-                                    const PairRow &rb = bx.row[sh.oldp[ky][a].w * kMaxTypes + t];
-                                    s0.c12 = ra.c12; s0.nc6 = -ra.c6;
-                                    s1.c12 = rb.c12; s1.nc6 = -rb.c6;
-                                }
+                                const LjSource s0 = lj_source(now, on0 ? k0 : k1, a, t, bx);
+                                const LjSource s1 = lj_source(now, on1 ? k1 : k0, a, t, bx);
                                 for (int g0 = 0; g0 < nst; g0 += 32 * 32) {
                                     unsigned n0, n1;
                                     if (!GSLICE) {
@@ -862,9 +1139,9 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 const int e = queue[i], k = e & 0xFF, col = e >> 8;
                 int t = 0;
                 while (sh.wd[t + 1] * 32 <= col) ++t;
-                const int c = col - sh.wd[t] * 32, m = sh.natoms[k], a0 = sh.a0[k];
-                const unsigned rw = sh.rows[k][t], todo = (rw | (rw >> 8)) & 0xFFu;
-                const int4 *np = sh.newp[par][k], *op = sh.oldp[k];
+                const int c = col - sh.wd[t] * 32, m = now.natoms[k], a0 = now.a0[k];
+                const unsigned rw = now.rows[k][t], todo = (rw | (rw >> 8)) & 0xFFu;
+                const int4 *np = now.newp[k], *op = now.oldp[k];
                 float v = 0.f;
                 for (int o = c << cs; o < ((c + 1) << cs); o += 32) {
                     const int s_ = o + lane;
@@ -897,214 +1174,19 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             const int k = warp + q * kMcWarps;
             if (k >= nb) continue;
             const float v = warp_sum(acc[q]);
-            if (lane == 0) sh.part[k] = v;
-        }
-        __syncthreads();
-        // ---- D. gather the partials of the box's CTA group (one bounded grid barrier) -------
-        // Slot buffer, per parity: partials [kBatchMax][grid] (one move's partials of the group
-        // are contiguous), then corrections, the box's pair pq at cta0 * kMcCorrPerCta + pq.
-        // Arrival: warp 0 writes the CTA's partials and corrections in parallel, then lane 0
-        // makes a release add on the group's counter and polls it with acquire loads (the warp
-        // barrier orders the other lanes' writes before the release, which is cumulative; the
-        // CTA barrier after the poll orders every thread's reads after the acquire).
-        ++seq;
-        const int gk = tid >> 3, gsub = tid & 7;     // gather group: move gk, member gsub
-        const bool gin = gk < nb;
-        float cv[8];                                  // corrections (j, gk), j = gsub + 8 i < gk
-        float gv = 0.f, gw = 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) cv[i] = 0.f;
-        if (G > 1) {
-            float *ps = A.slots + (size_t)(seq & 1u) * A.grid * kMcSlotStride;
-            float *cs = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
-            if (warp == 0) {
-                const bool arrive = cta != A.skip_arrival_cta;
-                if (arrive) {
-                    for (int k = lane; k < nb; k += 32) ps[(size_t)k * A.grid + cta] = sh.part[k];
-                    for (int u = lane; u < n_local; u += 32) cs[rank + u * G] = corr_sum(corr_part, u, mm, fine);
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    if (arrive) red_add_release_gpu(&A.flags[box], 1u);
-                    const unsigned target = seq * (unsigned)G;
-                    const uint64_t t_start = globaltimer_ns();
-                    long long it = 0;
-                    bool timed_out = false;
-                    while (ld_acquire_gpu(&A.flags[box]) < target) {
-                        if ((++it & 255) == 0 &&
-                            ((globaltimer_ns() - t_start > A.timeout_ns) || it > A.max_spin ||
-                             ld_relaxed_gpu(A.status) != 0)) {
-                            timed_out = true;
-                            break;
-                        }
-                    }
-                    if (timed_out) {
-                        atomicOr(A.status, kStatusTimeout);
-                        sh.abort_flag = 1;
-                    }
-                }
-            }
-            __syncthreads();
-            if (sh.abort_flag) return;
-            // 8 threads per move k: every 8th CTA's partial and every 8th correction (j, k),
-            // j < k, all loads in flight at once (one L2 round trip)
-            if (gin) {
-                const float *pk = ps + (size_t)gk * A.grid + bx.cta0;
-                const float *ck = cs + gk * (gk - 1) / 2;
-                float pv[kGatherLoads];
-#pragma unroll
-                for (int i = 0; i < kGatherLoads; ++i) {
-                    const int r = gsub + 8 * i;
-                    pv[i] = r < G ? __ldcg(&pk[r]) : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int j = gsub + 8 * i;
-                    cv[i] = j < gk ? __ldcg(&ck[j]) : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < kGatherLoads; ++i) gv += pv[i];
-                for (int r = gsub + 8 * kGatherLoads; r < G; r += 8) gv += __ldcg(&pk[r]);
-            }
-        } else if (gin) {
-            gv = gsub == 0 ? sh.part[gk] : 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int j = gsub + 8 * i;
-                cv[i] = j < gk ? corr_sum(corr_part, gk * (gk - 1) / 2 + j, mm, fine) : 0.f;
-            }
-        }
-        // the group's sums in a fixed shuffle tree (the same order in every run): the move's
-        // partial dU and the magnitude sum of its corrections
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int j = gsub + 8 * i;
-            if (gin && j < gk) corr[j][gk] = cv[i];
-            gw += fabsf(cv[i]);
-        }
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) {
-            gv += __shfl_xor_sync(0xffffffffu, gv, o);
-            gw += __shfl_xor_sync(0xffffffffu, gw, o);
-        }
-        // ---- F. Metropolis decisions of the batch, in order: move k's dU includes the
-        // corrections of every earlier accepted move. Fast path: when no move's decision can
-        // change with any subset of its earlier corrections (|dU - threshold| beyond the sum of
-        // their magnitudes plus the FP32 rounding of that many additions), every group decides
-        // its move at once and then adds its accepted corrections (fixed tree order); otherwise
-        // warp 0 decides one move after the other (lane l holds moves l and l + 32) and adds
-        // the corrections in the chain's order. Both give the same decisions.
-        {
-            const float d = gin ? gv + sh.intra[gk] : 0.f;
-            const float thr = gin ? sh.thr[gk] : 0.f;
-            const float wv = gw + (fabsf(d) + gw) * 0x1p-16f;
-            const bool sure = !gin || metropolis(d + wv, thr) || !metropolis(d - wv, thr);
-            if (gin && gsub == 0) sh.base[gk] = gv;
-            if (__syncthreads_and(sure)) {
-                const bool acc = gin && metropolis(d, thr);
-                if (gin && gsub == 0) sh.acc[par][gk] = acc;
-                __syncthreads();
-                float c = 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int j = gsub + 8 * i;
-                    if (j < gk && sh.acc[par][j]) c += cv[i];
-                }
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                if (gin && gsub == 0) sh.dU[gk] = d + c;
-            } else if (warp == 0) {
-                const bool in0 = lane < nb, in1 = lane + 32 < nb;
-                float d0 = in0 ? sh.base[lane] + sh.intra[lane] : 0.f;
-                float d1 = in1 ? sh.base[lane + 32] + sh.intra[lane + 32] : 0.f;
-                const float thr0 = in0 ? sh.thr[lane] : 0.f, thr1 = in1 ? sh.thr[lane + 32] : 0.f;
-                int acc0 = 0, acc1 = 0;
-#pragma unroll 8
-                for (int j = 0; j < 32; ++j) {
-                    if (j < nb) {
-                        const float c0 = corr[j][lane], c1 = corr[j][lane + 32];
-                        const int aj = __shfl_sync(0xffffffffu, metropolis(d0, thr0), j);
-                        if (lane == j) acc0 = aj;
-                        if (aj) {
-                            if (lane > j) d0 += c0;
-                            d1 += c1;
-                        }
-                    }
-                }
-#pragma unroll 8
-                for (int j = 32; j < kBatchMax; ++j) {
-                    if (j < nb) {
-                        const float c1 = corr[j][lane + 32];
-                        const int aj = __shfl_sync(0xffffffffu, metropolis(d1, thr1), j - 32);
-                        if (lane == j - 32) acc1 = aj;
-                        if (aj && lane + 32 > j) d1 += c1;
-                    }
-                }
-                if (in0) {
-                    sh.dU[lane] = d0;
-                    sh.acc[par][lane] = acc0;
-                }
-                if (in1) {
-                    sh.dU[lane + 32] = d1;
-                    sh.acc[par][lane + 32] = acc1;
-                }
-            }
-        }
-        __syncthreads();
-        if (rank == 0 && warp == 0) {
-            // counts now; the FP64 sum of accepted dU once per staged block of moves
-            const bool in0 = lane < nb, in1 = lane + 32 < nb;
-            const bool acc0 = in0 && sh.acc[par][lane], acc1 = in1 && sh.acc[par][lane + 32];
-            const float d0 = in0 ? sh.dU[lane] : 0.f, d1 = in1 ? sh.dU[lane + 32] : 0.f;
-            const unsigned b_acc = __ballot_sync(0xffffffffu, acc0), b_acc1 = __ballot_sync(0xffffffffu, acc1);
-            const unsigned b_nf = __ballot_sync(0xffffffffu, in0 && !isfinite(d0)),
-                           b_nf1 = __ballot_sync(0xffffffffu, in1 && !isfinite(d1));
-            if (in0) sh.acc_du[t0 - mv_base + lane] = acc0 ? d0 : 0.f;
-            if (in1) sh.acc_du[t0 - mv_base + lane + 32] = acc1 ? d1 : 0.f;
             if (lane == 0) {
-                sh.st_att += nb;
-                sh.st_acc += __popc(b_acc) + __popc(b_acc1);
-                sh.st_nonfinite += __popc(b_nf) + __popc(b_nf1);
+                if (G == 1) sh.part[k] = v;
+                else if (arrive) ps[(size_t)k * A.grid + cta] = v;
             }
         }
-        // ---- G. apply accepted moves: shared slice, global coordinates, log ------------------
-        for (int it = tid; it < nb * kMaxMolAtoms; it += kMcThreads) {
-            const int k = it / kMaxMolAtoms, a = it % kMaxMolAtoms;
-            if (!sh.acc[par][k] || a >= sh.natoms[k]) continue;
-            const int ja = sh.a0[k] + a;
-            const int4 p = sh.newp[par][k][a];
-            const int t = p.w, sp = sh.spos[k][a] - bx.type_start[t], ch = (sp >> cs) - sh.first[t];
-            if (ch >= 0 && ch % G == 0) {
-                const int lc = ch / G, col = sh.wd[t] * 32 + lc, slot = sh.blk[t] + (lc << cs) + (sp & ((1 << cs) - 1));
-                slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
-                // the chunk's box grows to hold the new position
-                atomicMax(&cb[3 * cols + col], mi_abs(p.x - cb[col], L));
-                atomicMax(&cb[4 * cols + col], mi_abs(p.y - cb[cols + col], L));
-                atomicMax(&cb[5 * cols + col], mi_abs(p.z - cb[2 * cols + col], L));
-                if (!GSLICE)
-                    sx[slot] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
-                                          scale32(p.z, L, bx.sc_rcp), (unsigned)ja);
-            }
-            if (rank == 0) A.coords[bx.atom0 + ja] = p;
-        }
-        if (rank == 0 && A.log && tid < nb) {
-            epsr_move_log *lg = A.log + (size_t)box * A.log_stride + (size_t)(A.log_off + t0 + tid);
-            lg->mol = sh.mol[par][tid];
-            lg->accepted = sh.acc[par][tid];
-            lg->dU = sh.dU[tid];
-            lg->n_atoms = sh.natoms[tid];
-            lg->u_acc = sh.u_acc[tid];
-            for (int a = 0; a < kMaxMolAtoms; ++a) {
-                const int4 p = a < sh.natoms[tid] ? sh.newp[par][tid][a] : make_int4(0, 0, 0, 0);
-                lg->trial[a][0] = p.x; lg->trial[a][1] = p.y; lg->trial[a][2] = p.z;
-            }
-        }
-        if (tid == 0) sh.nb_min = 1 << 30;      // every thread read it before phase B
+        // Arrival: the CTA barrier and the release (cumulative) put every thread's writes before the
+        // group's counter. Slot buffer, per parity: partials [kBatchMax][grid] (one move's partials of
+        // the group are contiguous), then corrections, the box's pair pq at cta0 * kMcCorrPerCta + pq.
+        cp_async_wait();
         __syncthreads();
-        t0 += nb;
+        if (arrive && tid == 0) red_add_release_gpu(&A.flags[box], 1u);
     }
-
-    if (rank == 0 && warp == 0) block_sum_du(sh.acc_du, (int)(A.n_moves - mv_base), lane, sh.st_sum);
+    if (rank == 0 && warp == 0) block_sum_du(sh.acc_du, n_du, lane, sh.st_sum);
     if (rank == 0 && tid == 0) {
         epsr_mc_stats *st = A.stats + box;
         st->attempted += sh.st_att;
