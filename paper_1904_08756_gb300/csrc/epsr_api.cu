@@ -278,7 +278,7 @@ static void fill_boxdev(const epsr_box_desc &d, const int *type, BoxDev &b)
     b.sc_rcp = UINT64_MAX / (uint64_t)d.L_fx;
     const double unit = (double)d.L_fx * 0x1p-32;                  // grid units per 2^32-grid unit
     b.sc_s2 = (float)(unit * unit * std::ldexp(1.0, -2 * d.scale_log2));
-    b.sc_k2 = (float)(1.0 / (unit * unit));
+    b.sc_k = (float)(1.0 / unit);
     b.inv_dr_fx = (float)((double)d.bin_q / ((double)d.bin_p * S));
     for (long long i = 0; i < d.n_atoms; ++i) b.count[type[i]]++;
     const double ke = coulomb_k();
@@ -481,6 +481,9 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         }
         BoxDev &bx = h->hb[b];
         fill_boxdev(d, ty, bx);
+        int64_t widest = 1;
+        for (long long m = 0; m < d.n_mol; ++m) widest = std::max(widest, ms[m + 1] - ms[m]);
+        bx.lanes_log = widest <= 4 ? 2 : 3;
         bx.atom0 = atom0;
         bx.mol0 = mol0;
         bx.hist_off = hist0;

@@ -67,7 +67,8 @@ struct BoxDev {
     int32_t gc0;          // first key of this box in the cell-list sort
     uint64_t sc_rcp;      // floor((2^64 - 1) / L): grid coordinate -> 2^32-periodic coordinate
     float sc_s2;          // A^2 per squared unit of the 2^32-periodic grid, (L / 2^32)^2 inv_s2
-    float sc_k2;          // squared units of the 2^32-periodic grid per grid unit^2, (2^32 / L)^2
+    float sc_k;           // units of the 2^32-periodic grid per grid unit, 2^32 / L
+    int32_t lanes_log;    // log2 of the lanes per move of the sweep's trial coordinates (2 or 3)
     int32_t type_start[kMaxTypes];  // first type-major sorted position of each type (box-local)
     int64_t count[kMaxTypes];   // atoms per type
     PairRow row[kMaxTypes * kMaxTypes];

@@ -123,7 +123,7 @@ struct McBatch {
     int natoms[kBatchMax];
     int a0[kBatchMax];
     int spos[kBatchMax][kMaxMolAtoms];   // type-major sorted position of each moved atom
-    float hw2[kBatchMax];                // square of the near radius around old atom 0 (grid units)
+    float hw2[kBatchMax];                // square of the near radius around old atom 0 (2^32-periodic grid)
     // per move and partner type: bit a of the low (high) byte set when moved atom a has a
     // Lennard-Jones (near-only) row with the type
     unsigned short rows[kBatchMax][kMaxTypes];
@@ -256,6 +256,14 @@ __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b)
     return d;
 }
 
+// floor(x 2^32 / L) or one less, for 0 <= x < L, from rcp = floor((2^64 - 1) / L): the coordinate
+// on the 2^32-periodic grid, where a 32-bit difference wraps to the minimum image. The sweep uses
+// it for far pairs and for chunk boxes only, so one unit (2^-32 of the box side) does not matter.
+__device__ __forceinline__ unsigned scale32_near(int x, uint64_t rcp)
+{
+    return (unsigned)x * (unsigned)(rcp >> 32) + __umulhi((unsigned)x, (unsigned)rcp);
+}
+
 // Lennard-Jones change u(r') - u(r) of two far partners p and q (one f32x2 lane pair) on the
 // 2^32-periodic grid, against a moved atom's new and old position there: a 32-bit difference
 // wraps to the minimum image, so a separation component costs one subtraction and one
@@ -292,8 +300,8 @@ __device__ __forceinline__ LjSource lj_source(const McBatch &b, int k, int a, in
         s.ox = b.sco[k][a][0]; s.oy = b.sco[k][a][1]; s.oz = b.sco[k][a][2];
     } else {
         const int4 n = b.newp[k][a], o = b.oldp[k][a];
-        s.nx = scale32(n.x, bx.L, bx.sc_rcp); s.ny = scale32(n.y, bx.L, bx.sc_rcp); s.nz = scale32(n.z, bx.L, bx.sc_rcp);
-        s.ox = scale32(o.x, bx.L, bx.sc_rcp); s.oy = scale32(o.y, bx.L, bx.sc_rcp); s.oz = scale32(o.z, bx.L, bx.sc_rcp);
+        s.nx = scale32_near(n.x, bx.sc_rcp); s.ny = scale32_near(n.y, bx.sc_rcp); s.nz = scale32_near(n.z, bx.sc_rcp);
+        s.ox = scale32_near(o.x, bx.sc_rcp); s.oy = scale32_near(o.y, bx.sc_rcp); s.oz = scale32_near(o.z, bx.sc_rcp);
     }
     const PairRow &r = bx.row[b.oldp[k][a].w * kMaxTypes + t];
     s.c12 = r.c12;
@@ -403,15 +411,15 @@ __device__ __forceinline__ float near_du(const int4 *np, const int4 *op, int m, 
 }
 
 // Trial coordinates and what follows from them alone, for the moves of batch b (from move record
-// tn on): four moves of the warp at once, one per 8-lane group, one lane per atom of the molecule
-// (all three axes in the lane). oldp holds the current coordinates.
+// tn on): thread t takes atom t mod 2^lanes_log of move t >> lanes_log, all three axes; 2^lanes_log
+// (4 or 8) holds the box's largest molecule, so that half the warps do this where they can. oldp
+// holds the current coordinates.
 template <bool CUT>
 __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long long tn, int nb, const BoxDev &bx)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int L = bx.L, nt = bx.n_types;
-    const int k = warp + (lane >> 3) * kMcWarps;
-    const int kk = lane & 7;
+    const int L = bx.L, nt = bx.n_types, lg = bx.lanes_log;
+    const int k = threadIdx.x >> lg;
+    const int kk = threadIdx.x & ((1 << lg) - 1);
     const bool act = k < nb;
     const MoveRec &mr = ring[(tn + (act ? k : 0)) & (kMoveRing - 1)];
     const int a0 = mr.a0, m = act ? mr.m : 0;
@@ -456,12 +464,12 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         np4 = make_int4(nx, ny, nz, op4.w);
         b.newp[k][kk] = np4;
         if (kk < 3) {
-            b.scn[k][kk][0] = scale32(nx, L, bx.sc_rcp);
-            b.scn[k][kk][1] = scale32(ny, L, bx.sc_rcp);
-            b.scn[k][kk][2] = scale32(nz, L, bx.sc_rcp);
-            b.sco[k][kk][0] = scale32(op4.x, L, bx.sc_rcp);
-            b.sco[k][kk][1] = scale32(op4.y, L, bx.sc_rcp);
-            b.sco[k][kk][2] = scale32(op4.z, L, bx.sc_rcp);
+            b.scn[k][kk][0] = scale32_near(nx, bx.sc_rcp);
+            b.scn[k][kk][1] = scale32_near(ny, bx.sc_rcp);
+            b.scn[k][kk][2] = scale32_near(nz, bx.sc_rcp);
+            b.sco[k][kk][0] = scale32_near(op4.x, bx.sc_rcp);
+            b.sco[k][kk][1] = scale32_near(op4.y, bx.sc_rcp);
+            b.sco[k][kk][2] = scale32_near(op4.z, bx.sc_rcp);
         }
     }
     __syncwarp();
@@ -496,35 +504,45 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         const int4 o = b.oldp[k][0];
         reach2 = fmaxf(g2_of(sep(op4, o, L)), g2_of(sep(np4, o, L)));
     }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
+    for (int o = (1 << lg) >> 1; o > 0; o >>= 1) reach2 = fmaxf(reach2, __shfl_xor_sync(0xffffffffu, reach2, o));
     if (act && kk == 0) {
-        const float r = ((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f;
+        const float r = (((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f) * bx.sc_k + 8.f;
         b.hw2[k] = r * r;
     }
-    // rows of the moved atoms with partner type kk (an atom that stays where it is has none)
-    if (act) {
+    // rows of the moved atoms with each partner type (an atom that stays where it is has none)
+    for (int t = kk; act && t < nt; t += 1 << lg) {
         unsigned lj = 0u, nr = 0u;
-        for (int a = 0; a < m && kk < nt; ++a) {
+        for (int a = 0; a < m; ++a) {
             const int4 n = b.newp[k][a], o = b.oldp[k][a];
             if (n.x == o.x && n.y == o.y && n.z == o.z) continue;
-            const PairRow &pr = bx.row[n.w * kMaxTypes + kk];
+            const PairRow &pr = bx.row[n.w * kMaxTypes + t];
             if (lj_full_row<CUT>(pr, bx)) lj |= 1u << a;
             else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
         }
-        b.rows[k][kk] = (unsigned short)(lj | (nr << 8));
+        b.rows[k][t] = (unsigned short)(lj | (nr << 8));
     }
     __syncwarp();
 }
 
-// Index in batch b of an accepted move of molecule mol, or -1 (whole warp; the molecules of a
-// batch are distinct).
-__device__ __forceinline__ int accepted_index(const McBatch &b, int mol, int lane)
+// Half width (2^32-periodic grid, rounded up) that reaches a point at wrapped difference d.
+__device__ __forceinline__ int grow_half(unsigned d)
 {
-    const bool hit0 = lane < b.nb && b.acc[lane] && b.mol[lane] == mol;
-    const bool hit1 = lane + 32 < b.nb && b.acc[lane + 32] && b.mol[lane + 32] == mol;
-    const unsigned h0 = __ballot_sync(0xffffffffu, hit0), h1 = __ballot_sync(0xffffffffu, hit1);
-    return h1 ? 63 - __clz(h1) : h0 ? 31 - __clz(h0) : -1;
+    return (int)min((unsigned)abs((int)d) + 8u, 0x7fffffffu);
+}
+
+// Index in batch b of an accepted move of molecule mol, or -1, by groups of 8 lanes with one
+// molecule each (the molecules of a batch are distinct).
+__device__ __forceinline__ int accepted_index(const McBatch &b, int mol, int sub)
+{
+    int idx = -1;
+#pragma unroll
+    for (int i = 0; i < kBatchMax / 8; ++i) {
+        const int j = sub + 8 * i;
+        if (j < b.nb && b.mol[j] == mol && b.acc[j]) idx = j;
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) idx = max(idx, __shfl_xor_sync(0xffffffffu, idx, o));
+    return idx;
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
@@ -609,8 +627,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             c.w = c.w | (atom << 3);
             slice[sh.blk[t] + i] = c;
             if (!GSLICE)
-                sx[sh.blk[t] + i] = make_uint4(scale32(c.x, L, bx.sc_rcp), scale32(c.y, L, bx.sc_rcp),
-                                               scale32(c.z, L, bx.sc_rcp), (unsigned)atom);
+                sx[sh.blk[t] + i] = make_uint4(scale32_near(c.x, bx.sc_rcp), scale32_near(c.y, bx.sc_rcp),
+                                               scale32_near(c.z, bx.sc_rcp), (unsigned)atom);
         }
     for (int k = tid; k <= bx.n_bins; k += kMcThreads) T[k] = A.thresholds[bx.tbl_off + k];
     if (bx.has_ep)
@@ -631,9 +649,11 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             for (int a = 0; a < 3; ++a) {
                 const int l = __reduce_min_sync(0xffffffffu, lo[a]), u = __reduce_max_sync(0xffffffffu, hi[a]);
                 if (lane == 0) {
+                    // centre and half width on the 2^32-periodic grid, rounded up
                     const int col = sh.wd[t] * 32 + c, ce = l + ((u - l) >> 1);
-                    cb[a * cols + col] = ce;
-                    cb[(3 + a) * cols + col] = u - ce;
+                    const unsigned h = scale32_near(u - ce, bx.sc_rcp);
+                    cb[a * cols + col] = (int)scale32_near(ce, bx.sc_rcp);
+                    cb[(3 + a) * cols + col] = (int)min(h + 8u, 0x7fffffffu);
                 }
             }
         }
@@ -648,9 +668,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     constexpr int kRecI4 = (int)(sizeof(MoveRec) / sizeof(int4));
     // copies the records of moves [m0, m1) into the ring (asynchronously, 16 bytes a thread)
     auto copy_records = [&](long long m0, long long m1) {
-        for (int i = tid; i < (int)(m1 - m0) * kRecI4; i += kMcThreads) {
-            const long long t = m0 + i / kRecI4;
-            cp_async16(reinterpret_cast<int4 *>(&sh.ring[t & (kMoveRing - 1)]) + i % kRecI4, moves + t * kRecI4 + i % kRecI4);
+        const unsigned r0 = (unsigned)m0 & (kMoveRing - 1);
+        for (unsigned i = tid; i < (unsigned)(m1 - m0) * kRecI4; i += kMcThreads) {
+            const unsigned t = i / kRecI4, w = i - t * kRecI4;
+            cp_async16(reinterpret_cast<int4 *>(&sh.ring[(r0 + t) & (kMoveRing - 1)]) + w, moves + m0 * kRecI4 + i);
         }
     };
     long long held = min(A.n_moves, (long long)kMoveRing);      // records copied so far
@@ -662,6 +683,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     int par = 0, nb = 0;             // the current batch: b[par], moves [t0, t0 + nb)
     int n_du = 0;                    // entries of acc_du (rank 0)
     const int gk = tid >> 3, gsub = tid & 7;   // gather group: move gk, member gsub
+    const bool prep_warp = (warp * 32 >> bx.lanes_log) < kBatchMax;      // has moves in trial_moves
     int n_local = 0, mm = 0;         // this CTA's share of the current batch's corrections
     bool fine = false;
     long long t0 = 0;
@@ -684,52 +706,35 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 for (int j = gsub; j < gk; j += 8) dup |= sh.ring[(tn + j) & (kMoveRing - 1)].mol == mol;
                 if (dup) atomicMin(&sh.nb_min, gk);
             }
-            int4 gc[kPerWarp];
-            int gp[kPerWarp];
-#pragma unroll
-            for (int h = 0; h < kPerWarp; ++h) {
-                const int k = warp + h * kMcWarps;
-                gc[h] = make_int4(0, 0, 0, 0);
-                gp[h] = 0;
-                if (k < kmax) {
-                    const MoveRec &mr = sh.ring[(tn + k) & (kMoveRing - 1)];
-                    if (lane < mr.m) {
-                        gc[h] = __ldcg(&A.coords[bx.atom0 + mr.a0 + lane]);
-                        gp[h] = A.pos_of[bx.atom0 + mr.a0 + lane];
-                    }
+            int4 gc = make_int4(0, 0, 0, 0);
+            int gp = 0, mol = -1;
+            bool mine = gk < kmax;          // thread: atom gsub of move gk
+            if (mine) {
+                const MoveRec &mr = sh.ring[(tn + gk) & (kMoveRing - 1)];
+                mol = mr.mol;
+                mine = gsub < mr.m;
+                if (mine) {
+                    gc = __ldcg(&A.coords[bx.atom0 + mr.a0 + gsub]);
+                    gp = A.pos_of[bx.atom0 + mr.a0 + gsub];
                 }
             }
             const long long want = min(A.n_moves, tn + kMoveRing);
             copy_records(held, want);
             held = want;
-            int mol[kPerWarp];
-#pragma unroll
-            for (int h = 0; h < kPerWarp; ++h) {
-                const int k = warp + h * kMcWarps;
-                mol[h] = -1;
-                if (k < kmax) {
-                    mol[h] = sh.ring[(tn + k) & (kMoveRing - 1)].mol;
-                    const int idx = accepted_index(nxt, mol[h], lane);
-                    if (idx >= 0 && lane < kMaxMolAtoms) gc[h] = nxt.newp[idx][lane];
-                }
-            }
+            const int idx = accepted_index(nxt, mol, gsub);
+            if (idx >= 0 && mine) gc = nxt.newp[idx][gsub];
             __syncthreads();                // the previous batch is no longer needed
             nb_next = min(kmax, sh.nb_min);
             if (tid == 0) nxt.nb = nb_next;
-#pragma unroll
-            for (int h = 0; h < kPerWarp; ++h) {
-                const int k = warp + h * kMcWarps;
-                if (k < nb_next) {
-                    if (lane < sh.ring[(tn + k) & (kMoveRing - 1)].m) {
-                        nxt.oldp[k][lane] = gc[h];
-                        nxt.spos[k][lane] = gp[h] - (int)bx.atom0;
-                    }
-                    if (lane == 0) nxt.mol[k] = mol[h];
-                }
+            if (mine && gk < nb_next) {
+                nxt.oldp[gk][gsub] = gc;
+                nxt.spos[gk][gsub] = gp - (int)bx.atom0;
+                if (gsub == 0) nxt.mol[gk] = mol;
             }
-            __syncwarp();
-            trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
+            __syncthreads();
+            if (prep_warp) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
         }
+        bool again = false;
         if (nb > 0) {
             // ---- D. gather the partials of the box's CTA group (one bounded grid barrier) -------
             // Lane 0 of warp 0 polls the group's counter with acquire loads; the CTA barrier after it
@@ -900,12 +905,12 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                     const int lc = ch / G, col = sh.wd[t] * 32 + lc, slot = sh.blk[t] + (lc << cs) + (sp & ((1 << cs) - 1));
                     slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
                     // the chunk's box grows to hold the new position
-                    atomicMax(&cb[3 * cols + col], mi_abs(p.x - cb[col], L));
-                    atomicMax(&cb[4 * cols + col], mi_abs(p.y - cb[cols + col], L));
-                    atomicMax(&cb[5 * cols + col], mi_abs(p.z - cb[2 * cols + col], L));
-                    if (!GSLICE)
-                        sx[slot] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
-                                              scale32(p.z, L, bx.sc_rcp), (unsigned)ja);
+                    const unsigned X = scale32_near(p.x, bx.sc_rcp), Y = scale32_near(p.y, bx.sc_rcp),
+                                   Z = scale32_near(p.z, bx.sc_rcp);
+                    atomicMax(&cb[3 * cols + col], grow_half(X - (unsigned)cb[col]));
+                    atomicMax(&cb[4 * cols + col], grow_half(Y - (unsigned)cb[cols + col]));
+                    atomicMax(&cb[5 * cols + col], grow_half(Z - (unsigned)cb[2 * cols + col]));
+                    if (!GSLICE) sx[slot] = make_uint4(X, Y, Z, (unsigned)ja);
                 }
                 if (rank == 0) A.coords[bx.atom0 + ja] = p;
             }
@@ -923,25 +928,19 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             }
             // ---- the moves of the next batch whose molecules the current one has moved --------------
             if (nb_next > 0) {
-                bool again = false;
-#pragma unroll
-                for (int h = 0; h < kPerWarp; ++h) {
-                    const int k = warp + h * kMcWarps;
-                    if (k >= nb_next) continue;
-                    const int idx = accepted_index(cur, nxt.mol[k], lane);
-                    if (idx < 0) continue;
-                    again = true;
-                    if (lane < cur.natoms[idx]) nxt.oldp[k][lane] = cur.newp[idx][lane];
-                }
-                __syncwarp();
-                if (again) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
+                const int idx = accepted_index(cur, gk < nb_next ? nxt.mol[gk] : -1, gsub);
+                again = idx >= 0;
+                if (again && gsub < cur.natoms[idx]) nxt.oldp[gk][gsub] = cur.newp[idx][gsub];
             }
         }
         if (nb_next == 0) break;
         par ^= 1;
         t0 = tn;
         nb = nb_next;
-        __syncthreads();
+        if (__syncthreads_or(again)) {
+            if (prep_warp) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
+            __syncthreads();
+        }
         McBatch &now = sh.b[par];
         if (tid == 0) {
             sh.nb_min = 1 << 30;
@@ -1000,14 +999,16 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         const int n_words = sh.wd[nt];
         const unsigned ltm = (1u << lane) - 1u;
         {
-            int4 o0[kPerWarp];
+            unsigned ox[kPerWarp], oy[kPerWarp], oz[kPerWarp];
             float hw2[kPerWarp];
             int cnt[kPerWarp];
 #pragma unroll
             for (int q = 0; q < kPerWarp; ++q) {
                 const int k = min(warp + q * kMcWarps, nb - 1);
-                o0[q] = now.oldp[k][0];
-                hw2[q] = A.near_all ? 3e38f : now.hw2[k];
+                ox[q] = now.sco[k][0][0];
+                oy[q] = now.sco[k][0][1];
+                oz[q] = now.sco[k][0][2];
+                hw2[q] = warp + q * kMcWarps >= nb ? -1.f : A.near_all ? 3e38f : now.hw2[k];
                 cnt[q] = 0;
             }
             for (int t = 0; t < nt; ++t) {
@@ -1019,10 +1020,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
 #pragma unroll
                     for (int q = 0; q < kPerWarp; ++q) {
                         const int k = warp + q * kMcWarps;
-                        const float x = (float)max(0, mi_abs(o0[q].x - cx, L) - hx);
-                        const float y = (float)max(0, mi_abs(o0[q].y - cy, L) - hy);
-                        const float z = (float)max(0, mi_abs(o0[q].z - cz, L) - hz);
-                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && k < nb && now.rows[k][t] != 0;
+                        const float x = (float)max(0, abs((int)(ox[q] - (unsigned)cx)) - hx);
+                        const float y = (float)max(0, abs((int)(oy[q] - (unsigned)cy)) - hy);
+                        const float z = (float)max(0, abs((int)(oz[q] - (unsigned)cz)) - hz);
+                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && now.rows[min(k, nb - 1)][t] != 0;
                         const unsigned mk = __ballot_sync(0xffffffffu, hit);
                         if (lane == 0 && k < nb) near[k * A.words_cap + w] = mk;
                         cnt[q] += __popc(mk);
@@ -1093,8 +1094,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                             __syncthreads();
                             for (int i = tid; i < nst; i += kMcThreads) {
                                 const int4 p = __ldcg(&slice[sh.blk[t] + c0 + i]);
-                                sx[i] = make_uint4(scale32(p.x, L, bx.sc_rcp), scale32(p.y, L, bx.sc_rcp),
-                                                   scale32(p.z, L, bx.sc_rcp), 0u);
+                                sx[i] = make_uint4(scale32_near(p.x, bx.sc_rcp), scale32_near(p.y, bx.sc_rcp),
+                                                   scale32_near(p.z, bx.sc_rcp), 0u);
                             }
                             __syncthreads();
                         }
@@ -1170,11 +1171,16 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             }
         }
 #pragma unroll
-        for (int q = 0; q < kPerWarp; ++q) {
-            const int k = warp + q * kMcWarps;
-            if (k >= nb) continue;
-            const float v = warp_sum(acc[q]);
-            if (lane == 0) {
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < kPerWarp; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+        // lane q writes the sum of the warp's move q
+        {
+            float v = acc[0];
+#pragma unroll
+            for (int q = 1; q < kPerWarp; ++q) v = lane == q ? acc[q] : v;
+            const int k = warp + lane * kMcWarps;
+            if (lane < kPerWarp && k < nb) {
                 if (G == 1) sh.part[k] = v;
                 else if (arrive) ps[(size_t)k * A.grid + cta] = v;
             }
