@@ -210,9 +210,8 @@ int epsr_mc_sweep_async(epsr_box *box, int64_t n_moves, uint64_t seed, uint64_t 
 int epsr_mc_status(epsr_box *box, int32_t *status, epsr_stream_t stream);
 /* Reads the running statistics without running moves (synchronises). */
 int epsr_mc_stats_get(epsr_box *box, epsr_mc_stats *stats, epsr_stream_t stream);
-/* Moves per speculative batch (1 .. 64; 0, the default: 64 for boxes swept by at least 64
- * CTAs, 32 for at least 32, else 16; a box swept by fewer than 8 CTAs takes at most 32):
- * the sweep evaluates up to this many
+/* Moves per speculative batch (1 .. 64; 0, the default: 64; a box swept by fewer than 8 CTAs takes
+ * at most 32): the sweep evaluates up to this many
  * consecutive moves with distinct molecules per grid barrier and resolves them in order
  * with exact pairwise corrections, so every value gives the sequential Metropolis chain
  * (up to FP32 rounding of dU). Host only. */
@@ -220,14 +219,13 @@ int epsr_mc_set_batch(epsr_box *box, int32_t batch_k);
 /* CTAs per box of the sweep (0 = automatic). For a batch of boxes, a total budget split
  * in proportion to the atom counts. Host only; takes effect at the next sweep. */
 int epsr_mc_set_ctas(epsr_box *box, int32_t ctas);
-/* Cell queries of the sweep (a performance device, no effect on results): partners whose
- * pair rows have no Lennard-Jones term are looked up in the 8^3 cells of each CTA's slice
- * that meet the cube around the moved molecule widened by margin_fx grid units; a partner
- * that drifts more than margin_fx out of its cell during a launch joins a per-CTA escapee
- * list of escapee_cap entries (-1: the maximum, 256; 0: no cell queries, every partner is
- * scanned) and, when that list is full, the CTA scans every partner for the rest of the
- * launch. Defaults: 2^20 (1 A), -1. EPSR_EINVAL for margin_fx < 0, margin_fx >= L_fx / 4
- * of a box, or escapee_cap outside [-1, 256]. Host only; takes effect at the next sweep. */
+/* Box queries of the sweep (a performance device, no effect on results): a move's pairs with
+ * the partners near it are evaluated for the chunks of 32 partners whose bounding box meets the
+ * range of its Coulomb and empirical-potential terms; the boxes grow with the partners' moves.
+ * escapee_cap 0 switches the queries off (every chunk is near); any other value, and margin_fx,
+ * which an earlier cell-list form needed, are checked and have no effect. Defaults: 2^20, -1.
+ * EPSR_EINVAL for margin_fx < 0, margin_fx >= L_fx / 4 of a box, or escapee_cap outside
+ * [-1, 256]. Host only; takes effect at the next sweep. */
 int epsr_mc_set_cells(epsr_box *box, int32_t margin_fx, int32_t escapee_cap);
 /* Persistent CTAs per SM of the all-pair histogram kernel (1 .. 4; 0 restores the default, 4).
  * A performance setting: the integer counts do not depend on it. Host only. */

@@ -659,11 +659,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         }
     __syncthreads();
 
-    // moves per batch: as set, else 64 for large CTA groups (the per-batch phases amortise
-    // over more moves), 32 for middling and 16 for small ones (corrections grow with the
-    // square of the batch); above 32 only with 8 or more CTAs per box, so that a CTA's share
-    // of the batch-pair corrections fits its item buffer
-    const int batch_k = min(A.batch_k > 0 ? A.batch_k : (G >= 64 ? 64 : G >= 32 ? 32 : 16), G >= 8 ? kBatchMax : 32);
+    // moves per batch: as set, else the most (the per-batch phases amortise over more moves: 0.27
+    // against 0.41 us a move with 32, 99,999-atom water); above 32 only with 8 or more CTAs per box,
+    // so that a CTA's share of the batch-pair corrections fits its item buffer
+    const int batch_k = min(A.batch_k > 0 ? A.batch_k : kBatchMax, G >= 8 ? kBatchMax : 32);
     const int4 *moves = reinterpret_cast<const int4 *>(A.moves + (size_t)box * A.chunk);
     constexpr int kRecI4 = (int)(sizeof(MoveRec) / sizeof(int4));
     // copies the records of moves [m0, m1) into the ring (asynchronously, 16 bytes a thread)
