@@ -146,22 +146,23 @@ __device__ __forceinline__ ICluster load_icluster(const ClArgs &A, int cl, int L
     return I;
 }
 
-// Visits the partners of an i-cluster in later clusters (share `part` of 2^plog): calls
+// Visits the partners of an i-cluster in later clusters, or (ALL) in every other cluster (share
+// `part` of 2^plog): calls
 // scan(list, n) for up to 32 listed partners at a time (n <= 32, the tail of an item may be
 // shorter), every lane taking its own i-atom against each. value(j) gives the list's w.
-template <class Value, class Scan>
+template <bool ALL, class Value, class Scan>
 __device__ __forceinline__ void visit_partners(const ClArgs &A, const ClBox &cb, const ICluster &I, int ci, int part,
                                                int plog, int L, float r2, JList &list, int lane, Value value, Scan scan)
 {
     const unsigned lt = (1u << lane) - 1u;
     int cnt = 0;
-    for (int s0 = ci >> 5; s0 < cb.n_su; s0 += 32) {
+    for (int s0 = ALL ? 0 : ci >> 5; s0 < cb.n_su; s0 += 32) {
         const int s = s0 + lane;
         bool near = s < cb.n_su;
         if (near) near = boxes_near(I.c, I.h, A.su_c[cb.su0 + s], A.su_h[cb.su0 + s], L, r2);
         for (unsigned ms = __ballot_sync(0xffffffffu, near); ms; ms &= ms - 1u) {
             const int jc = ((s0 + __ffs(ms) - 1) << 5) + lane;
-            bool nj = jc > ci && jc < cb.n_cl && (jc & ((1 << plog) - 1)) == part;
+            bool nj = (ALL ? jc != ci : jc > ci) && jc < cb.n_cl && (jc & ((1 << plog) - 1)) == part;
             int first = 0, num = 0;
             if (nj) {
                 const int4 cj = A.cl_c[cb.cl0 + jc], hj = A.cl_h[cb.cl0 + jc];

@@ -158,13 +158,12 @@ struct epsr_box {
     long long ep_cap_Q = 0;
     float *lambda = nullptr;     // adjoint of the smeared normalisation [hist_len]
     unsigned long long *smear_acc = nullptr;   // fixed-point smeared counts [hist_len]
-    // cell-list histogram: keys, items, per-box tile ranges of the all-pairs list (fallback)
-    int total_gcells = 0;
-    std::vector<GcItem> gc_items_h;
-    GcItem *gc_items = nullptr;
-    int *gc_count = nullptr, *gc_offset = nullptr, *gc_block = nullptr;
-    uint4 *gc_scaled = nullptr;
-    int4 *gc_coords = nullptr;
+    // smeared histogram on nodes: moments and derivative table, first node of each box, weights
+    std::vector<long long> node_off_h;
+    long long *node_off = nullptr, *moments = nullptr;
+    float4 *sm_table = nullptr;
+    double *sm_weights = nullptr;
+    long long n_nodes = 0;
     // clusters of 32 atoms in Hilbert order (pair histogram)
     std::vector<ClBox> cl_box_h;
     ClBox *cl_box = nullptr;
@@ -183,7 +182,7 @@ struct epsr_box {
                         sorted_scaled, sorted_coords, moves, mc_sort.count, mc_sort.offset,
                         mc_sort.block, mc_sort.key, mc_sort.rank, mc_sort.index, pos_of,
                         ep_F, ep_Y, ep_C, ep_Q, lambda, smear_acc, slice_g,
-                        gc_items, gc_count, gc_offset, gc_block, gc_scaled, gc_coords,
+                        node_off, moments, sm_table, sm_weights,
                         cl_box, cl_su_box, cl.count, cl.offset, cl.block, cl.coords,
                         cl.cl_c, cl.cl_h, cl.su_c, cl.su_h};
         for (void *p : ptrs)
@@ -529,16 +528,11 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         }
         set_near(bx);
         set_prefilter(bx);
-        // cell-list histogram: cells at least the histogram range plus two grid units wide
-        const long long rcut = (long long)std::ceil(std::sqrt((double)bx.tmax)) + 2 +
-                               (long long)std::ceil(kCellSmearMarginA * std::ldexp(1.0, descs[b].scale_log2));
-        long long side = 1;                       // more cells than atoms gain nothing
-        while (side * side * side < bx.n_atoms) ++side;
-        const long long gn = std::min<long long>(std::min<long long>(bx.L / rcut, side), 512);
-        bx.gc_n = gn >= 3 ? (int)gn : 0;
-        bx.gc0 = h->total_gcells;
-        h->total_gcells += bx.gc_n ? bx.gc_n * bx.gc_n * bx.gc_n : 1;
-        for (int c = 0; c < bx.gc_n * bx.gc_n * bx.gc_n; ++c) h->gc_items_h.push_back(GcItem{b, c});
+        // nodes of the smeared histogram: the most that kSmMaxS per bin, the reach of 5 sigma
+        // (kSmOffsets / 2) and shared memory allow
+        h->node_off_h.push_back(h->n_nodes);
+        h->n_nodes += (long long)bx.n_pairs * std::min<long long>((long long)bx.n_bins * kSmMaxS + kSmOffsets / 2,
+                                                                  kClMaxSmem / 16 / bx.n_pairs + 1);
         // clusters: about 3 A Hilbert cells (a power of two per side, at most one cell per atom)
         ClBox cb;
         memset(&cb, 0, sizeof(cb));
@@ -597,11 +591,9 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         (rc = dalloc(&h->mc_sort.key, atom0)) || (rc = dalloc(&h->mc_sort.rank, atom0)) ||
         (rc = dalloc(&h->mc_sort.index, atom0)) || (rc = dalloc(&h->pos_of, atom0)) ||
         (rc = dalloc(&h->lambda, (size_t)hist0)) || (rc = dalloc(&h->smear_acc, (size_t)hist0)) ||
-        (rc = dalloc(&h->gc_items, std::max<size_t>(1, h->gc_items_h.size()))) ||
-        (rc = dalloc(&h->gc_count, (size_t)h->total_gcells + 1)) ||
-        (rc = dalloc(&h->gc_offset, (size_t)h->total_gcells + 1)) ||
-        (rc = dalloc(&h->gc_block, ((size_t)h->total_gcells + 1 + 1023) / 1024)) ||
-        (rc = dalloc(&h->gc_scaled, atom0)) || (rc = dalloc(&h->gc_coords, atom0)) ||
+        (rc = dalloc(&h->node_off, n_boxes)) || (rc = dalloc(&h->moments, (size_t)4 * h->n_nodes)) ||
+        (rc = dalloc(&h->sm_table, (size_t)h->n_nodes)) ||
+        (rc = dalloc(&h->sm_weights, (size_t)n_boxes * 5 * kSmOffsets)) ||
         (rc = dalloc(&h->cl_box, n_boxes)) || (rc = dalloc(&h->cl_su_box, su_box.size())) ||
         (rc = dalloc(&h->cl.count, (size_t)h->cl.n_keys_pad + n_boxes)) ||
         (rc = dalloc(&h->cl.offset, h->cl.n_keys)) ||
@@ -628,8 +620,7 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
     CKD(cudaMemcpyAsync(h->thresholds, T.data(), T.size() * sizeof(long long), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemsetAsync(h->ep, 0, (size_t)std::max(ep0, 1) * sizeof(float), stream));
     CKD(cudaMemcpyAsync(h->tiles, h->tiles_h.data(), h->tiles_h.size() * sizeof(GrTile), cudaMemcpyHostToDevice, stream));
-    if (!h->gc_items_h.empty())
-        CKD(cudaMemcpyAsync(h->gc_items, h->gc_items_h.data(), h->gc_items_h.size() * sizeof(GcItem), cudaMemcpyHostToDevice, stream));
+    CKD(cudaMemcpyAsync(h->node_off, h->node_off_h.data(), n_boxes * sizeof(long long), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->cl_box, h->cl_box_h.data(), n_boxes * sizeof(ClBox), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->cl_su_box, su_box.data(), su_box.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->hist_box, h->hist_box_h.data(), n_boxes * sizeof(long long), cudaMemcpyHostToDevice, stream));
@@ -1471,77 +1462,65 @@ extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t
 }
 
 // ---- differentiable form: smeared histogram, adjoints, chi^2 ----------------------------------
-// The cell-list form serves when every box has a cell list and 5 sigma fits in the cells'
-// margin; otherwise the all-pairs tiles (any sigma, any box).
-static bool smear_uses_cells(const epsr_box *box, double sigma)
-{
-    if (box->gc_items_h.empty() || 5.0 * sigma > kCellSmearMarginA) return false;
-    for (const auto &b : box->hb)
-        if (b.gc_n == 0) return false;
-    return true;
-}
+// One traversal of the smeared form: on nodes when every box's node grid fits in shared memory,
+// pair by pair otherwise.
+struct SmearPlan {
+    ClArgs c;
+    SmearArgs a;
+    bool table;
+    size_t smem;
+    int grid;
+};
 
-static int smear_common(epsr_box *box, double sigma, cudaStream_t s)
+static int smear_plan(epsr_box *box, double sigma, SmearPlan *p, cudaStream_t s)
 {
     if (!(sigma > 0) || sigma > 2.0) return set_error(EPSR_EINVAL, "smeared g: sigma must be in (0, 2] A");
-    int rc = launch_scale_coords(box->boxes, box->atom_box, box->coords, box->scaled, box->n_atoms, s);
-    if (rc) return rc;
-    if (smear_uses_cells(box, sigma)) {
-        SortScratch sc = box->sort;
-        sc.count = box->gc_count;
-        sc.offset = box->gc_offset;
-        sc.block = box->gc_block;
-        return launch_spatial_sort(box->boxes, box->atom_box, box->scaled, box->coords, box->n_atoms,
-                                   box->total_gcells + 1, 2, sc, box->gc_scaled, box->gc_coords, nullptr, s);
+    memset(&p->a, 0, sizeof(p->a));
+    int np = 1, rows = 1;
+    for (const auto &b : box->hb) {
+        np = std::max(np, b.n_pairs);
+        rows = std::max(rows, b.n_pairs * b.n_bins);
     }
-    return launch_spatial_sort(box->boxes, box->atom_box, box->scaled, box->coords, box->n_atoms,
-                               box->total_cells, 0, box->sort, box->sorted_scaled, box->sorted_coords,
-                               nullptr, s);
-}
-
-static SmearArgs smear_args(epsr_box *box, double sigma)
-{
-    SmearArgs a;
-    memset(&a, 0, sizeof(a));
-    a.boxes = box->boxes;
-    a.index = smear_uses_cells(box, sigma) ? box->sort.index : box->sort.rank;
-    a.sigma = sigma;
-    a.max_pairs_bins = box->ep_cap;
-    if (smear_uses_cells(box, sigma)) {
-        a.coords = box->gc_coords;
-        a.scaled = box->gc_scaled;
-        a.items = box->gc_items;
-        a.n_items = (long long)box->gc_items_h.size();
-        a.cell_start = box->gc_offset;
-        a.cell_count = box->gc_count;
-    } else {
-        a.coords = box->sorted_coords;
-        a.scaled = box->sorted_scaled;
-        a.tiles = box->tiles;
-        a.n_tiles = (long long)box->tiles_h.size();
+    const size_t lists = smear_smem(true, 0);
+    p->a.nodes_cap = (int)(((size_t)kClMaxSmem - lists) / 16 / np);
+    p->table = true;
+    long long most = 0;
+    for (const auto &b : box->hb) {
+        const SmearGrid g = smear_grid(b.n_bins, b.dr_A, sigma, p->a.nodes_cap);
+        p->table = p->table && g.S > 0;
+        if (g.S > 0) most = std::max(most, (long long)b.n_pairs * g.nodes);
     }
-    return a;
-}
-
-static int smear_launch(epsr_box *box, const SmearArgs &a, bool backward, cudaStream_t s)
-{
-    if (a.items) return launch_smear_cells(a, backward, (int)std::min<long long>(a.n_items, (long long)box->sms * 8), s);
-    return launch_smear(a, backward, box->sms * 2, s);
+    p->smem = p->table ? smear_smem(true, most) : smear_smem(false, rows);
+    if (p->smem > (size_t)kClMaxSmem) return set_error(EPSR_EINVAL, "smeared g: n_pairs*n_bins too large");
+    p->grid = box->sms * (p->table ? 1 : 2);
+    p->c = cl_args(box, p->grid * smear_warps_per_cta());
+    p->a.index = box->cl.index;
+    p->a.sigma = sigma;
+    p->a.node_off = box->node_off;
+    p->a.moments = box->moments;
+    p->a.table = box->sm_table;
+    p->a.acc = box->smear_acc;
+    p->a.lambda = box->lambda;
+    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, s);
+    if (!rc && p->table)
+        rc = launch_smear_weights(box->boxes, box->n_boxes, sigma, p->a.nodes_cap, box->sm_weights, s);
+    return rc;
 }
 
 extern "C" int epsr_gr_smeared_fwd(epsr_box *box, double sigma, double *Ht, float *gt, epsr_stream_t stream)
 {
     if (!box || !Ht) return set_error(EPSR_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = smear_common(box, sigma, s);
+    SmearPlan p;
+    int rc = smear_plan(box, sigma, &p, s);
     if (rc) return rc;
-    CK(cudaMemsetAsync(box->smear_acc, 0, (size_t)box->hist_len * sizeof(unsigned long long), s));
-    SmearArgs a = smear_args(box, sigma);
-    a.acc = box->smear_acc;
-    rc = smear_launch(box, a, false, s);
-    if (rc) return rc;
-    return launch_smear_norm(box->boxes, box->n_boxes, box->smear_acc, Ht, gt, box->hist_len,
-                             box->hist_box, s);
+    if (p.table) CK(cudaMemsetAsync(box->moments, 0, (size_t)4 * box->n_nodes * sizeof(long long), s));
+    else CK(cudaMemsetAsync(box->smear_acc, 0, (size_t)box->hist_len * sizeof(unsigned long long), s));
+    if ((rc = launch_smear(p.c, p.a, false, p.table, p.smem, p.grid, s))) return rc;
+    if (p.table)
+        return launch_smear_bins(box->boxes, box->n_boxes, sigma, p.a.nodes_cap, box->node_off, box->moments,
+                                 box->sm_weights, Ht, gt, box->hist_len, box->hist_box, s);
+    return launch_smear_norm(box->boxes, box->n_boxes, box->smear_acc, Ht, gt, box->hist_len, box->hist_box, s);
 }
 
 extern "C" int epsr_gr_smeared_bwd(epsr_box *box, double sigma, const float *dgt, float *grad,
@@ -1549,15 +1528,17 @@ extern "C" int epsr_gr_smeared_bwd(epsr_box *box, double sigma, const float *dgt
 {
     if (!box || !dgt || !grad) return set_error(EPSR_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = smear_common(box, sigma, s);
+    SmearPlan p;
+    int rc = smear_plan(box, sigma, &p, s);
     if (rc) return rc;
     rc = launch_smear_lambda(box->boxes, box->n_boxes, dgt, box->lambda, box->hist_len, box->hist_box, s);
+    if (!rc && p.table)
+        rc = launch_smear_table(box->boxes, box->n_boxes, sigma, p.a.nodes_cap, box->node_off, box->sm_weights,
+                                box->lambda, box->sm_table, s);
     if (rc) return rc;
     CK(cudaMemsetAsync(grad, 0, (size_t)box->n_atoms * 3 * sizeof(float), s));
-    SmearArgs a = smear_args(box, sigma);
-    a.lambda = box->lambda;
-    a.grad = grad;
-    return smear_launch(box, a, true, s);
+    p.a.grad = grad;
+    return launch_smear(p.c, p.a, true, p.table, p.smem, p.grid, s);
 }
 
 extern "C" int epsr_sq_exec_adjoint(epsr_sq_plan *plan, const float *dS_total, int32_t n_cols,

@@ -62,9 +62,6 @@ struct BoxDev {
     int32_t lj_cut;       // 1: Lennard-Jones truncated at d2 < lj2; 0: over every pair
     int64_t lj2;          // (llround(r_lj * S))^2, grid units^2
     float lj2_lo, lj2_hi; // lj2 * (1 -/+ 2^-20)
-    int32_t gc_n;         // cell-list histogram: cells per side (>= 3, each at least the
-                          // histogram range wide), or 0 when the box is too small for it
-    int32_t gc0;          // first key of this box in the cell-list sort
     uint64_t sc_rcp;      // floor((2^64 - 1) / L): grid coordinate -> 2^32-periodic coordinate
     float sc_s2;          // A^2 per squared unit of the 2^32-periodic grid, (L / 2^32)^2 inv_s2
     float sc_k;           // units of the 2^32-periodic grid per grid unit, 2^32 / L

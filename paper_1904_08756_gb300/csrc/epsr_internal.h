@@ -116,13 +116,6 @@ struct GrArgs {
 
 constexpr int kGrTile = 1024;    // atoms per tile (both sides)
 
-// Cell-list histogram: one work item per (box, home cell); pairs of the home cell with itself
-// and with its 13 forward neighbours.
-struct GcItem {
-    int box, cell;
-};
-
-
 // ---- clusters of 32 atoms in Hilbert order (clusters.cuh) ------------------------------------
 struct ClBox {            // one box
     int cl0, n_cl;        // first cluster and number of clusters
@@ -188,27 +181,56 @@ int launch_total_energy(const BoxDev *boxes, const int4 *coords, const int *atom
                         long long n_tiles, double *U, int grid, cudaStream_t stream);
 
 // ---- smeared histogram and adjoint -----------------------------------------------------------
-struct SmearArgs {
-    const BoxDev *boxes;
-    const int4 *coords;        // spatially sorted
-    const uint4 *scaled;       // spatially sorted, 2^32-periodic copy
-    const int *index;          // atom at each sorted position
-    const GrTile *tiles;
-    long long n_tiles;
-    double sigma;
-    unsigned long long *acc;   // forward output: weights * 2^24, accumulated
-    const float *lambda;       // backward input: dL/dHt [hist_len]
-    float *grad;               // backward output [n_atoms_total][3] (accumulated)
-    int max_pairs_bins;
-    // cell-list form (coords, index in cell order): items and cell ranges
-    const GcItem *items;
-    long long n_items;
-    const int *cell_start, *cell_count;
+// Node grid of one box (k_smear.cu): h = dr / S, nodes 0 .. nodes - 1 up to r_max + 5 sigma,
+// bins in reach of a node within `reach` nodes of the bin, n_off = S + 2 reach + 1 offsets.
+struct SmearGrid {
+    double h;
+    int S, nodes, reach, n_off;
 };
-int launch_smear(const SmearArgs &a, bool backward, int grid, cudaStream_t stream);
-int launch_smear_cells(const SmearArgs &a, bool backward, int grid, cudaStream_t stream);
-// cell-list cells are widened by this margin so that smearing with 5 sigma up to it fits
-constexpr double kCellSmearMarginA = 0.5;
+constexpr int kSmOffsets = 2048;      // offsets of the weight table, at most
+constexpr int kSmMaxS = 16;           // nodes per bin, at most
+// h = sigma / 12, or as fine as nodes_cap nodes allow; S = 0 when that leaves it above sigma / 8.
+inline
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+SmearGrid smear_grid(int n_bins, double dr, double sigma, int nodes_cap)
+{
+    SmearGrid g;
+    const double fine = 12.0 * dr / sigma, least = 8.0 * dr / sigma;
+    for (int S = fine < kSmMaxS ? (int)fine + 1 : kSmMaxS;; --S) {
+        g.S = S;
+        if ((double)S < least || S < 1) { g.S = 0; return g; }
+        g.h = dr / (double)S;
+        g.reach = (int)(5.0 * sigma / g.h) + 2;
+        g.nodes = n_bins * S + g.reach;
+        g.n_off = S + 2 * g.reach + 1;
+        if (g.nodes <= nodes_cap) break;
+    }
+    if (g.n_off > kSmOffsets) g.S = 0;
+    return g;
+}
+
+struct SmearArgs {
+    const int *index;          // atom at each position in cluster order
+    double sigma;
+    int nodes_cap;             // nodes per type pair that fit in shared memory
+    const long long *node_off; // [n_boxes] first node of the box in the moments (x 4) and the table
+    long long *moments;        // forward, nodes: [4][n_pairs][nodes] per box, accumulated
+    const float4 *table;       // backward, nodes: [n_pairs][nodes] per box
+    unsigned long long *acc;   // forward, direct: weights * 2^20, accumulated
+    const float *lambda;       // backward, direct: dL/dHt [hist_len]
+    float *grad;               // backward output [n_atoms_total][3] (accumulated)
+};
+size_t smear_smem(bool table, long long rows);
+int smear_warps_per_cta();
+int launch_smear(const ClArgs &c, const SmearArgs &a, bool backward, bool table, size_t smem, int grid, cudaStream_t stream);
+int launch_smear_weights(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, double *W, cudaStream_t stream);
+int launch_smear_bins(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, const long long *node_off,
+                      const long long *moments, const double *W, double *Ht, float *gt, long long hist_len,
+                      const long long *hist_box, cudaStream_t stream);
+int launch_smear_table(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, const long long *node_off,
+                       const double *W, const float *lam, float4 *table, cudaStream_t stream);
 int launch_smear_norm(const BoxDev *boxes, int n_boxes, const unsigned long long *acc, double *Ht,
                       float *gt, long long hist_len, const long long *hist_box, cudaStream_t stream);
 int launch_smear_lambda(const BoxDev *boxes, int n_boxes, const float *dgt, float *lam, long long hist_len,

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
             auto value = [nb](const int4 &q) { return __int_as_float(q.w * nb); };
             if (I.fast) {
                 const uint64_t XI = pk2(I.fx, I.fx), YI = pk2(I.fy, I.fy), ZI = pk2(I.fz, I.fz);
-                visit_partners(A, cb, I, ci, part, A.plog, L, r2, list, lane, value, [&](JList &l, int n) {
+                visit_partners<false>(A, cb, I, ci, part, A.plog, L, r2, list, lane, value, [&](JList &l, int n) {
                     if ((n & 1) && lane == 0) l.put(n, 3e9f, 0.f, 0.f, 0.f, 0);     // pads the last pair: out of every lane's range
                     __syncwarp();
                     const int np = (n + 1) >> 1;
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kClThreads, 4) gr_clusters_kernel(ClArgs A)
                     }
                 });
             } else {
-                visit_partners(A, cb, I, ci, part, A.plog, L, r2, list, lane, value, [&](JList &l, int n) {
+                visit_partners<false>(A, cb, I, ci, part, A.plog, L, r2, list, lane, value, [&](JList &l, int n) {
                     if (I.pos < 0) return;
                     for (int s = 0; s < n; ++s) {
                         const float *pa = reinterpret_cast<const float *>(&l.a[s >> 1]) + (s & 1);

@@ -80,11 +80,7 @@ __global__ void cell_key_kernel(const BoxDev *boxes, const int *atom_box, const 
         const unsigned nc = (unsigned)b.cells;
         const unsigned cx = __umulhi(s.x, nc), cy = __umulhi(s.y, nc), cz = __umulhi(s.z, nc);
         int k;
-        if (type_major == 2) {
-            // cell-list order: cells of at least the histogram range per side, x fastest
-            const unsigned n = (unsigned)(b.gc_n > 0 ? b.gc_n : 1);
-            k = b.gc0 + (int)((__umulhi(s.z, n) * n + __umulhi(s.y, n)) * n + __umulhi(s.x, n));
-        } else if (type_major) {
+        if (type_major) {
             // Monte Carlo partition: type by type, each along the Hilbert curve of its cells
             const unsigned m = 1u << b.mc_bits;
             k = b.mc_cell0 + ((int)s.w << (3 * b.mc_bits)) +
@@ -201,17 +197,6 @@ __global__ void cell_order_kernel(const int *key, const int *count, const int *o
     }
 }
 
-__global__ void gather_sorted_kernel(const int *idx, const uint4 *scaled, const int4 *coords,
-                                     uint4 *s_scaled, int4 *s_coords, long long n)
-{
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int i = idx[p];
-        if (s_scaled) s_scaled[p] = scaled[i];
-        if (s_coords) s_coords[p] = coords[i];
-    }
-}
-
 // One launch up to kScanOneMax counts: its blocks sum the counts before their own from L2,
 // which costs less than two more launches (3.4 against 9.6 us for 32,768 counts) as long as
 // the sums stay short; three launches beyond.
@@ -253,15 +238,8 @@ int launch_spatial_sort(const BoxDev *boxes, const int *atom_box, const uint4 *s
     int rc = launch_scan(sc.count, total_cells, sc.offset, sc.block, stream);
     if (rc) return rc;
     if ((rc = launch_scatter(sc.key, sc.rank, sc.offset, sc.index, n, stream))) return rc;
-    if (type_major == 2) {
-        // the cell-list order only feeds integer counts: the order inside a cell does not
-        // matter there and its cells are large, so the scatter's order is kept and the
-        // coordinates are gathered by position, in parallel
-        gather_sorted_kernel<<<grid, 256, 0, stream>>>(sc.index, scaled, coords, s_scaled, s_coords, n);
-    } else {
-        cell_order_kernel<<<grid, 256, 0, stream>>>(sc.key, sc.count, sc.offset, sc.index, scaled, coords, sc.rank,
-                                                    s_scaled, s_coords, pos_of, n);
-    }
+    cell_order_kernel<<<grid, 256, 0, stream>>>(sc.key, sc.count, sc.offset, sc.index, scaled, coords, sc.rank,
+                                                s_scaled, s_coords, pos_of, n);
     note_launch();
     e = cudaGetLastError();
     return e == cudaSuccess ? EPSR_OK : set_cuda_error(e, "spatial sort");
