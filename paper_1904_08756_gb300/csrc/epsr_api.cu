@@ -153,7 +153,7 @@ struct epsr_box {
     SortScratch mc_sort{};
     int *pos_of = nullptr;
     // empirical-potential update scratch (allocated on first use)
-    double *ep_F = nullptr, *ep_Y = nullptr, *ep_C = nullptr;
+    double *ep_F = nullptr, *ep_Y = nullptr, *ep_C = nullptr, *ep_B = nullptr;   // C: then the table's largest change
     float *ep_Q = nullptr;
     long long ep_cap_Q = 0;
     float *lambda = nullptr;     // adjoint of the smeared normalisation [hist_len]
@@ -181,7 +181,7 @@ struct epsr_box {
                         sort.count, sort.offset, sort.block, sort.key, sort.rank, sort.index,
                         sorted_scaled, sorted_coords, moves, mc_sort.count, mc_sort.offset,
                         mc_sort.block, mc_sort.key, mc_sort.rank, mc_sort.index, pos_of,
-                        ep_F, ep_Y, ep_C, ep_Q, lambda, smear_acc, slice_g,
+                        ep_F, ep_Y, ep_C, ep_B, ep_Q, lambda, smear_acc, slice_g,
                         node_off, moments, sm_table, sm_weights,
                         cl_box, cl_su_box, cl.count, cl.offset, cl.block, cl.coords,
                         cl.cl_c, cl.cl_h, cl.su_c, cl.su_h};
@@ -1399,10 +1399,9 @@ extern "C" int epsr_sq_plan_status(epsr_sq_plan *p, int32_t *status, epsr_stream
 }
 
 // ---- empirical-potential update -------------------------------------------------------------
-extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t n_data,
-                              const double *w, const float *Q, int32_t nQ, int32_t n_basis,
-                              double s_basis, double gamma, double alpha, double *C_out,
-                              epsr_stream_t stream)
+int epsr::ep_update_change(epsr_box *box, int32_t b, const float *dS, int32_t n_data, const double *w, const float *Q,
+                           int32_t nQ, int32_t n_basis, double s_basis, double gamma, double alpha, double *C_out,
+                           double *change, epsr_stream_t stream)
 {
     if (!box || b < 0 || b >= box->n_boxes || !dS || !w || !Q)
         return set_error(EPSR_EINVAL, "ep update: bad argument");
@@ -1417,15 +1416,16 @@ extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t
         if (!(Q[i] > 0) || !std::isfinite(Q[i])) return set_error(EPSR_EINVAL, "ep update: Q[%d] must be > 0", i);
     cudaStream_t s = (cudaStream_t)stream;
     if (box->ep_cap_Q < nQ) {
-        void *ptrs[] = {box->ep_F, box->ep_Y, box->ep_C, box->ep_Q};
+        void *ptrs[] = {box->ep_F, box->ep_Y, box->ep_C, box->ep_B, box->ep_Q};
         for (void *p : ptrs)
             if (p) cudaFree(p);
-        box->ep_F = box->ep_Y = box->ep_C = nullptr;
+        box->ep_F = box->ep_Y = box->ep_C = box->ep_B = nullptr;
         box->ep_Q = nullptr;
         box->ep_cap_Q = 0;
         int rc;
         if ((rc = dalloc(&box->ep_F, (size_t)kEpMaxBasis * nQ)) || (rc = dalloc(&box->ep_Y, (size_t)kEpMaxPairs * nQ)) ||
-            (rc = dalloc(&box->ep_C, (size_t)kEpMaxPairs * kEpMaxBasis)) || (rc = dalloc(&box->ep_Q, (size_t)nQ)))
+            (rc = dalloc(&box->ep_C, (size_t)kEpMaxPairs * kEpMaxBasis + 1)) ||
+            (rc = dalloc(&box->ep_B, (size_t)kEpMaxBasis * EPSR_MAX_BINS)) || (rc = dalloc(&box->ep_Q, (size_t)nQ)))
             return rc;
         box->ep_cap_Q = nQ;
     }
@@ -1447,7 +1447,9 @@ extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t
     a->dr = bx.dr_A;
     a->F = box->ep_F;
     a->Y = box->ep_Y;
+    a->B = box->ep_B;
     a->C_out = box->ep_C;
+    a->change = box->ep_C + kEpMaxPairs * kEpMaxBasis;
     a->ep = box->ep + bx.ep_off;
     cudaError_t e = cudaMemcpyAsync(box->ep_Q, Q, nQ * sizeof(float), cudaMemcpyHostToDevice, s);
     int rc = e == cudaSuccess ? launch_ep_update(*a, s) : set_cuda_error(e, "ep update: Q upload");
@@ -1457,8 +1459,17 @@ extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t
     set_near(bx);
     CK(cudaMemcpyAsync(box->boxes + b, &bx, sizeof(BoxDev), cudaMemcpyHostToDevice, s));
     if (C_out) CK(cudaMemcpyAsync(C_out, box->ep_C, (size_t)P * n_basis * sizeof(double), cudaMemcpyDeviceToHost, s));
+    if (change) CK(cudaMemcpyAsync(change, box->ep_C + kEpMaxPairs * kEpMaxBasis, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return EPSR_OK;
+}
+
+extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t n_data,
+                              const double *w, const float *Q, int32_t nQ, int32_t n_basis,
+                              double s_basis, double gamma, double alpha, double *C_out,
+                              epsr_stream_t stream)
+{
+    return ep_update_change(box, b, dS, n_data, w, Q, nQ, n_basis, s_basis, gamma, alpha, C_out, nullptr, stream);
 }
 
 // ---- differentiable form: smeared histogram, adjoints, chi^2 ----------------------------------

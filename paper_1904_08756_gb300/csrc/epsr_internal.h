@@ -249,10 +249,16 @@ struct EpArgs {
     double s, gamma, alpha, kT, rho, dr;
     double *F;           // [n_basis][nQ] scratch
     double *Y;           // [n_pairs][nQ] scratch
+    double *B;           // [n_basis][n_bins] scratch
     double *C_out;       // [n_pairs][n_basis] device
+    double *change;      // [1] device: largest change of the table (kJ/mol)
     float *ep;           // [n_pairs][n_bins] the box's table, updated in place
 };
 int launch_ep_update(const EpArgs &a, cudaStream_t stream);
+// epsr_ep_update, also returning the largest change it makes to the table (kJ/mol)
+int ep_update_change(epsr_box *box, int32_t b, const float *dS, int32_t n_data, const double *w, const float *Q, int32_t nQ,
+                     int32_t n_basis, double s_basis, double gamma, double alpha, double *C_out, double *change,
+                     epsr_stream_t stream);
 
 struct ChiParams {
     int P, n_basis;

@@ -91,12 +91,6 @@ int dalloc_n(T **p, size_t n)
     return EPSR_OK;
 }
 
-// p_n(r) = (r / (n s))^n exp(n - r / s): the Poisson function with its peak, 1, at r = n s.
-double poisson_p(int n, double s, double r)
-{
-    return r > 0 ? std::exp(n * std::log(r / (n * s)) + n - r / s) : 0.0;
-}
-
 }  // namespace
 
 extern "C" int epsr_refiner_create(epsr_box *box, epsr_sq_plan *plan, const float *target, int32_t n_data,
@@ -193,26 +187,18 @@ extern "C" int epsr_refine_step(epsr_refiner *r, epsr_move_log *log, epsr_refine
     CK(cudaGetLastError());
     // V: fit the Poisson series to Delta S (pair-resolved through the weights) and add it (Eq. 2)
     r->C.assign((size_t)r->P * r->prm.n_basis, 0.0);
-    if ((rc = epsr_ep_update(r->box, 0, r->dS, r->n_data, r->w.data(), r->Q.data(), r->nQ, r->prm.n_basis,
-                             r->prm.s_basis, r->prm.gamma, r->prm.alpha, r->C.data(), stream)))
+    double change = 0.0;
+    if ((rc = ep_update_change(r->box, 0, r->dS, r->n_data, r->w.data(), r->Q.data(), r->nQ, r->prm.n_basis,
+                               r->prm.s_basis, r->prm.gamma, r->prm.alpha, r->C.data(), &change, stream)))
         return rc;
     double chi2 = 0.0;
     CK(cudaMemcpyAsync(&chi2, r->chi2, sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     ++r->iteration;
     if (res) {
-        // the largest change this pass made to the table: alpha kT |sum_n C_pn p_n(r_k)|
-        double dmax = 0.0;
-        for (int p = 0; p < r->P; ++p)
-            for (int k = 0; k < r->n_bins; ++k) {
-                const double rk = (k + 0.5) * r->dr;
-                double v = 0.0;
-                for (int nb = 1; nb <= r->prm.n_basis; ++nb) v += r->C[(size_t)p * r->prm.n_basis + nb - 1] * poisson_p(nb, r->prm.s_basis, rk);
-                dmax = std::max(dmax, std::fabs(r->prm.alpha * r->kT * v));
-            }
         res->iteration = r->iteration;
         res->chi2 = chi2;
-        res->ep_change_max = dmax;
+        res->ep_change_max = change;   // max over the table of alpha kT |sum_n C_pn p_n(r_k)|
         res->attempted = st.attempted;
         res->accepted = st.accepted;
         res->n_configs = r->n_cfg;
