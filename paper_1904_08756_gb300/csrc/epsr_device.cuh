@@ -369,9 +369,12 @@ struct __align__(16) MoveRec {
     float thr;       // FP32 rounded up from -kT ln u_acc
     double u_acc;
     int a0, m;       // first atom (box-local) and atom count of the molecule
-    int kind;        // 0 translate every atom, 1 rotate (and translate), 2 translate atom `atom`
-    int atom;
+    short kind;      // 0 translate every atom, 1 rotate (and translate), 2 translate atom `atom`
+    short atom;
+    int prev;        // moves since the last move of the same molecule, or kMovePrevNone
 };
+constexpr int kMovePrevWindow = 192;        // moves looked back: two batches and the place in a third
+constexpr int kMovePrevNone = 1 << 30;
 
 // ---- spatial order ----------------------------------------------------------------------------
 // Index of cell (x, y, z), `bits` bits per axis, along the Hilbert curve: the transpose form of

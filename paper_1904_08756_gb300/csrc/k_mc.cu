@@ -47,17 +47,36 @@ static_assert(kPerWarp == 4 && kBatchMax == 64, "phase A / F: two moves per lane
 static_assert(kMaxMolAtoms <= 8, "phase B: one lane per atom in 8-lane groups");
 
 // ---- 1. configuration-independent part of each move ----------------------------------------
-__global__ void mc_moves_kernel(const BoxDev *boxes, const int *mol_start, int n_boxes,
-                                long long chunk, long long n, unsigned long long seed,
-                                unsigned long long move0, MoveRec *out)
+// A block takes 128 consecutive moves of one box; the molecules of the 192 moves before them are
+// drawn again, so that every move knows how long ago its molecule was last moved (the batches of
+// the sweep and the coordinates in flight between them follow from that without any search).
+constexpr int kMovesThreads = 128;
+
+__global__ void __launch_bounds__(kMovesThreads) mc_moves_kernel(const BoxDev *boxes, const int *mol_start, int n_boxes,
+                                                                 long long chunk, long long n, unsigned long long seed,
+                                                                 unsigned long long move0, MoveRec *out)
 {
-    const long long total = (long long)n_boxes * chunk;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / chunk);
-        const long long t = e % chunk;
-        if (t >= n) continue;
+    __shared__ int s_mol[kMovePrevWindow + kMovesThreads];
+    const long long per_box = (n + kMovesThreads - 1) / kMovesThreads;
+    for (long long blk = blockIdx.x; blk < per_box * n_boxes; blk += gridDim.x) {
+        const int b = (int)(blk / per_box);
+        const long long t = (blk % per_box) * kMovesThreads + threadIdx.x;
         const BoxDev &bx = boxes[b];
+        __syncthreads();
+        for (int i = threadIdx.x; i < kMovePrevWindow + kMovesThreads; i += kMovesThreads) {
+            const long long ti = t - threadIdx.x - kMovePrevWindow + i;
+            int mol = -1;
+            if (ti >= 0 && ti < n) {
+                const unsigned long long mi = move0 + (unsigned long long)ti;
+                const U32x4 r = philox4x32_10((uint32_t)mi, (uint32_t)(mi >> 32), (uint32_t)b, 0u, (uint32_t)seed,
+                                              (uint32_t)(seed >> 32));
+                mol = (int)(((unsigned long long)r.v[0] * (unsigned long long)bx.n_mol) >> 32);
+            }
+            s_mol[i] = mol;
+        }
+        __syncthreads();
+        if (t >= n) continue;
+        const long long e = b * chunk + t;
         const unsigned long long mv = move0 + (unsigned long long)t;
         const bool flex = bx.move_kind == EPSR_MOVE_FLEXIBLE_MOLECULE;
         uint32_t w[16];
@@ -70,7 +89,10 @@ __global__ void mc_moves_kernel(const BoxDev *boxes, const int *mol_start, int n
             for (int i = 0; i < 4; ++i) w[4 * lane + i] = r.v[i];
         }
         MoveRec m;
-        m.mol = (int)(((unsigned long long)w[0] * (unsigned long long)bx.n_mol) >> 32);
+        m.mol = s_mol[kMovePrevWindow + threadIdx.x];
+        m.prev = kMovePrevNone;
+        for (int d = kMovePrevWindow; d > 0; --d)
+            if (s_mol[kMovePrevWindow + threadIdx.x - d] == m.mol) m.prev = d;
         m.a0 = mol_start[bx.mol0 + m.mol];
         m.m = mol_start[bx.mol0 + m.mol + 1] - m.a0;
         const unsigned span = 2u * (unsigned)bx.max_shift + 1u;
@@ -78,8 +100,8 @@ __global__ void mc_moves_kernel(const BoxDev *boxes, const int *mol_start, int n
         // kind: 0 translate every atom, 1 rotate about the centre (then translate, for rigid
         // molecules), 2 translate one atom; flexible molecules draw the kind from w12 and the
         // atom from w13, and their rotations are not translated
-        m.kind = flex ? (int)(w[12] % 3u) : (bx.move_kind == EPSR_MOVE_RIGID_MOLECULE ? 1 : 0);
-        m.atom = flex ? (int)(w[13] % (uint32_t)m.m) : 0;
+        m.kind = (short)(flex ? (int)(w[12] % 3u) : (bx.move_kind == EPSR_MOVE_RIGID_MOLECULE ? 1 : 0));
+        m.atom = (short)(flex ? (int)(w[13] % (uint32_t)m.m) : 0);
         if (flex && m.kind == 1) m.shift[0] = m.shift[1] = m.shift[2] = 0;
         if (m.kind == 1) {
             const double vx = __dmul_rn(bx.h_rot, __dsub_rn(__dmul_rn(2.0, uniform53(w[4], w[5])), 1.0));
@@ -102,9 +124,9 @@ int launch_mc_moves(const BoxDev *boxes, const int *mol_start, int n_boxes, long
                     long long n, unsigned long long seed, unsigned long long move0, MoveRec *out,
                     cudaStream_t stream)
 {
-    const long long total = (long long)n_boxes * chunk;
-    const int grid = (int)((total + 127) / 128 < 8192 ? (total + 127) / 128 : 8192);
-    mc_moves_kernel<<<grid, 128, 0, stream>>>(boxes, mol_start, n_boxes, chunk, n, seed, move0, out);
+    const long long blocks = (n + kMovesThreads - 1) / kMovesThreads * n_boxes;
+    const int grid = (int)(blocks < 8192 ? blocks : 8192);
+    mc_moves_kernel<<<grid, kMovesThreads, 0, stream>>>(boxes, mol_start, n_boxes, chunk, n, seed, move0, out);
     note_launch();
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? EPSR_OK : set_cuda_error(e, "mc_moves");
@@ -140,7 +162,7 @@ struct McShared {
     McBatch b[2];
     MoveRec ring[kMoveRing];                 // move t at t mod kMoveRing, copied in ahead of use
     int nb_min;                              // first move of the next batch that repeats a molecule
-    int n_near[kBatchMax];                  // near chunks of each move
+    int n_queue;                             // near items of the batch
     // this CTA's partners: per type t, the chunks first[t], first[t] + G, .. of its sorted order, rl[t]
     // atoms in slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
     int first[kMaxTypes];
@@ -410,6 +432,23 @@ __device__ __forceinline__ float near_du(const int4 *np, const int4 *op, int m, 
     return valid ? acc : 0.f;
 }
 
+// Signed minimum image of a difference of two coordinates, in (-L/2, L/2] (hl = floor(L / 2)).
+__device__ __forceinline__ int mi_signed32(int d, int L, int hl)
+{
+    if (d > hl) return d - L;
+    if (d <= hl - L) return d + L;
+    return d;
+}
+
+// x + e wrapped to [0, L), for x in [0, L).
+__device__ __forceinline__ int wrap_near(int x, int e, int L)
+{
+    if (e >= L || e <= -L) return wrap_coord((long long)x + e, L);
+    const int t = (int)((unsigned)x + (unsigned)e);  // negative, or past 2^31 - 1 as unsigned
+    if (e < 0) return t < 0 ? t + L : t;
+    return (unsigned)t >= (unsigned)L ? (int)((unsigned)t - (unsigned)L) : t;
+}
+
 // Trial coordinates and what follows from them alone, for the moves of batch b (from move record
 // tn on): thread t takes atom t mod 2^lanes_log of move t >> lanes_log, all three axes; 2^lanes_log
 // (4 or 8) holds the box's largest molecule, so that half the warps do this where they can. oldp
@@ -429,37 +468,36 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         op4 = op[kk];
         int nx, ny, nz;
         if (mr.kind == 1) {
-            // minimum-image offsets from atom 0, summed over the molecule, and this atom's own
+            // minimum-image offsets from atom 0 (below 2^25), summed over the molecule, and this atom's own
             const int4 b0 = op[0];
-            long long sx = 0, sy = 0, sz = 0, ox = 0, oy = 0, oz = 0;
+            const int hl = L >> 1;
+            int sx = 0, sy = 0, sz = 0, ox = 0, oy = 0, oz = 0;
             for (int i = 0; i < m; ++i) {
                 const int4 c = op[i];
-                const long long dx = mi_signed((long long)c.x - b0.x, L);
-                const long long dy = mi_signed((long long)c.y - b0.y, L);
-                const long long dz = mi_signed((long long)c.z - b0.z, L);
+                const int dx = mi_signed32(c.x - b0.x, L, hl), dy = mi_signed32(c.y - b0.y, L, hl),
+                          dz = mi_signed32(c.z - b0.z, L, hl);
                 sx += dx; sy += dy; sz += dz;
                 if (i == kk) { ox = dx; oy = dy; oz = dz; }
             }
-            const long long ux = (long long)m * ox - sx, uy = (long long)m * oy - sy,
-                            uz = (long long)m * oz - sz;
+            const int ux = m * ox - sx, uy = m * oy - sy, uz = m * oz - sz;
             const int *R = mr.R;
             // per axis: s 2^30 + R (m o - s), then floor((. + m 2^29) / 2^30) (32 bits) and
             // floor division by m
-            const long long numx = sx * 1073741824LL + (long long)R[0] * ux + (long long)R[1] * uy +
+            const long long numx = (long long)sx * 1073741824LL + (long long)R[0] * ux + (long long)R[1] * uy +
                                    (long long)R[2] * uz;
-            const long long numy = sy * 1073741824LL + (long long)R[3] * ux + (long long)R[4] * uy +
+            const long long numy = (long long)sy * 1073741824LL + (long long)R[3] * ux + (long long)R[4] * uy +
                                    (long long)R[5] * uz;
-            const long long numz = sz * 1073741824LL + (long long)R[6] * ux + (long long)R[7] * uy +
+            const long long numz = (long long)sz * 1073741824LL + (long long)R[6] * ux + (long long)R[7] * uy +
                                    (long long)R[8] * uz;
             const long long half = (long long)m * 536870912LL;
-            nx = wrap_coord((long long)b0.x + floordiv32((int)((numx + half) >> 30), m) + mr.shift[0], L);
-            ny = wrap_coord((long long)b0.y + floordiv32((int)((numy + half) >> 30), m) + mr.shift[1], L);
-            nz = wrap_coord((long long)b0.z + floordiv32((int)((numz + half) >> 30), m) + mr.shift[2], L);
+            nx = wrap_near(b0.x, floordiv32((int)((numx + half) >> 30), m) + mr.shift[0], L);
+            ny = wrap_near(b0.y, floordiv32((int)((numy + half) >> 30), m) + mr.shift[1], L);
+            nz = wrap_near(b0.z, floordiv32((int)((numz + half) >> 30), m) + mr.shift[2], L);
         } else {
             const bool moved = mr.kind != 2 || kk == mr.atom;
-            nx = wrap_coord((long long)op4.x + (moved ? mr.shift[0] : 0), L);
-            ny = wrap_coord((long long)op4.y + (moved ? mr.shift[1] : 0), L);
-            nz = wrap_coord((long long)op4.z + (moved ? mr.shift[2] : 0), L);
+            nx = wrap_near(op4.x, moved ? mr.shift[0] : 0, L);
+            ny = wrap_near(op4.y, moved ? mr.shift[1] : 0, L);
+            nz = wrap_near(op4.z, moved ? mr.shift[2] : 0, L);
         }
         np4 = make_int4(nx, ny, nz, op4.w);
         b.newp[k][kk] = np4;
@@ -530,21 +568,6 @@ __device__ __forceinline__ int grow_half(unsigned d)
     return (int)min((unsigned)abs((int)d) + 8u, 0x7fffffffu);
 }
 
-// Index in batch b of an accepted move of molecule mol, or -1, by groups of 8 lanes with one
-// molecule each (the molecules of a batch are distinct).
-__device__ __forceinline__ int accepted_index(const McBatch &b, int mol, int sub)
-{
-    int idx = -1;
-#pragma unroll
-    for (int i = 0; i < kBatchMax / 8; ++i) {
-        const int j = sub + 8 * i;
-        if (j < b.nb && b.mol[j] == mol && b.acc[j]) idx = j;
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) idx = max(idx, __shfl_xor_sync(0xffffffffu, idx, o));
-    return idx;
-}
-
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
@@ -568,6 +591,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         sh.b[0].nb = sh.b[1].nb = 0;
         sh.b[0].mm = sh.b[1].mm = 0;
         sh.nb_min = 1 << 30;
+        sh.n_queue = 0;
         sh.abort_flag = 0;
         sh.st_att = sh.st_acc = sh.st_nonfinite = 0;
         sh.st_sum = 0.0;
@@ -690,6 +714,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         McBatch &cur = sh.b[par], &nxt = sh.b[par ^ 1];
         const long long tn = t0 + nb;
         int nb_next = 0;
+        int last = -1;                      // index in the current batch of the molecule of next move gk, or < 0
         // ---- A, B. the next batch, while the partials of the current one reach the other CTAs --------
         // Its molecules and end, the current coordinates of its molecules and the trial coordinates
         // (integer arithmetic). The decisions of the current batch are not known yet: the few
@@ -699,29 +724,30 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // moves is dropped later.
         if (tn < A.n_moves) {
             const int kmax = (int)min((long long)batch_k, A.n_moves - tn);
-            if (gk < kmax) {                // the batch ends before the first repeated molecule
-                const int mol = sh.ring[(tn + gk) & (kMoveRing - 1)].mol;
-                bool dup = false;
-                for (int j = gsub; j < gk; j += 8) dup |= sh.ring[(tn + j) & (kMoveRing - 1)].mol == mol;
-                if (dup) atomicMin(&sh.nb_min, gk);
-            }
             int4 gc = make_int4(0, 0, 0, 0);
             int gp = 0, mol = -1;
             bool mine = gk < kmax;          // thread: atom gsub of move gk
+            last = -1;
             if (mine) {
                 const MoveRec &mr = sh.ring[(tn + gk) & (kMoveRing - 1)];
                 mol = mr.mol;
                 mine = gsub < mr.m;
+                if (gsub == 0 && mr.prev <= gk) atomicMin(&sh.nb_min, gk);   // the batch ends before a repeated molecule
+                // where the molecule was last moved: in the current batch (taken as not accepted for
+                // now), in the previous one, or before (then the global coordinates are up to date)
+                last = nb + gk - mr.prev;                                    // index in the current batch
+                const int before = last + nxt.nb;                           // index in the previous batch
                 if (mine) {
-                    gc = __ldcg(&A.coords[bx.atom0 + mr.a0 + gsub]);
                     gp = A.pos_of[bx.atom0 + mr.a0 + gsub];
+                    if (last >= 0 && last < nb) gc = cur.oldp[last][gsub];
+                    else if (last < 0 && before >= 0) gc = nxt.acc[before] ? nxt.newp[before][gsub] : nxt.oldp[before][gsub];
+                    else gc = __ldcg(&A.coords[bx.atom0 + mr.a0 + gsub]);
                 }
+                if (last >= nb) last = -1;
             }
             const long long want = min(A.n_moves, tn + kMoveRing);
             copy_records(held, want);
             held = want;
-            const int idx = accepted_index(nxt, mol, gsub);
-            if (idx >= 0 && mine) gc = nxt.newp[idx][gsub];
             __syncthreads();                // the previous batch is no longer needed
             nb_next = min(kmax, sh.nb_min);
             if (tid == 0) nxt.nb = nb_next;
@@ -927,9 +953,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             }
             // ---- the moves of the next batch whose molecules the current one has moved --------------
             if (nb_next > 0) {
-                const int idx = accepted_index(cur, gk < nb_next ? nxt.mol[gk] : -1, gsub);
-                again = idx >= 0;
-                if (again && gsub < cur.natoms[idx]) nxt.oldp[gk][gsub] = cur.newp[idx][gsub];
+                again = gk < nb_next && last >= 0 && cur.acc[last];
+                if (again && gsub < cur.natoms[last]) nxt.oldp[gk][gsub] = cur.newp[last][gsub];
             }
         }
         if (nb_next == 0) break;
@@ -997,6 +1022,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // Lennard-Jones terms, scanned by the move's warp without any test per pair.
         const int n_words = sh.wd[nt];
         const unsigned ltm = (1u << lane) - 1u;
+        int n_near[kPerWarp], base[kPerWarp];          // near chunks of the warp's moves, and their first items
         {
             unsigned ox[kPerWarp], oy[kPerWarp], oz[kPerWarp];
             float hw2[kPerWarp];
@@ -1029,50 +1055,34 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                     }
                 }
             }
+            // the warp's moves take consecutive places in the item queue (the order of the warps does not
+            // matter: every move sums its own items in their order)
+            int all = 0;
 #pragma unroll
-            for (int q = 0; q < kPerWarp; ++q)
-                if (lane == 0 && warp + q * kMcWarps < nb) sh.n_near[warp + q * kMcWarps] = cnt[q];
+            for (int q = 0; q < kPerWarp; ++q) {
+                n_near[q] = cnt[q];
+                base[q] = all;
+                all += cnt[q];
+            }
+            int first = 0;
+            if (lane == 0 && all) first = atomicAdd(&sh.n_queue, all);
+            first = __shfl_sync(0xffffffffu, first, 0);
+#pragma unroll
+            for (int q = 0; q < kPerWarp; ++q) base[q] += first;
         }
-        __syncthreads();
-        // the CTA's corrections go out now; the partials of every move from its own warp below
+        __syncwarp();
         ++seq;
         float *ps = A.slots + (size_t)(seq & 1u) * A.grid * kMcSlotStride;
         const bool arrive = G > 1 && cta != A.skip_arrival_cta;
-        if (arrive) {
-            float *pc = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
-            for (int u = kMcThreads - 1 - tid; u < n_local; u += kMcThreads) pc[rank + u * G] = corr_sum(corr_part, u, mm, fine);
-        }
-        // first item of each move (lane l holds moves l and l + 32), and this warp's items of a round
-        int n_all;
-        int base[kPerWarp];
-        {
-            const int c0 = lane < nb ? sh.n_near[lane] : 0, c1 = lane + 32 < nb ? sh.n_near[lane + 32] : 0;
-            int x0 = c0, x1 = c1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
-                if (lane >= o) {
-                    x0 += y0;
-                    x1 += y1;
-                }
-            }
-            const int t0n = __shfl_sync(0xffffffffu, x0, 31);
-            n_all = t0n + __shfl_sync(0xffffffffu, x1, 31);
-#pragma unroll
-            for (int q = 0; q < kPerWarp; ++q) {
-                const int k = warp + q * kMcWarps;
-                const int b0 = __shfl_sync(0xffffffffu, x0 - c0, k & 31), b1 = __shfl_sync(0xffffffffu, x1 - c1, k & 31);
-                base[q] = k < 32 ? b0 : t0n + b1;
-            }
-        }
         float acc[kPerWarp];
 #pragma unroll
         for (int q = 0; q < kPerWarp; ++q) acc[q] = 0.f;
+        int n_all = 0;
         for (int r0 = 0; r0 == 0 || r0 < n_all; r0 += kQueue) {
 #pragma unroll
             for (int q = 0; q < kPerWarp; ++q) {
                 const int k = warp + q * kMcWarps;
-                if (k >= nb || sh.n_near[k] == 0) continue;
+                if (n_near[q] == 0) continue;
                 int at = base[q] - r0;
                 for (int w = 0; w < n_words; ++w) {
                     const unsigned mk = near[k * A.words_cap + w];
@@ -1134,6 +1144,12 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 }
             }
             __syncthreads();
+            n_all = sh.n_queue;
+            if (r0 == 0 && arrive) {
+                // the CTA's corrections go out now; the partials of every move from its own warp below
+                float *pc = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
+                for (int u = kMcThreads - 1 - tid; u < n_local; u += kMcThreads) pc[rank + u * G] = corr_sum(corr_part, u, mm, fine);
+            }
             // near items, one per warp at a time
             for (int i = warp; i < min(kQueue, n_all - r0); i += kMcWarps) {
                 const int e = queue[i], k = e & 0xFF, col = e >> 8;
@@ -1163,7 +1179,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             for (int q = 0; q < kPerWarp; ++q) {
                 const int k = warp + q * kMcWarps;
                 if (k >= nb) continue;
-                for (int i = lane; i < sh.n_near[k]; i += 32) {
+                for (int i = lane; i < n_near[q]; i += 32) {
                     const int at = base[q] + i - r0;
                     if (at >= 0 && at < kQueue) acc[q] += q_res[at];
                 }
@@ -1189,7 +1205,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // the group are contiguous), then corrections, the box's pair pq at cta0 * kMcCorrPerCta + pq.
         cp_async_wait();
         __syncthreads();
-        if (arrive && tid == 0) red_add_release_gpu(&A.flags[box], 1u);
+        if (tid == 0) {
+            sh.n_queue = 0;
+            if (arrive) red_add_release_gpu(&A.flags[box], 1u);
+        }
     }
     if (rank == 0 && warp == 0) block_sum_du(sh.acc_du, n_du, lane, sh.st_sum);
     if (rank == 0 && tid == 0) {
