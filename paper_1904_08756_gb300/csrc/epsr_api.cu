@@ -368,18 +368,18 @@ static int mc_layout(const epsr_box *h, McLayout *L)
         L->slice_cap = 0;
         L->words_cap = 1;
         for (auto &b : h->hb) {
-            int slots = 0, words = 0;
+            // chunk c of a box (all types in turn) goes to CTA c mod G: at most one more per type
+            int chunks = 0;
             for (int t = 0; t < b.n_types; ++t) {
-                const int nch = (int)((b.count[t] + (1 << cs) - 1) >> cs), nc = (nch + b.n_cta - 1) / b.n_cta;
-                slots += nc << cs;
-                words += (nc + 31) / 32;
+                const int nch = (int)((b.count[t] + (1 << cs) - 1) >> cs);
+                chunks += (nch + b.n_cta - 1) / b.n_cta;
             }
-            L->slice_cap = std::max(L->slice_cap, slots);
-            L->words_cap = std::max(L->words_cap, words);
+            L->slice_cap = std::max(L->slice_cap, chunks << cs);
+            L->words_cap = std::max(L->words_cap, (chunks + 31) / 32);
         }
         return (size_t)h->tbl_cap * sizeof(long long) + (size_t)h->ep_cap * sizeof(float) +
                (size_t)kMcBatchMax * kMcBatchMax * sizeof(float) + (size_t)kMcCorrItems * sizeof(float) +
-               (size_t)L->words_cap * (32 * 6 * sizeof(int) + kMcBatchMax * sizeof(unsigned));
+               (size_t)L->words_cap * (32 * (6 * sizeof(int) + 1) + 2 * kMcBatchMax * sizeof(unsigned));
     };
     size_t tables = sizes(5);
     L->smem = ((size_t)L->slice_cap * 2 * sizeof(int4) + tables + 15) & ~(size_t)15;

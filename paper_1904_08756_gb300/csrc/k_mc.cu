@@ -38,11 +38,12 @@ constexpr int kMoveRing = 2 * kBatchMax;        // move records held: a batch an
 constexpr int kCorrItems = kMcCorrItems;       // >= 496 pairs x 8 atoms (coarse items at G = 1)
 constexpr int kStage = kMcStageChunk;          // partners staged at once (slices in global memory)
 constexpr int kQueue = kBatchMax * kBatchMax / 2;   // near items of one round (in the corrections' buffer)
+constexpr int kNoAtom = -1;                    // .w of a slot past the end of its type
 constexpr int kEscMax = 256;                   // largest escapee_cap that epsr_mc_set_cells accepts
 static_assert(kMcCorrPerCta == kBatchMax * (kBatchMax - 1) / 2 && kMcSlotStride == kBatchMax + kMcCorrPerCta,
               "barrier slot layout");
 static_assert(kMcThreads == 8 * kBatchMax, "gather: 8 threads per move");
-constexpr int kGatherLoads = 20;                // partials per gather thread in flight (CTA groups up to 160)
+constexpr int kGatherLoads = 5;                 // gather: 16-byte loads per thread in flight (CTA groups up to 160)
 static_assert(kPerWarp == 4 && kBatchMax == 64, "phase A / F: two moves per lane of warp 0; phase B: the four moves of a warp in 8-lane groups");
 static_assert(kMaxMolAtoms <= 8, "phase B: one lane per atom in 8-lane groups");
 
@@ -149,6 +150,7 @@ struct McBatch {
     // per move and partner type: bit a of the low (high) byte set when moved atom a has a
     // Lennard-Jones (near-only) row with the type
     unsigned short rows[kBatchMax][kMaxTypes];
+    int lj_atoms[kBatchMax];                 // moved atoms with a Lennard-Jones row
     // first three atoms of each move on the 2^32-periodic grid, new and old: [move][atom][axis]
     unsigned scn[kBatchMax][3][3];
     unsigned sco[kBatchMax][3][3];
@@ -163,12 +165,10 @@ struct McShared {
     MoveRec ring[kMoveRing];                 // move t at t mod kMoveRing, copied in ahead of use
     int nb_min;                              // first move of the next batch that repeats a molecule
     int n_queue;                             // near items of the batch
-    // this CTA's partners: per type t, the chunks first[t], first[t] + G, .. of its sorted order, rl[t]
-    // atoms in slice slots [blk[t], blk[t] + rl[t]), chunk masks in words [wd[t], wd[t + 1])
+    // this CTA's partners: per type t, the chunks first[t], first[t] + G, .. of its sorted order, held
+    // as its chunks [cbase[t], cbase[t + 1]); chunk c at slice slots [c 2^cs, (c + 1) 2^cs)
     int first[kMaxTypes];
-    int rl[kMaxTypes];
-    int blk[kMaxTypes + 1];
-    int wd[kMaxTypes + 1];
+    int cbase[kMaxTypes + 1];
     float part[kBatchMax];
     float base[kBatchMax];
     float dU[kBatchMax];
@@ -294,6 +294,7 @@ __device__ __forceinline__ unsigned scale32_near(int x, uint64_t rcp)
 struct LjSource {
     unsigned nx, ny, nz, ox, oy, oz;
     float c12, nc6;
+    int type;
 };
 __device__ __forceinline__ uint64_t far_du2(uint4 p, uint4 q, const LjSource &s, uint64_t S2)
 {
@@ -313,10 +314,11 @@ __device__ __forceinline__ uint64_t far_du2(uint4 p, uint4 q, const LjSource &s,
     return f2_sub(f2_mul(f2_fma(C12, S6N, NC6), S6N), f2_mul(f2_fma(C12, S6O, NC6), S6O));
 }
 
-// Moved atom a of move k against partners of type t.
-__device__ __forceinline__ LjSource lj_source(const McBatch &b, int k, int a, int t, const BoxDev &bx)
+// Moved atom a of move k (the coefficients are set per partner type).
+__device__ __forceinline__ LjSource lj_source(const McBatch &b, int k, int a, const BoxDev &bx)
 {
     LjSource s;
+    s.type = b.oldp[k][a].w;
     if (a < 3) {
         s.nx = b.scn[k][a][0]; s.ny = b.scn[k][a][1]; s.nz = b.scn[k][a][2];
         s.ox = b.sco[k][a][0]; s.oy = b.sco[k][a][1]; s.oz = b.sco[k][a][2];
@@ -325,33 +327,31 @@ __device__ __forceinline__ LjSource lj_source(const McBatch &b, int k, int a, in
         s.nx = scale32_near(n.x, bx.sc_rcp); s.ny = scale32_near(n.y, bx.sc_rcp); s.nz = scale32_near(n.z, bx.sc_rcp);
         s.ox = scale32_near(o.x, bx.sc_rcp); s.oy = scale32_near(o.y, bx.sc_rcp); s.oz = scale32_near(o.z, bx.sc_rcp);
     }
-    const PairRow &r = bx.row[b.oldp[k][a].w * kMaxTypes + t];
-    s.c12 = r.c12;
-    s.nc6 = -r.c6;
+    s.c12 = s.nc6 = 0.f;
     return s;
 }
 
 // Lennard-Jones terms of one moved atom each of two moves (s0, s1) with the groups of 32 slots
-// g0 .. g0 + ng - 1 of a run of n slots (sx: their 2^32-periodic copy, from its slot 0), group
-// g taken by a move unless bit g of its mask (near: left to the items) is set. A lane takes two
-// partners per step and both moves share their loads: four independent packed chains.
-__device__ __forceinline__ void far_groups(float &acc0, float &acc1, const LjSource &s0, const LjSource &s1,
-                                           unsigned near0, unsigned near1, const uint4 *sx, int ng, int n, uint64_t S2,
-                                           int lane)
+// lo .. up - 1 that are in their masks m0, m1 (sx: the 2^32-periodic copy from group 0 on; a group
+// past `up` may be loaded, and is in neither mask). A lane takes one partner each of two groups per step,
+// and both moves share their loads: four independent packed chains.
+__device__ __forceinline__ void far_groups(float &acc0, float &acc1, const LjSource &s0, const LjSource &s1, unsigned m0,
+                                           unsigned m1, int lo, int up, const uint4 *sx, uint64_t S2, int lane)
 {
-    const unsigned both = near0 & near1;
-    for (int g = 0; g < ng; g += 2) {
-        if (((both >> g) & 3u) == 3u) continue;
-        const int j0 = g * 32 + lane, j1 = j0 + 32;
-        const uint4 p = sx[j0], q = sx[g + 1 < ng ? j1 : j0];
+    const uint4 *pp = sx + lo * 32 + lane;
+    m0 >>= lo;
+    m1 >>= lo;
+    for (int n = up - lo; n > 0; n -= 2, pp += 64, m0 >>= 2, m1 >>= 2) {
+        if (!((m0 | m1) & 3u)) continue;
+        const uint4 p = pp[0], q = pp[32];
         float a0, a1, b0, b1;
         f2_unpack(far_du2(p, q, s0, S2), a0, a1);
         f2_unpack(far_du2(p, q, s1, S2), b0, b1);
-        const bool v0 = j0 < n, v1 = j1 < n;             // the second group past ng has v1 false or its bit set
-        if (v0 && !((near0 >> g) & 1u)) acc0 += a0;
-        if (v1 && !((near0 >> (g + 1)) & 1u)) acc0 += a1;
-        if (v0 && !((near1 >> g) & 1u)) acc1 += b0;
-        if (v1 && !((near1 >> (g + 1)) & 1u)) acc1 += b1;
+        const bool vp = p.w != (unsigned)kNoAtom, vq = q.w != (unsigned)kNoAtom;
+        if (vp && (m0 & 1u)) acc0 += a0;
+        if (vq && (m0 & 2u)) acc0 += a1;
+        if (vp && (m1 & 1u)) acc1 += b0;
+        if (vq && (m1 & 2u)) acc1 += b1;
     }
 }
 
@@ -531,6 +531,7 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         b.intra[k] = di;
         atomicMax(&b.mm, m);
         b.natoms[k] = m;
+        b.lj_atoms[k] = 0;
         b.a0[k] = a0;
         b.thr[k] = mr.thr;
         b.u_acc[k] = mr.u_acc;
@@ -547,6 +548,7 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         const float r = (((float)bx.near_fx + sqrtf(reach2)) * 1.0001f + 2.f) * bx.sc_k + 8.f;
         b.hw2[k] = r * r;
     }
+    __syncwarp();                        // lj_atoms is cleared
     // rows of the moved atoms with each partner type (an atom that stays where it is has none)
     for (int t = kk; act && t < nt; t += 1 << lg) {
         unsigned lj = 0u, nr = 0u;
@@ -558,6 +560,7 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
             else if (near_row<CUT>(pr, bx)) nr |= 1u << a;
         }
         b.rows[k][t] = (unsigned short)(lj | (nr << 8));
+        if (lj) atomicOr(&b.lj_atoms[k], (int)lj);
     }
     __syncwarp();
 }
@@ -609,24 +612,20 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     // chunks, instead of all on the one that owns the region (the barrier waits for the busiest).
     const int cs = A.chunk_log;
     if (tid == 0) {
-        int b = 0, w = 0;
+        int c = 0;
         long long f = 0;
         for (int t = 0; t < nt; ++t) {
-            const int n = (int)bx.count[t], nch = (n + (1 << cs) - 1) >> cs;      // chunks of the type
+            const int nch = (int)((bx.count[t] + (1 << cs) - 1) >> cs);            // chunks of the type
             const int first = (int)(((long long)rank - f % G + G) % G);           // this CTA's first chunk
-            const int nc = first < nch ? (nch - first + G - 1) / G : 0;
             sh.first[t] = first;
-            sh.rl[t] = nc == 0 ? 0 : first + (nc - 1) * G == nch - 1 ? ((nc - 1) << cs) + n - ((nch - 1) << cs) : nc << cs;
-            sh.blk[t] = b;
-            sh.wd[t] = w;
-            b += nc << cs;
-            w += (nc + 31) >> 5;
+            sh.cbase[t] = c;
+            c += first < nch ? (nch - first + G - 1) / G : 0;
             f += nch;
         }
-        sh.blk[nt] = b;
-        sh.wd[nt] = w;
+        sh.cbase[nt] = c;
     }
     __syncthreads();
+    const int n_chunks = sh.cbase[nt], n_words = (n_chunks + 31) >> 5;
 
     // shared memory: partner slice {x, y, z, type | atom << 3} and its 2^32-periodic copy {X, Y, Z,
     // atom} (or, with the slice in global memory, a staged part of the copy), thresholds, empirical
@@ -643,44 +642,57 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     const int cols = A.words_cap * 32;
     int *cb = reinterpret_cast<int *>(corr_part + kCorrItems);                         // [6][cols]
     unsigned *near = reinterpret_cast<unsigned *>(cb + 6 * cols);                      // [kBatchMax][words_cap]
-    for (int t = 0; t < nt; ++t)
-        for (int i = tid; i < sh.rl[t]; i += kMcThreads) {
-            const int pos = bx.type_start[t] + ((sh.first[t] + (i >> cs) * G) << cs) + (i & ((1 << cs) - 1));
-            const int atom = A.sorted_index[bx.atom0 + pos] - (int)bx.atom0;
-            int4 c = A.coords[bx.atom0 + atom];
-            c.w = c.w | (atom << 3);
-            slice[sh.blk[t] + i] = c;
-            if (!GSLICE)
-                sx[sh.blk[t] + i] = make_uint4(scale32_near(c.x, bx.sc_rcp), scale32_near(c.y, bx.sc_rcp),
-                                               scale32_near(c.z, bx.sc_rcp), (unsigned)atom);
+    unsigned *far = near + kBatchMax * A.words_cap;                                    // [kBatchMax][words_cap]
+    unsigned char *ct = reinterpret_cast<unsigned char *>(far + kBatchMax * A.words_cap);   // [cols] type of each chunk
+    for (int c = tid; c < cols; c += kMcThreads) {
+        int t = 0;
+        while (t + 1 < nt && c >= sh.cbase[t + 1]) ++t;
+        ct[c] = (unsigned char)t;
+    }
+    __syncthreads();
+    for (int i = tid; i < n_chunks << cs; i += kMcThreads) {
+        const int t = ct[i >> cs];
+        const long long pos = ((long long)(sh.first[t] + ((i >> cs) - sh.cbase[t]) * G) << cs) + (i & ((1 << cs) - 1));
+        if (pos >= bx.count[t]) {                        // the end of a type's last chunk
+            slice[i] = make_int4(0, 0, 0, kNoAtom);
+            if (!GSLICE) sx[i] = make_uint4(0u, 0u, 0u, (unsigned)kNoAtom);
+            continue;
         }
+        const int atom = A.sorted_index[bx.atom0 + bx.type_start[t] + pos] - (int)bx.atom0;
+        int4 c = A.coords[bx.atom0 + atom];
+        c.w = c.w | (atom << 3);
+        slice[i] = c;
+        if (!GSLICE)
+            sx[i] = make_uint4(scale32_near(c.x, bx.sc_rcp), scale32_near(c.y, bx.sc_rcp), scale32_near(c.z, bx.sc_rcp),
+                               (unsigned)atom);
+    }
     for (int k = tid; k <= bx.n_bins; k += kMcThreads) T[k] = A.thresholds[bx.tbl_off + k];
     if (bx.has_ep)
         for (int k = tid; k < bx.n_pairs * bx.n_bins; k += kMcThreads) ep[k] = A.ep[bx.ep_off + k];
     __syncthreads();
     // boxes of the chunks (coordinates in [0, L); a chunk of Hilbert neighbours seldom meets the
     // seam, and its box is then merely wide)
-    for (int t = 0; t < nt; ++t)
-        for (int c = warp; c < ((sh.rl[t] + (1 << cs) - 1) >> cs); c += kMcWarps) {
-            int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-1, -1, -1};
-            for (int i = (c << cs) + lane; i < min(sh.rl[t], (c + 1) << cs); i += 32) {
-                const int4 p = slice[sh.blk[t] + i];
-                lo[0] = min(lo[0], p.x); hi[0] = max(hi[0], p.x);
-                lo[1] = min(lo[1], p.y); hi[1] = max(hi[1], p.y);
-                lo[2] = min(lo[2], p.z); hi[2] = max(hi[2], p.z);
-            }
+    for (int c = warp; c < n_chunks; c += kMcWarps) {
+        int lo[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, hi[3] = {-1, -1, -1};
+        for (int i = (c << cs) + lane; i < (c + 1) << cs; i += 32) {
+            const int4 p = slice[i];
+            if (p.w == kNoAtom) continue;
+            lo[0] = min(lo[0], p.x); hi[0] = max(hi[0], p.x);
+            lo[1] = min(lo[1], p.y); hi[1] = max(hi[1], p.y);
+            lo[2] = min(lo[2], p.z); hi[2] = max(hi[2], p.z);
+        }
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const int l = __reduce_min_sync(0xffffffffu, lo[a]), u = __reduce_max_sync(0xffffffffu, hi[a]);
-                if (lane == 0) {
-                    // centre and half width on the 2^32-periodic grid, rounded up
-                    const int col = sh.wd[t] * 32 + c, ce = l + ((u - l) >> 1);
-                    const unsigned h = scale32_near(u - ce, bx.sc_rcp);
-                    cb[a * cols + col] = (int)scale32_near(ce, bx.sc_rcp);
-                    cb[(3 + a) * cols + col] = (int)min(h + 8u, 0x7fffffffu);
-                }
+        for (int a = 0; a < 3; ++a) {
+            const int l = __reduce_min_sync(0xffffffffu, lo[a]), u = __reduce_max_sync(0xffffffffu, hi[a]);
+            if (lane == 0) {
+                // centre and half width on the 2^32-periodic grid, rounded up
+                const int ce = l + ((u - l) >> 1);
+                const unsigned h = scale32_near(u - ce, bx.sc_rcp);
+                cb[a * cols + c] = (int)scale32_near(ce, bx.sc_rcp);
+                cb[(3 + a) * cols + c] = (int)min(h + 8u, 0x7fffffffu);
             }
         }
+    }
     __syncthreads();
 
     // moves per batch: as set, else the most (the per-batch phases amortise over more moves: 0.27
@@ -710,47 +722,47 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     int n_local = 0, mm = 0;         // this CTA's share of the current batch's corrections
     bool fine = false;
     long long t0 = 0;
+    // Looks up the moves from tn on, the current batch being b[par] (nb moves before tn): thread gsub
+    // of move gk takes atom gsub. Current coordinates come from the current batch's old ones (as if it
+    // were not accepted) or the previous batch's accepted move, b[par ^ 1] (its global update may not be
+    // visible yet), else from the global array, which holds every earlier one. The batch ends before
+    // its first repeated molecule.
+    int4 gc = make_int4(0, 0, 0, 0);
+    int gp = 0, mol = -1, last = -1;     // last: index in the current batch of the molecule, or -1
+    bool mine = false;
+    auto look_up = [&](long long tn) {
+        const McBatch &cur = sh.b[par], &nxt = sh.b[par ^ 1];
+        mine = gk < (int)min((long long)batch_k, A.n_moves - tn);
+        last = -1;
+        if (!mine) return;
+        const MoveRec &mr = sh.ring[(tn + gk) & (kMoveRing - 1)];
+        mol = mr.mol;
+        mine = gsub < mr.m;
+        if (gsub == 0 && mr.prev <= gk) atomicMin(&sh.nb_min, gk);
+        last = nb + gk - mr.prev;
+        const int before = last + nxt.nb;                           // index in the previous batch
+        if (mine) {
+            gp = A.pos_of[bx.atom0 + mr.a0 + gsub];
+            if (last >= 0 && last < nb) gc = cur.oldp[last][gsub];
+            else if (last < 0 && before >= 0) gc = nxt.acc[before] ? nxt.newp[before][gsub] : nxt.oldp[before][gsub];
+            else gc = __ldcg(&A.coords[bx.atom0 + mr.a0 + gsub]);
+        }
+        if (last >= nb) last = -1;
+    };
+    look_up(0);
+    __syncthreads();
     for (;;) {
         McBatch &cur = sh.b[par], &nxt = sh.b[par ^ 1];
         const long long tn = t0 + nb;
         int nb_next = 0;
-        int last = -1;                      // index in the current batch of the molecule of next move gk, or < 0
         // ---- A, B. the next batch, while the partials of the current one reach the other CTAs --------
-        // Its molecules and end, the current coordinates of its molecules and the trial coordinates
-        // (integer arithmetic). The decisions of the current batch are not known yet: the few
-        // molecules that they move are taken up again after them. Coordinates come from the previous
-        // batch's accepted moves (b[par ^ 1], about to be replaced; their global update may not be
-        // visible yet), else from the global array, whose value for a molecule that the current batch
-        // moves is dropped later.
+        // Its current and trial coordinates (integer arithmetic). The decisions of the current batch are
+        // not known yet: the few molecules that they move are taken up again after them.
         if (tn < A.n_moves) {
-            const int kmax = (int)min((long long)batch_k, A.n_moves - tn);
-            int4 gc = make_int4(0, 0, 0, 0);
-            int gp = 0, mol = -1;
-            bool mine = gk < kmax;          // thread: atom gsub of move gk
-            last = -1;
-            if (mine) {
-                const MoveRec &mr = sh.ring[(tn + gk) & (kMoveRing - 1)];
-                mol = mr.mol;
-                mine = gsub < mr.m;
-                if (gsub == 0 && mr.prev <= gk) atomicMin(&sh.nb_min, gk);   // the batch ends before a repeated molecule
-                // where the molecule was last moved: in the current batch (taken as not accepted for
-                // now), in the previous one, or before (then the global coordinates are up to date)
-                last = nb + gk - mr.prev;                                    // index in the current batch
-                const int before = last + nxt.nb;                           // index in the previous batch
-                if (mine) {
-                    gp = A.pos_of[bx.atom0 + mr.a0 + gsub];
-                    if (last >= 0 && last < nb) gc = cur.oldp[last][gsub];
-                    else if (last < 0 && before >= 0) gc = nxt.acc[before] ? nxt.newp[before][gsub] : nxt.oldp[before][gsub];
-                    else gc = __ldcg(&A.coords[bx.atom0 + mr.a0 + gsub]);
-                }
-                if (last >= nb) last = -1;
-            }
-            const long long want = min(A.n_moves, tn + kMoveRing);
-            copy_records(held, want);
-            held = want;
-            __syncthreads();                // the previous batch is no longer needed
-            nb_next = min(kmax, sh.nb_min);
+            nb_next = min((int)min((long long)batch_k, A.n_moves - tn), sh.nb_min);
             if (tid == 0) nxt.nb = nb_next;
+            copy_records(held, min(A.n_moves, tn + kMoveRing));
+            held = min(A.n_moves, tn + kMoveRing);
             if (mine && gk < nb_next) {
                 nxt.oldp[gk][gsub] = gc;
                 nxt.spos[gk][gsub] = gp - (int)bx.atom0;
@@ -800,11 +812,25 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 if (gin) {
                     const float *pk = ps + (size_t)gk * A.grid + bx.cta0;
                     const float *ck = pc + gk * (gk - 1) / 2;
-                    float pv[kGatherLoads];
+                    float4 pv[kGatherLoads];             // four CTAs' partials each, where the rows are aligned
+                    if (((A.grid | bx.cta0) & 3) == 0) {
 #pragma unroll
-                    for (int i = 0; i < kGatherLoads; ++i) {
-                        const int r = gsub + 8 * i;
-                        pv[i] = r < G ? __ldcg(&pk[r]) : 0.f;
+                        for (int i = 0; i < kGatherLoads; ++i) {
+                            const int r = 4 * (gsub + 8 * i);
+                            pv[i] = r < G ? __ldcg(reinterpret_cast<const float4 *>(pk + r)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (r + 1 >= G) pv[i].y = 0.f;
+                            if (r + 2 >= G) pv[i].z = 0.f;
+                            if (r + 3 >= G) pv[i].w = 0.f;
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < kGatherLoads; ++i) {
+                            const int r = gsub + 8 * i;
+                            pv[i].x = r < G ? __ldcg(&pk[r]) : 0.f;
+                            pv[i].y = r + 8 * kGatherLoads < G ? __ldcg(&pk[r + 8 * kGatherLoads]) : 0.f;
+                            pv[i].z = r + 16 * kGatherLoads < G ? __ldcg(&pk[r + 16 * kGatherLoads]) : 0.f;
+                            pv[i].w = r + 24 * kGatherLoads < G ? __ldcg(&pk[r + 24 * kGatherLoads]) : 0.f;
+                        }
                     }
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -812,8 +838,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                         cv[i] = j < gk ? __ldcg(&ck[j]) : 0.f;
                     }
 #pragma unroll
-                    for (int i = 0; i < kGatherLoads; ++i) gv += pv[i];
-                    for (int r = gsub + 8 * kGatherLoads; r < G; r += 8) gv += __ldcg(&pk[r]);
+                    for (int i = 0; i < kGatherLoads; ++i) gv += (pv[i].x + pv[i].y) + (pv[i].z + pv[i].w);
+                    for (int r = gsub + 32 * kGatherLoads; r < G; r += 8) gv += __ldcg(&pk[r]);
                 }
             } else if (gin) {
                 gv = gsub == 0 ? sh.part[gk] : 0.f;
@@ -927,7 +953,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 const int4 p = cur.newp[k][a];
                 const int t = p.w, sp = cur.spos[k][a] - bx.type_start[t], ch = (sp >> cs) - sh.first[t];
                 if (ch >= 0 && ch % G == 0) {
-                    const int lc = ch / G, col = sh.wd[t] * 32 + lc, slot = sh.blk[t] + (lc << cs) + (sp & ((1 << cs) - 1));
+                    const int col = sh.cbase[t] + ch / G, slot = (col << cs) + (sp & ((1 << cs) - 1));
                     slice[slot] = make_int4(p.x, p.y, p.z, t | (ja << 3));
                     // the chunk's box grows to hold the new position
                     const unsigned X = scale32_near(p.x, bx.sc_rcp), Y = scale32_near(p.y, bx.sc_rcp),
@@ -1020,7 +1046,6 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // and the items of the CTA are spread over its warps: in a large box the few moves near this
         // CTA's region would otherwise keep single warps busy. The other chunks have at most
         // Lennard-Jones terms, scanned by the move's warp without any test per pair.
-        const int n_words = sh.wd[nt];
         const unsigned ltm = (1u << lane) - 1u;
         int n_near[kPerWarp], base[kPerWarp];          // near chunks of the warp's moves, and their first items
         {
@@ -1036,23 +1061,25 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 hw2[q] = warp + q * kMcWarps >= nb ? -1.f : A.near_all ? 3e38f : now.hw2[k];
                 cnt[q] = 0;
             }
-            for (int t = 0; t < nt; ++t) {
-                const int nc = (sh.rl[t] + (1 << cs) - 1) >> cs;
-                for (int w = sh.wd[t]; w < sh.wd[t + 1]; ++w) {
-                    const int c = (w - sh.wd[t]) * 32 + lane, col = w * 32 + min(lane, nc - 1 - (w - sh.wd[t]) * 32);
-                    const int cx = cb[col], cy = cb[cols + col], cz = cb[2 * cols + col];
-                    const int hx = cb[3 * cols + col], hy = cb[4 * cols + col], hz = cb[5 * cols + col];
+            for (int w = 0; w < n_words; ++w) {
+                const int c = w * 32 + lane, col = min(c, n_chunks - 1), t = ct[col];
+                const int cx = cb[col], cy = cb[cols + col], cz = cb[2 * cols + col];
+                const int hx = cb[3 * cols + col], hy = cb[4 * cols + col], hz = cb[5 * cols + col];
 #pragma unroll
-                    for (int q = 0; q < kPerWarp; ++q) {
-                        const int k = warp + q * kMcWarps;
-                        const float x = (float)max(0, abs((int)(ox[q] - (unsigned)cx)) - hx);
-                        const float y = (float)max(0, abs((int)(oy[q] - (unsigned)cy)) - hy);
-                        const float z = (float)max(0, abs((int)(oz[q] - (unsigned)cz)) - hz);
-                        const bool hit = c < nc && fmaf(x, x, fmaf(y, y, z * z)) < hw2[q] && now.rows[min(k, nb - 1)][t] != 0;
-                        const unsigned mk = __ballot_sync(0xffffffffu, hit);
-                        if (lane == 0 && k < nb) near[k * A.words_cap + w] = mk;
-                        cnt[q] += __popc(mk);
+                for (int q = 0; q < kPerWarp; ++q) {
+                    const int k = warp + q * kMcWarps;
+                    const float x = (float)max(0, abs((int)(ox[q] - (unsigned)cx)) - hx);
+                    const float y = (float)max(0, abs((int)(oy[q] - (unsigned)cy)) - hy);
+                    const float z = (float)max(0, abs((int)(oz[q] - (unsigned)cz)) - hz);
+                    const unsigned rw = c < n_chunks ? now.rows[min(k, nb - 1)][t] : 0u;
+                    const bool in = fmaf(x, x, fmaf(y, y, z * z)) < hw2[q];
+                    const unsigned mk = __ballot_sync(0xffffffffu, in && rw != 0u);
+                    const unsigned fk = __ballot_sync(0xffffffffu, !in && (rw & 0xFFu));
+                    if (lane == 0 && k < nb) {
+                        near[k * A.words_cap + w] = mk;
+                        far[k * A.words_cap + w] = fk;
                     }
+                    cnt[q] += __popc(mk);
                 }
             }
             // the warp's moves take consecutive places in the item queue (the order of the warps does not
@@ -1094,57 +1121,72 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             if (r0 == 0 && !(CUT && bx.lj_cut)) {
                 // Lennard-Jones terms with the far chunks, atom by atom for two moves at a time
                 const uint64_t S2 = f2_pack(bx.sc_s2, bx.sc_s2);
-                for (int t = 0; t < nt; ++t) {
-                    const int rl = sh.rl[t];
-                    for (int c0 = 0; c0 < rl; c0 += GSLICE ? kStage : rl) {
-                        const int nst = GSLICE ? min(kStage, rl - c0) : rl;
-                        if (GSLICE) {
-                            // stage the copy of the next partners, read once for the whole batch
-                            __syncthreads();
-                            for (int i = tid; i < nst; i += kMcThreads) {
-                                const int4 p = __ldcg(&slice[sh.blk[t] + c0 + i]);
-                                sx[i] = make_uint4(scale32_near(p.x, bx.sc_rcp), scale32_near(p.y, bx.sc_rcp),
-                                                   scale32_near(p.z, bx.sc_rcp), 0u);
-                            }
-                            __syncthreads();
+                const int all_groups = n_chunks << (cs - 5);              // groups of 32 slots
+                for (int g0 = 0; g0 < all_groups; g0 += GSLICE ? kStage / 32 : all_groups) {
+                    if (GSLICE) {
+                        // stage the copy of the next partners, read once for the whole batch
+                        __syncthreads();
+                        for (int i = tid; i < min(kStage, (all_groups - g0) * 32); i += kMcThreads) {
+                            const int4 p = __ldcg(&slice[g0 * 32 + i]);
+                            sx[i] = make_uint4(scale32_near(p.x, bx.sc_rcp), scale32_near(p.y, bx.sc_rcp),
+                                               scale32_near(p.z, bx.sc_rcp), (unsigned)(p.w == kNoAtom ? kNoAtom : 0));
                         }
-                        const uint4 *src = GSLICE ? sx : sx + sh.blk[t];
-#pragma unroll
-                        for (int h = 0; h < kPerWarp; h += 2) {
-                            const int k0 = warp + h * kMcWarps, k1 = k0 + kMcWarps;
-                            if (k0 >= nb) continue;
-                            const bool two = k1 < nb;
-                            const unsigned l0 = now.rows[k0][t] & 0xFFu, l1 = two ? now.rows[k1][t] & 0xFFu : 0u;
-                            for (unsigned todo = l0 | l1; todo; todo &= todo - 1u) {
-                                const int a = __ffs(todo) - 1;
-                                const bool on0 = (l0 >> a) & 1u, on1 = (l1 >> a) & 1u;
-                                const LjSource s0 = lj_source(now, on0 ? k0 : k1, a, t, bx);
-                                const LjSource s1 = lj_source(now, on1 ? k1 : k0, a, t, bx);
-                                for (int g0 = 0; g0 < nst; g0 += 32 * 32) {
-                                    unsigned n0, n1;
-                                    if (!GSLICE) {
-                                        n0 = near[k0 * A.words_cap + sh.wd[t] + (g0 >> 10)];
-                                        n1 = two ? near[k1 * A.words_cap + sh.wd[t] + (g0 >> 10)] : 0u;
-                                    } else {
-                                        // group g of the stage lies in chunk (c0 + g0) / 32 + g, cs - 5 bits coarser
-                                        const int c = (c0 + g0 + 32 * lane) >> cs;
-                                        const int w = min(sh.wd[t] + (c >> 5), n_words - 1);
-                                        n0 = __ballot_sync(0xffffffffu, (near[k0 * A.words_cap + w] >> (c & 31)) & 1u);
-                                        n1 = __ballot_sync(0xffffffffu, two && ((near[k1 * A.words_cap + w] >> (c & 31)) & 1u));
-                                    }
-                                    if (!on0) n0 = 0xFFFFFFFFu;
-                                    if (!on1) n1 = 0xFFFFFFFFu;
-                                    const int left = nst - g0;
-                                    far_groups(acc[h], acc[h + 1], s0, s1, n0, n1, src + g0, min(32, (left + 31) >> 5), left, S2,
-                                               lane);
+                        __syncthreads();
+                    }
+                    const int g1 = GSLICE ? min(all_groups, g0 + kStage / 32) : all_groups;
+#pragma unroll 1
+                    for (int h = 0; h < kPerWarp; h += 2) {               // (one copy of the scan's code)
+                        const int k0 = warp + h * kMcWarps;
+                        if (k0 >= nb) break;
+                        const bool two = k0 + kMcWarps < nb;
+                        const int k1 = two ? k0 + kMcWarps : k0;
+                        const unsigned atoms0 = (unsigned)now.lj_atoms[k0], atoms1 = two ? (unsigned)now.lj_atoms[k1] : 0u;
+                        float f0 = 0.f, f1 = 0.f;
+                        for (unsigned todo = atoms0 | atoms1; todo; todo &= todo - 1u) {
+                            const int a = __ffs(todo) - 1;
+                            LjSource s0 = lj_source(now, (atoms0 >> a) & 1u ? k0 : k1, a, bx);
+                            LjSource s1 = lj_source(now, (atoms1 >> a) & 1u ? k1 : k0, a, bx);
+                            for (int gw = g0; gw < g1; gw += 32) {
+                                // far groups of each move in this word
+                                unsigned m0, m1;
+                                if (!GSLICE) {
+                                    m0 = far[k0 * A.words_cap + (gw >> 5)];
+                                    m1 = two ? far[k1 * A.words_cap + (gw >> 5)] : 0u;
+                                } else {
+                                    const int c = min(gw + lane, g1 - 1) >> (cs - 5);        // chunks of 2^(cs - 5) groups
+                                    const bool in = gw + lane < g1;
+                                    m0 = __ballot_sync(0xffffffffu, in && ((far[k0 * A.words_cap + (c >> 5)] >> (c & 31)) & 1u));
+                                    m1 = __ballot_sync(0xffffffffu, in && two && ((far[k1 * A.words_cap + (c >> 5)] >> (c & 31)) & 1u));
+                                }
+                                for (int t = 0; t < nt; ++t) {
+                                    // groups of type t in this word
+                                    const int lo = max(0, (sh.cbase[t] << (cs - 5)) - gw), up = min(32, (sh.cbase[t + 1] << (cs - 5)) - gw);
+                                    if (lo >= up) continue;
+                                    unsigned tm = (up == 32 ? 0xFFFFFFFFu : (1u << up) - 1u) & ~((1u << lo) - 1u);
+                                    const unsigned t0m = (now.rows[k0][t] >> a) & 1u ? m0 & tm : 0u;
+                                    const unsigned t1m = (now.rows[k1][t] >> a) & 1u ? m1 & tm : 0u;
+                                    if (!(t0m | t1m)) continue;
+                                    const PairRow &ra = bx.row[s0.type * kMaxTypes + t], &rb = bx.row[s1.type * kMaxTypes + t];
+                                    s0.c12 = ra.c12; s0.nc6 = -ra.c6;
+                                    s1.c12 = rb.c12; s1.nc6 = -rb.c6;
+                                    far_groups(f0, f1, s0, s1, t0m, t1m, lo, up, sx + (gw - (GSLICE ? g0 : 0)) * 32, S2, lane);
                                 }
                             }
                         }
+#pragma unroll
+                        for (int u = 0; u < kPerWarp; u += 2)
+                            if (u == h) {
+                                acc[u] += f0;
+                                acc[u + 1] += f1;
+                            }
                     }
                 }
             }
+            if (r0 == 0) cp_async_wait();                // records of the next batch
             __syncthreads();
             n_all = sh.n_queue;
+            // (its loads run while the items do)
+            if (r0 == 0 && t0 + nb < A.n_moves) look_up(t0 + nb);
             if (r0 == 0 && arrive) {
                 // the CTA's corrections go out now; the partials of every move from its own warp below
                 float *pc = ps + (size_t)kBatchMax * A.grid + (size_t)bx.cta0 * kMcCorrPerCta;
@@ -1153,19 +1195,14 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             // near items, one per warp at a time
             for (int i = warp; i < min(kQueue, n_all - r0); i += kMcWarps) {
                 const int e = queue[i], k = e & 0xFF, col = e >> 8;
-                int t = 0;
-                while (sh.wd[t + 1] * 32 <= col) ++t;
-                const int c = col - sh.wd[t] * 32, m = now.natoms[k], a0 = now.a0[k];
+                const int t = ct[col], m = now.natoms[k], a0 = now.a0[k];
                 const unsigned rw = now.rows[k][t], todo = (rw | (rw >> 8)) & 0xFFu;
                 const int4 *np = now.newp[k], *op = now.oldp[k];
                 float v = 0.f;
-                for (int o = c << cs; o < ((c + 1) << cs); o += 32) {
-                    const int s_ = o + lane;
-                    bool valid = s_ < sh.rl[t];
-                    if (!__any_sync(0xffffffffu, valid)) break;
-                    const int4 pj = slice[sh.blk[t] + (valid ? s_ : 0)];
+                for (int o = col << cs; o < ((col + 1) << cs); o += 32) {
+                    const int4 pj = slice[o + lane];
                     const int ja = pj.w >> 3;
-                    valid = valid && !(ja >= a0 && ja < a0 + m);
+                    const bool valid = pj.w != kNoAtom && !(ja >= a0 && ja < a0 + m);
                     v += m == 1 ? near_du<1, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep)
                          : m <= 3 ? near_du<3, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep)
                                   : near_du<0, CUT>(np, op, m, todo, pj, t, valid, bx, T, ep);
@@ -1203,7 +1240,6 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         // Arrival: the CTA barrier and the release (cumulative) put every thread's writes before the
         // group's counter. Slot buffer, per parity: partials [kBatchMax][grid] (one move's partials of
         // the group are contiguous), then corrections, the box's pair pq at cta0 * kMcCorrPerCta + pq.
-        cp_async_wait();
         __syncthreads();
         if (tid == 0) {
             sh.n_queue = 0;
