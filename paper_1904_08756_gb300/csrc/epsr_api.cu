@@ -354,12 +354,17 @@ static void plan_mc_groups(epsr_box *h)
 // Shared-memory layout of the sweep for the current CTA split: thresholds, EP table, correction
 // tables, chunk boxes and near masks, and, when they fit, the partner slice (int4 per slot, and its
 // copy on the 2^32-periodic grid); otherwise the slices live in global memory, a part of the copy is
-// staged, and chunks double until their masks take at most kMcMaxWords words.
+// staged, and chunks double until their masks take at most kMcMaxWords words and everything fits.
+// Large empirical potentials leave the thresholds in global memory and shrink the stage: tables of up
+// to about 110 KB have room beside the least stage and four mask words.
 struct McLayout {
-    int slice_cap = 0, words_cap = 1, chunk_log = 5;
+    int slice_cap = 0, words_cap = 1, chunk_log = 5, stage = kMcStageChunk, tbl_cap = 0;
     size_t smem = 0;
     bool gslice = false;
 };
+
+// per mask word: 32 chunk boxes and types, a near and a far word of every move
+constexpr size_t kMcWordBytes = 32 * (6 * sizeof(int) + 1) + 2 * kMcBatchMax * sizeof(unsigned);
 
 static int mc_layout(const epsr_box *h, McLayout *L)
 {
@@ -377,16 +382,25 @@ static int mc_layout(const epsr_box *h, McLayout *L)
             L->slice_cap = std::max(L->slice_cap, chunks << cs);
             L->words_cap = std::max(L->words_cap, (chunks + 31) / 32);
         }
-        return (size_t)h->tbl_cap * sizeof(long long) + (size_t)h->ep_cap * sizeof(float) +
+        return (size_t)L->tbl_cap * sizeof(long long) + (size_t)h->ep_cap * sizeof(float) +
                (size_t)kMcBatchMax * kMcBatchMax * sizeof(float) + (size_t)kMcCorrItems * sizeof(float) +
-               (size_t)L->words_cap * (32 * (6 * sizeof(int) + 1) + 2 * kMcBatchMax * sizeof(unsigned));
+               (size_t)L->words_cap * kMcWordBytes;
     };
+    L->tbl_cap = h->tbl_cap;
     size_t tables = sizes(5);
     L->smem = ((size_t)L->slice_cap * 2 * sizeof(int4) + tables + 15) & ~(size_t)15;
     L->gslice = L->smem > kMcMaxDynSmem;
     if (L->gslice) {
-        for (int cs = 5; L->words_cap > kMcMaxWords; ) tables = sizes(++cs);
-        L->smem = ((size_t)kMcStageChunk * sizeof(uint4) + tables + 15) & ~(size_t)15;
+        auto total = [&] { return ((size_t)L->stage * sizeof(uint4) + tables + 15) & ~(size_t)15; };
+        // everything but the mask words, with four of them
+        auto too_large = [&] { return total() + 4 * kMcWordBytes > kMcMaxDynSmem + L->words_cap * kMcWordBytes; };
+        if (too_large()) {
+            L->tbl_cap = 0;
+            tables = sizes(5);
+        }
+        if (too_large()) L->stage = kMcStageLeast;
+        while ((L->words_cap > kMcMaxWords || total() > kMcMaxDynSmem) && L->words_cap > 1) tables = sizes(L->chunk_log + 1);
+        L->smem = total();
         if (L->smem > kMcMaxDynSmem)
             return set_error(EPSR_EINVAL, "mc sweep: %zu bytes of tables per CTA (limit %zu)", L->smem, kMcMaxDynSmem);
     }
@@ -937,7 +951,8 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     for (const auto &b : box->hb) a.lj_cut |= b.lj_cut;
     a.batch_k = box->mc_batch;
     a.slice_cap = slice_cap;
-    a.tbl_cap = box->tbl_cap;
+    a.tbl_cap = lay.tbl_cap;
+    a.stage = lay.stage;
     a.ep_cap = box->ep_cap;
     a.slice_g = gslice ? box->slice_g : nullptr;
     a.chunk_log = lay.chunk_log;

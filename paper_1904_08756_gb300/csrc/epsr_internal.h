@@ -45,8 +45,9 @@ constexpr int kMcSlotStride = kMcBatchMax + kMcCorrPerCta;
 // correction items of one batch in shared memory (>= 496 pairs x 8 atoms: batches above 32 moves
 // need 8 or more CTAs per box)
 constexpr int kMcCorrItems = 4096;
-// partners staged at once in shared memory when the slices live in global memory
-constexpr int kMcStageChunk = 2048;
+// partners staged at once in shared memory when the slices live in global memory, and with
+// empirical-potential tables that leave no room for as many
+constexpr int kMcStageChunk = 2048, kMcStageLeast = 512;
 constexpr int kMcMaxWords = 24;           // chunk mask words per CTA of such a slice, at most
 
 struct McArgs {
@@ -76,7 +77,8 @@ struct McArgs {
     int lj_cut;                   // 1: some box truncates Lennard-Jones (the cut instantiation runs)
     int batch_k;
     int slice_cap;                // int4 capacity of the shared partner slice
-    int tbl_cap;                  // capacity (entries) of the shared threshold table
+    int tbl_cap;                  // capacity (entries) of the shared threshold table, 0: read from global memory
+    int stage;                    // partners staged at once (slices in global memory)
     int ep_cap;                   // capacity (entries) of the shared empirical-potential table
     int4 *slice_g;                // [grid][slice_cap] partner slices in global memory, or NULL
     int chunk_log;                // log2 of the slots per chunk (5; more for slices in global memory)

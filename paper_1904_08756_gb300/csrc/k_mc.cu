@@ -36,7 +36,6 @@ constexpr int kBatchMax = kMcBatchMax;         // moves per batch: warp w takes 
 constexpr int kPerWarp = kBatchMax / kMcWarps;  // moves per warp and batch
 constexpr int kMoveRing = 2 * kBatchMax;        // move records held: a batch and the 64 moves after it
 constexpr int kCorrItems = kMcCorrItems;       // >= 496 pairs x 8 atoms (coarse items at G = 1)
-constexpr int kStage = kMcStageChunk;          // partners staged at once (slices in global memory)
 constexpr int kQueue = kBatchMax * kBatchMax / 2;   // near items of one round (in the corrections' buffer)
 constexpr int kNoAtom = -1;                    // .w of a slot past the end of its type
 constexpr int kEscMax = 256;                   // largest escapee_cap that epsr_mc_set_cells accepts
@@ -578,8 +577,10 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // GSLICE: the partner slices live in global memory ([grid][slice_cap], read through L1/L2)
-// because they do not fit in shared memory; the thresholds, EP table and cell index stay
-// in shared memory either way.
+// because they do not fit in shared memory; the EP table and the chunk boxes stay in shared
+// memory either way, and so do the thresholds where there is room (pairs within the FP32 error of a
+// bin edge read them, about one in 10^3: from global memory silica with an empirical potential took
+// 1480 instead of 1452 us).
 template <bool GSLICE, bool CUT>
 __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
 {
@@ -633,8 +634,9 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
     // bit) and near masks
     int4 *slice = GSLICE ? A.slice_g + (size_t)cta * A.slice_cap : reinterpret_cast<int4 *>(dyn);
     uint4 *sx = GSLICE ? reinterpret_cast<uint4 *>(dyn) : reinterpret_cast<uint4 *>(slice + A.slice_cap);
-    long long *T = reinterpret_cast<long long *>(sx + (GSLICE ? kStage : A.slice_cap));
-    float *ep = reinterpret_cast<float *>(T + A.tbl_cap);
+    long long *s_T = reinterpret_cast<long long *>(sx + (GSLICE ? A.stage : A.slice_cap));
+    const long long *T = A.tbl_cap ? s_T : A.thresholds + bx.tbl_off;
+    float *ep = reinterpret_cast<float *>(s_T + A.tbl_cap);
     float (*corr)[kBatchMax] = reinterpret_cast<float (*)[kBatchMax]>(ep + A.ep_cap);
     float *corr_part = &corr[kBatchMax][0];                                              // [kCorrItems]
     int *queue = reinterpret_cast<int *>(&corr[0][0]);                                  // [kQueue], during phase C
@@ -666,7 +668,8 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
             sx[i] = make_uint4(scale32_near(c.x, bx.sc_rcp), scale32_near(c.y, bx.sc_rcp), scale32_near(c.z, bx.sc_rcp),
                                (unsigned)atom);
     }
-    for (int k = tid; k <= bx.n_bins; k += kMcThreads) T[k] = A.thresholds[bx.tbl_off + k];
+    if (A.tbl_cap)
+        for (int k = tid; k <= bx.n_bins; k += kMcThreads) s_T[k] = A.thresholds[bx.tbl_off + k];
     if (bx.has_ep)
         for (int k = tid; k < bx.n_pairs * bx.n_bins; k += kMcThreads) ep[k] = A.ep[bx.ep_off + k];
     __syncthreads();
@@ -1122,18 +1125,18 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 // Lennard-Jones terms with the far chunks, atom by atom for two moves at a time
                 const uint64_t S2 = f2_pack(bx.sc_s2, bx.sc_s2);
                 const int all_groups = n_chunks << (cs - 5);              // groups of 32 slots
-                for (int g0 = 0; g0 < all_groups; g0 += GSLICE ? kStage / 32 : all_groups) {
+                for (int g0 = 0; g0 < all_groups; g0 += GSLICE ? A.stage / 32 : all_groups) {
                     if (GSLICE) {
                         // stage the copy of the next partners, read once for the whole batch
                         __syncthreads();
-                        for (int i = tid; i < min(kStage, (all_groups - g0) * 32); i += kMcThreads) {
+                        for (int i = tid; i < min(A.stage, (all_groups - g0) * 32); i += kMcThreads) {
                             const int4 p = __ldcg(&slice[g0 * 32 + i]);
                             sx[i] = make_uint4(scale32_near(p.x, bx.sc_rcp), scale32_near(p.y, bx.sc_rcp),
                                                scale32_near(p.z, bx.sc_rcp), (unsigned)(p.w == kNoAtom ? kNoAtom : 0));
                         }
                         __syncthreads();
                     }
-                    const int g1 = GSLICE ? min(all_groups, g0 + kStage / 32) : all_groups;
+                    const int g1 = GSLICE ? min(all_groups, g0 + A.stage / 32) : all_groups;
 #pragma unroll 1
                     for (int h = 0; h < kPerWarp; h += 2) {               // (one copy of the scan's code)
                         const int k0 = warp + h * kMcWarps;

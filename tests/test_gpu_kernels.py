@@ -1,0 +1,134 @@
+"""Edges of the GPU kernels' tiles and ranges against the oracle: clusters and super-clusters of the
+pair histograms, chunks, layouts and molecule sizes of the sweep, node grids of the smeared
+histogram, and the two places the fit keeps its columns in.
+
+Bars as in test_gpu_parity: counts and coordinates exact, dU within 1e-5 of its condition scale plus
+1e-4 kJ/mol; those of the smeared form and of the fit are derived where they stand.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1904_08756_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_1904_08756_gb300 import epsr  # noqa: E402
+from test_gpu_parity import DEV, gpu_hist, replay, run_logged  # noqa: E402
+
+
+def mixed_box(sizes, n_mol, n_types, seed, n_bins=200, spacing=4.0, r_lj=0.0):
+    """Rigid molecules of the sizes given in turn, on a jittered cubic lattice; types at random, every
+    other type without a Lennard-Jones term, charges +-0.3 e."""
+    rng = np.random.default_rng(seed)
+    k = int(np.ceil(n_mol ** (1 / 3) - 1e-9))
+    L_fx = int(synth.SCALE * spacing * max(k, 4))
+    at = rng.permutation(k ** 3)[:n_mol]
+    centre = (np.stack([at % k, at // k % k, at // (k * k)], 1) + 0.5) * spacing
+    m = np.array([sizes[i % len(sizes)] for i in range(n_mol)])
+    start = np.concatenate([[0], np.cumsum(m)])
+    off = rng.normal(size=(start[-1], 3))
+    off *= 0.9 / np.linalg.norm(off, axis=1, keepdims=True)
+    off[start[:-1][m == 1]] = 0.0
+    xyz = (np.repeat(centre, m, axis=0) + off + rng.uniform(-0.3, 0.3, (n_mol, 3)).repeat(m, axis=0)) * synth.SCALE
+    return synth.System(name="mixed", L_fx=L_fx, xyz=(np.rint(xyz).astype(np.int64) % L_fx).astype(np.int32),
+                        type=rng.integers(0, n_types, start[-1]).astype(np.int32), mol_start=start.astype(np.int64),
+                        type_names=[f"T{i}" for i in range(n_types)], q=[0.3 - 0.6 * (i % 2) for i in range(n_types)],
+                        sigma=[2.0 + 0.1 * i for i in range(n_types)], eps=[0.4 * (i % 2 == 0) for i in range(n_types)],
+                        b=[5.0] * n_types, r_coul=7.0, bin_p=1, bin_q=25, n_bins=n_bins, rigid_molecules=max(sizes) > 1,
+                        Q=0.5 + np.arange(50) * 0.1, r_lj=r_lj, seed=seed)
+
+
+@pytest.mark.parametrize("n,L,types,bins", [(31, 30.0, 1, 150), (32, 30.0, 2, 150), (33, 30.0, 2, 150),
+                                            (1024, 30.0, 3, 150), (1056, 30.0, 8, 150), (4097, 50.0, 2, 150),
+                                            (4097, 50.0, 1, 800), (300, 2000.0, 2, 4000), (1100, 30.0, 8, 800)])
+def test_cluster_histogram_edges(n, L, types, bins):
+    """Full and partial clusters and super-clusters; ranges below and above half the box; clusters too
+    wide for relative coordinates (a sparse box of 2,000 A); rows that leave no room in shared memory."""
+    s = synth.uniform_gas(n, L, seed=n + types, n_types=types)
+    s.bin_p, s.bin_q, s.n_bins = 1, 25, bins
+    H = gpu_hist(epsr.Box(s)).reshape(-1, bins)
+    assert np.array_equal(H, oracle.Box(s).histogram(threads=8))
+
+
+@pytest.mark.parametrize("sizes,n_mol,types,bins,ctas,r_lj,ep", [
+    ([3], 1, 2, 100, 0, 0.0, False),                       # one molecule: every batch is one move
+    ([1], 33, 1, 100, 0, 0.0, True),                       # two chunks, the second with one atom
+    ([2, 3], 300, 3, 100, 7, 0.0, True),                   # batches of 32, unaligned gather rows
+    (list(range(1, 9)), 300, 8, 100, 0, 0.0, True),        # every molecule size and type
+    (list(range(1, 9)), 300, 5, 100, 9, 6.0, True),        # the same with Lennard-Jones cut
+    ([1, 4], 400, 4, 2000, 0, 0.0, True),                  # 80 KB of tables in shared memory
+    ([1, 2], 4000, 8, 640, 1, 0.0, True),                  # 92 KB of tables, slices in global memory
+], ids=["one", "chunk-end", "groups", "sizes", "sizes-cut", "tables", "tables-global"])
+def test_sweep_edges_replay(sizes, n_mol, types, bins, ctas, r_lj, ep):
+    s = mixed_box(sizes, n_mol, types, seed=n_mol + types, n_bins=bins, r_lj=r_lj)
+    P = types * (types + 1) // 2
+    table = (np.random.default_rng(5).normal(size=(P, bins)) * 0.3).astype(np.float32) if ep else None
+    box = epsr.Box(s)
+    if ep:
+        box.epsr_box_set_ep(0, table)
+    if ctas:
+        box.epsr_mc_set_ctas(ctas)
+    stats, log = run_logged(box, 600, seed=8)
+    ob, _, _, flips = replay(s, s.xyz, log[0], 8, ep=table.astype(np.float64) if ep else None)
+    assert flips <= 2
+    assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
+
+
+@pytest.mark.parametrize("n,L,sigma,bin_q", [(33, 20.0, 0.05, 25), (1057, 22.0, 0.02, 25), (1057, 40.0, 0.3, 5),
+                                             (1057, 40.0, 0.05, 5), (65, 300.0, 0.05, 25)],
+                         ids=["one-atom-cluster", "fine-nodes", "wide", "direct", "sparse"])
+def test_smeared_edges(n, L, sigma, bin_q):
+    """Histogram within 1e-5 of its largest entry (the rounding of the 2^-20 weights and of FP32
+    distances), gradient of a smooth functional within 1e-4 in the 2-norm, as in test_gpu_parity."""
+    s = synth.uniform_gas(n, L, seed=n, n_types=2)
+    s.bin_p, s.bin_q, s.n_bins = 1, bin_q, 8 * bin_q
+    box, ob = epsr.Box(s), oracle.Box(s)
+    Ht = torch.zeros(box.hist_len, dtype=torch.float64, device=DEV)
+    box.epsr_gr_smeared_fwd(sigma, Ht)
+    ref = ob.smeared_hist(sigma)
+    assert np.abs(Ht.cpu().numpy().reshape(ref.shape) - ref).max() <= 1e-5 * np.abs(ref).max()
+    lam = np.cos(np.arange(3 * s.n_bins).reshape(3, -1) * s.dr * 2.0)
+    _, factor = oracle.smeared_g(ob, ref)                              # g = Ht factor
+    grad = torch.zeros((n, 3), dtype=torch.float32, device=DEV)
+    box.epsr_gr_smeared_bwd(sigma, torch.from_numpy((lam / factor).astype(np.float32).reshape(-1)).to(DEV), grad)
+    gref = ob.smeared_grad(sigma, lam)
+    assert np.linalg.norm(grad.cpu().numpy() - gref) <= 1e-4 * np.linalg.norm(gref)
+
+
+def test_smeared_moments_do_not_wrap():
+    """40,000 atoms on two points: all 4e8 pairs that are apart fall on one node, hundreds of times what
+    a 32-bit moment holds. The offset from the node is rounded to 2^-13 (4e-7 A) and the distance of 2 A to 2e-7 A for
+    every pair alike; the steepest weight changes by 2.9 per A and the largest is 0.24: 8e-6 of it."""
+    n = 40000
+    s = synth.uniform_gas(n, 30.0, seed=1, n_types=1)
+    s.bin_p, s.bin_q, s.n_bins = 3, 100, 100
+    s.xyz[:] = int(5 * synth.SCALE)
+    s.xyz[n // 2:, 0] += int(2 * synth.SCALE) + 12345
+    box = epsr.Box(s)
+    Ht = torch.zeros(box.hist_len, dtype=torch.float64, device=DEV)
+    box.epsr_gr_smeared_fwd(0.05, Ht)
+    two = synth.System(**{**s.__dict__, "xyz": s.xyz[[0, n - 1]].copy(), "type": s.type[:2], "mol_start": s.mol_start[:3]})
+    ref = oracle.Box(two).smeared_hist(0.05)[0] * (n // 2) ** 2
+    assert np.abs(Ht.cpu().numpy() - ref).max() <= 2e-5 * ref.max()
+
+
+@pytest.mark.parametrize("nQ,n_basis", [(6, 6), (13, 5), (999, 24), (20000, 20)],
+                         ids=["square", "few-rows", "uneven-rows", "columns-in-global-memory"])
+def test_ep_fit_edges(nQ, n_basis):
+    """The fitted Delta S within 1e-8 of its largest (the bar of test_gpu_parity); rows fewer than the
+    CTAs' shares, as many as the functions, and more than shared memory holds."""
+    s = synth.water_box(60, seed=3, L_A=14.0)
+    box = epsr.Box(s)
+    rng = np.random.default_rng(nQ)
+    Q = np.linspace(0.4, 25.0, nQ)
+    w = rng.uniform(0.05, 0.3, (3, 3))
+    F = oracle.ep_basis_matrix(n_basis, 0.5, Q.astype(np.float32).astype(np.float64), s.n_atoms / s.L ** 3)
+    dS = (w @ (rng.normal(size=(3, n_basis)) * 0.01 @ F.T)).astype(np.float32)
+    C = box.epsr_ep_update(0, torch.from_numpy(dS).to(DEV), w, Q, n_basis=n_basis, s_basis=0.5, gamma=0.0, alpha=1.0)
+    dSp = oracle.pair_resolve(dS.astype(np.float64), w, 0.0)
+    assert np.abs(C @ F.T - oracle.ep_fit(dSp, F) @ F.T).max() <= 1e-8 * np.abs(dSp).max()
