@@ -97,8 +97,8 @@ typedef struct {
     /* Lennard-Jones cutoff (A). 0, the form the paper's dU takes (every atom of the box):
      * LJ over every minimum-image pair. > 0: LJ plainly truncated at r_lj (the exact integer
      * test d^2 < llround(r_lj S)^2, no shift), so every partner beyond max(r_lj, r_coul, the
-     * EP table) contributes nothing and the sweep finds the others by cell queries: the cost
-     * of a move is O(neighbours) instead of O(N) (Sec. 2.3's cost statement). */
+     * EP table) contributes nothing and the sweep visits only the regions near the move: the
+     * cost of a move is O(neighbours) instead of O(N) (Sec. 2.3's cost statement). */
     double r_lj;
 } epsr_box_desc;
 
@@ -306,12 +306,9 @@ int epsr_checkpoint_load(epsr_box *box, const void *buf, size_t len, epsr_stream
  * the exact minimum-image counts. Asynchronous. Errors: EINVAL, ECUDA.                   */
 int epsr_partial_gr(epsr_box *box, uint64_t *hist, float *g, int64_t n_configs,
                     epsr_stream_t stream);
-/* The same histogram counted over cell lists: cells at least the histogram range wide
- * (at least 3 per side), each pair counted from its home cell against itself and the 13
- * forward neighbour cells, so the work is O(N * rho * r_max^3) instead of O(N^2) while
- * the integer counts are identical to epsr_partial_gr's. Boxes with fewer than three cells
- * per side are counted with the all-pairs kernel. Same arguments, accumulation and errors
- * as epsr_partial_gr. No counterpart in the paper, whose kernel is the O(N^2) scan. */
+/* The same histogram, once the entry of a cell-list form: both entries now count over compact
+ * clusters of atoms, with work O(N * rho * r_max^3) instead of the paper's O(N^2) scan and
+ * the same integer counts. Same arguments, accumulation and errors as epsr_partial_gr. */
 int epsr_partial_gr_cells(epsr_box *box, uint64_t *hist, float *g, int64_t n_configs,
                           epsr_stream_t stream);
 /* The same over a sub-range [pair_begin, pair_end) of the handle's pair-tile work list

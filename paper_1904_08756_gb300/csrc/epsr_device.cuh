@@ -172,7 +172,7 @@ __device__ __forceinline__ float ep_at(const float *row, float g2, Sep s, const 
 
 // A pair row whose Lennard-Jones term reaches every partner (LJ not cut): evaluated against
 // the whole slice. Any other row with a term is "near": non-zero only within near_fx of the
-// moved atom, so its partners can come from cell queries. CUT = false compiles the form
+// moved atom, so only the chunks of partners near it are visited. CUT = false compiles the form
 // without a cutoff (boxes with r_lj = 0); CUT = true reads the box's setting.
 template <bool CUT = true>
 __device__ __forceinline__ bool lj_full_row(const PairRow &r, const BoxDev &bx)
