@@ -1076,7 +1076,7 @@ static int gr_all(epsr_box *box, uint64_t *hist, cudaStream_t s)
     const int grid = box->sms * box->gr_ctas_per_sm;
     ClArgs a = cl_args(box, grid * 8);
     if (gr_clusters_smem(a.hist_cap) > (size_t)kClMaxSmem) return gr_range(box, 0, (long long)box->tiles_h.size(), hist, s);
-    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, s);
+    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, false, nullptr, s);
     if (rc) return rc;
     a.hist = (unsigned long long *)hist;
     return launch_gr_clusters(a, grid, s);
@@ -1498,7 +1498,7 @@ struct SmearPlan {
     int grid;
 };
 
-static int smear_plan(epsr_box *box, double sigma, SmearPlan *p, cudaStream_t s)
+static int smear_plan(epsr_box *box, double sigma, bool forward, SmearPlan *p, cudaStream_t s)
 {
     if (!(sigma > 0) || sigma > 2.0) return set_error(EPSR_EINVAL, "smeared g: sigma must be in (0, 2] A");
     memset(&p->a, 0, sizeof(p->a));
@@ -1520,14 +1520,15 @@ static int smear_plan(epsr_box *box, double sigma, SmearPlan *p, cudaStream_t s)
     if (p->smem > (size_t)kClMaxSmem) return set_error(EPSR_EINVAL, "smeared g: n_pairs*n_bins too large");
     p->grid = box->sms * (p->table ? 1 : 2);
     p->c = cl_args(box, p->grid * smear_warps_per_cta());
-    p->a.index = box->cl.index;
     p->a.sigma = sigma;
     p->a.node_off = box->node_off;
     p->a.moments = box->moments;
     p->a.table = box->sm_table;
     p->a.acc = box->smear_acc;
     p->a.lambda = box->lambda;
-    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, s);
+    // the forward repeats bit for bit, so its clusters must not depend on the timing of atomics: what is
+    // rounded into the moments depends on the centre of the i-cluster
+    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, forward, &p->a.index, s);
     if (!rc && p->table)
         rc = launch_smear_weights(box->boxes, box->n_boxes, sigma, p->a.nodes_cap, box->sm_weights, s);
     return rc;
@@ -1538,7 +1539,7 @@ extern "C" int epsr_gr_smeared_fwd(epsr_box *box, double sigma, double *Ht, floa
     if (!box || !Ht) return set_error(EPSR_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
     SmearPlan p;
-    int rc = smear_plan(box, sigma, &p, s);
+    int rc = smear_plan(box, sigma, true, &p, s);
     if (rc) return rc;
     if (p.table) CK(cudaMemsetAsync(box->moments, 0, (size_t)4 * box->n_nodes * sizeof(long long), s));
     else CK(cudaMemsetAsync(box->smear_acc, 0, (size_t)box->hist_len * sizeof(unsigned long long), s));
@@ -1555,7 +1556,7 @@ extern "C" int epsr_gr_smeared_bwd(epsr_box *box, double sigma, const float *dgt
     if (!box || !dgt || !grad) return set_error(EPSR_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
     SmearPlan p;
-    int rc = smear_plan(box, sigma, &p, s);
+    int rc = smear_plan(box, sigma, false, &p, s);
     if (rc) return rc;
     rc = launch_smear_lambda(box->boxes, box->n_boxes, dgt, box->lambda, box->hist_len, box->hist_box, s);
     if (!rc && p.table)

@@ -151,8 +151,12 @@ struct ClArgs {           // one traversal
 };
 constexpr int kClMaxSmem = 200 * 1024;
 size_t gr_clusters_smem(int hist_cap);
+// ordered: the order, and so the clusters, depend on the coordinates alone (one launch more); otherwise
+// atoms of one Hilbert cell may change places from call to call. *order: the atom at each position.
 int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords, long long n, const ClScratch &sc,
-                    cudaStream_t stream);
+                    bool ordered, const int **order, cudaStream_t stream);
+int launch_cell_order(const int *key, const int *count, const int *offset, const int *index, int *out, long long n,
+                      cudaStream_t stream);
 int launch_gr_clusters(const ClArgs &args, int grid, cudaStream_t stream);
 // exclusive scan of n counts (block: scratch [ceil(n / 1024)]), and the scatter of a counting sort
 int launch_scan(const int *count, int n, int *offset, int *block, cudaStream_t stream);

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(1024) cluster_boxes_kernel(const BoxDev *boxes
 }
 
 int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords, long long n, const ClScratch &sc,
-                    cudaStream_t stream)
+                    bool ordered, const int **order, cudaStream_t stream)
 {
     const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
     // the item counters of the traversal lie behind the key counts: one clear for both
@@ -157,7 +157,11 @@ int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords
     int rc = launch_scan(sc.count, sc.n_keys, sc.offset, sc.block, stream);
     if (rc) return rc;
     if ((rc = launch_scatter(sc.key, sc.rank, sc.offset, sc.index, n, stream))) return rc;
-    cluster_boxes_kernel<<<sc.n_su, 1024, 0, stream>>>(boxes, sc.box, sc.su_box, sc.index, coords, sc.coords, sc.cl_c,
+    // the ranks came from atomics; in order of the atoms' numbers (into the ranks' buffer) they do not matter
+    if (ordered && (rc = launch_cell_order(sc.key, sc.count, sc.offset, sc.index, sc.rank, n, stream))) return rc;
+    const int *index = ordered ? sc.rank : sc.index;
+    if (order) *order = index;
+    cluster_boxes_kernel<<<sc.n_su, 1024, 0, stream>>>(boxes, sc.box, sc.su_box, index, coords, sc.coords, sc.cl_c,
                                                        sc.cl_h, sc.su_c, sc.su_h);
     note_launch();
     e = cudaGetLastError();

@@ -223,6 +223,16 @@ int launch_scatter(const int *key, const int *rank, const int *offset, int *inde
     return e == cudaSuccess ? EPSR_OK : set_cuda_error(e, "scatter");
 }
 
+int launch_cell_order(const int *key, const int *count, const int *offset, const int *index, int *out, long long n,
+                      cudaStream_t stream)
+{
+    const int grid = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+    cell_order_kernel<<<grid, 256, 0, stream>>>(key, count, offset, index, nullptr, nullptr, out, nullptr, nullptr, nullptr, n);
+    note_launch();
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? EPSR_OK : set_cuda_error(e, "cell order");
+}
+
 int launch_spatial_sort(const BoxDev *boxes, const int *atom_box, const uint4 *scaled,
                         const int4 *coords, long long n, int total_cells, int type_major,
                         SortScratch sc, uint4 *s_scaled, int4 *s_coords, int *pos_of,

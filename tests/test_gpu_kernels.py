@@ -132,3 +132,15 @@ def test_ep_fit_edges(nQ, n_basis):
     C = box.epsr_ep_update(0, torch.from_numpy(dS).to(DEV), w, Q, n_basis=n_basis, s_basis=0.5, gamma=0.0, alpha=1.0)
     dSp = oracle.pair_resolve(dS.astype(np.float64), w, 0.0)
     assert np.abs(C @ F.T - oracle.ep_fit(dSp, F) @ F.T).max() <= 1e-8 * np.abs(dSp).max()
+
+
+def test_smeared_forward_repeats():
+    """Partners up to about 20 A from an i-cluster's centre, where relative coordinates are rounded: the
+    sums are the same bits in every call (the order of the clusters may not depend on timing)."""
+    s = synth.uniform_gas(30000, 76.8, seed=9, n_types=2)
+    s.bin_p, s.bin_q, s.n_bins = 1, 25, 350
+    box = epsr.Box(s)
+    Ht = torch.zeros((8, box.hist_len), dtype=torch.float64, device=DEV)
+    for row in Ht:
+        box.epsr_gr_smeared_fwd(0.05, row)
+    assert torch.equal(Ht[0].expand_as(Ht), Ht)
