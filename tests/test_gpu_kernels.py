@@ -144,3 +144,35 @@ def test_smeared_forward_repeats():
     for row in Ht:
         box.epsr_gr_smeared_fwd(0.05, row)
     assert torch.equal(Ht[0].expand_as(Ht), Ht)
+
+
+@pytest.mark.parametrize("types", [(2, 1, 3), (4, 2, 5)], ids=["nodes", "direct"])
+def test_smeared_boxes_of_one_handle(types):
+    """Boxes of different types, sizes and bins in one handle, each against the oracle with the bars of
+    test_smeared_edges; on the node grid, and with more types than it holds, pair by pair from queues."""
+    systems = []
+    for i, (n, L, bins) in enumerate([(2100, 27.0, 200), (40, 20.0, 160), (1057, 22.0, 120)]):
+        s = synth.uniform_gas(n, L, seed=n, n_types=types[i])
+        s.bin_p, s.bin_q, s.n_bins = 1, 25, bins
+        systems.append(s)
+    box = epsr.Box(systems)
+    Ht = torch.zeros(box.hist_len, dtype=torch.float64, device=DEV)
+    box.epsr_gr_smeared_fwd(0.05, Ht)
+    dgt, want = [], []
+    h0 = 0
+    for s in systems:
+        ob = oracle.Box(s)
+        ref = ob.smeared_hist(0.05)
+        got = Ht[h0:h0 + ref.size].cpu().numpy().reshape(ref.shape)
+        assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max()
+        h0 += ref.size
+        lam = np.cos(np.arange(ref.size).reshape(ref.shape) * s.dr * 2.0)
+        _, factor = oracle.smeared_g(ob, ref)
+        dgt.append((lam / factor).astype(np.float32).reshape(-1))
+        want.append(ob.smeared_grad(0.05, lam))
+    grad = torch.zeros((box.n_atoms, 3), dtype=torch.float32, device=DEV)
+    box.epsr_gr_smeared_bwd(0.05, torch.from_numpy(np.concatenate(dgt)).to(DEV), grad)
+    a0 = 0
+    for g in want:
+        assert np.linalg.norm(grad[a0:a0 + len(g)].cpu().numpy() - g) <= 1e-4 * np.linalg.norm(g)
+        a0 += len(g)
