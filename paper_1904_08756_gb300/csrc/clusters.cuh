@@ -241,7 +241,7 @@ __device__ __forceinline__ int next_box(const ClArgs &A, int from, int *s_found)
 // First box of a CTA: the one holding cluster blockIdx / gridDim of all clusters.
 __device__ __forceinline__ int start_box(const ClArgs &A)
 {
-    const long long c = (long long)blockIdx.x * A.n_cl_total / gridDim.x;
+    const long long c = A.box[0].cl0 + (long long)blockIdx.x * A.n_cl_total / gridDim.x;
     int lo = 0, hi = A.n_boxes;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;

@@ -158,12 +158,9 @@ struct epsr_box {
     long long ep_cap_Q = 0;
     float *lambda = nullptr;     // adjoint of the smeared normalisation [hist_len]
     unsigned long long *smear_acc = nullptr;   // fixed-point smeared counts [hist_len]
-    // smeared histogram on nodes: moments and derivative table, first node of each box, weights
-    std::vector<long long> node_off_h;
-    long long *node_off = nullptr, *moments = nullptr;
-    float4 *sm_table = nullptr;
-    double *sm_weights = nullptr;
-    long long n_nodes = 0;
+    // smeared histogram on nodes: moments or derivative table, then weights, of a group of boxes
+    unsigned char *sm_ws = nullptr;
+    size_t sm_ws_bytes = 0;
     // clusters of 32 atoms in Hilbert order (pair histogram)
     std::vector<ClBox> cl_box_h;
     ClBox *cl_box = nullptr;
@@ -182,7 +179,7 @@ struct epsr_box {
                         sorted_scaled, sorted_coords, moves, mc_sort.count, mc_sort.offset,
                         mc_sort.block, mc_sort.key, mc_sort.rank, mc_sort.index, pos_of,
                         ep_F, ep_Y, ep_C, ep_B, ep_Q, lambda, smear_acc, slice_g,
-                        node_off, moments, sm_table, sm_weights,
+                        sm_ws,
                         cl_box, cl_su_box, cl.count, cl.offset, cl.block, cl.coords,
                         cl.cl_c, cl.cl_h, cl.su_c, cl.su_h};
         for (void *p : ptrs)
@@ -542,11 +539,12 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         }
         set_near(bx);
         set_prefilter(bx);
-        // nodes of the smeared histogram: the most that kSmMaxS per bin, the reach of 5 sigma
-        // (kSmOffsets / 2) and shared memory allow
-        h->node_off_h.push_back(h->n_nodes);
-        h->n_nodes += (long long)bx.n_pairs * std::min<long long>((long long)bx.n_bins * kSmMaxS + kSmOffsets / 2,
-                                                                  kClMaxSmem / 16 / bx.n_pairs + 1);
+        // the smeared form's most: kSmMaxS nodes a bin, the reach of 5 sigma (kSmOffsets / 2), but no
+        // more than shared memory holds
+        const size_t need = (size_t)bx.n_pairs * std::min<size_t>((size_t)bx.n_bins * kSmMaxS + kSmOffsets / 2,
+                                                                  kClMaxSmem / 16 / bx.n_pairs + 1) * 32 +
+                            5 * kSmOffsets * sizeof(double);
+        h->sm_ws_bytes = std::max(need, std::min(h->sm_ws_bytes + need, kSmWorkspace));
         // clusters: about 3 A Hilbert cells (a power of two per side, at most one cell per atom)
         ClBox cb;
         memset(&cb, 0, sizeof(cb));
@@ -605,9 +603,7 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
         (rc = dalloc(&h->mc_sort.key, atom0)) || (rc = dalloc(&h->mc_sort.rank, atom0)) ||
         (rc = dalloc(&h->mc_sort.index, atom0)) || (rc = dalloc(&h->pos_of, atom0)) ||
         (rc = dalloc(&h->lambda, (size_t)hist0)) || (rc = dalloc(&h->smear_acc, (size_t)hist0)) ||
-        (rc = dalloc(&h->node_off, n_boxes)) || (rc = dalloc(&h->moments, (size_t)4 * h->n_nodes)) ||
-        (rc = dalloc(&h->sm_table, (size_t)h->n_nodes)) ||
-        (rc = dalloc(&h->sm_weights, (size_t)n_boxes * 5 * kSmOffsets)) ||
+        (rc = dalloc(&h->sm_ws, h->sm_ws_bytes)) ||
         (rc = dalloc(&h->cl_box, n_boxes)) || (rc = dalloc(&h->cl_su_box, su_box.size())) ||
         (rc = dalloc(&h->cl.count, (size_t)h->cl.n_keys_pad + n_boxes)) ||
         (rc = dalloc(&h->cl.offset, h->cl.n_keys)) ||
@@ -634,7 +630,6 @@ static int create_impl(const epsr_box_desc *descs, int n_boxes, const int32_t *x
     CKD(cudaMemcpyAsync(h->thresholds, T.data(), T.size() * sizeof(long long), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemsetAsync(h->ep, 0, (size_t)std::max(ep0, 1) * sizeof(float), stream));
     CKD(cudaMemcpyAsync(h->tiles, h->tiles_h.data(), h->tiles_h.size() * sizeof(GrTile), cudaMemcpyHostToDevice, stream));
-    CKD(cudaMemcpyAsync(h->node_off, h->node_off_h.data(), n_boxes * sizeof(long long), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->cl_box, h->cl_box_h.data(), n_boxes * sizeof(ClBox), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->cl_su_box, su_box.data(), su_box.size() * sizeof(int), cudaMemcpyHostToDevice, stream));
     CKD(cudaMemcpyAsync(h->hist_box, h->hist_box_h.data(), n_boxes * sizeof(long long), cudaMemcpyHostToDevice, stream));
@@ -1046,26 +1041,29 @@ extern "C" int epsr_partial_gr_range(epsr_box *box, int64_t tile_begin, int64_t 
     return gr_range(box, tile_begin, tile_end, hist, (cudaStream_t)stream);
 }
 
-// Traversal of every box's clusters, set up for the current coordinates.
-static ClArgs cl_args(epsr_box *box, int warps)
+// Traversal of the clusters of n boxes from b0 on, set up for the current coordinates.
+static ClArgs cl_args(epsr_box *box, int b0, int n, int warps)
 {
     ClArgs a;
     memset(&a, 0, sizeof(a));
-    a.boxes = box->boxes;
-    a.box = box->cl_box;
+    a.boxes = box->boxes + b0;
+    a.box = box->cl_box + b0;
     a.coords = box->cl.coords;
     a.cl_c = box->cl.cl_c;
     a.cl_h = box->cl.cl_h;
     a.su_c = box->cl.su_c;
     a.su_h = box->cl.su_h;
-    a.next_item = box->cl.count + box->cl.n_keys_pad;
+    a.next_item = box->cl.count + box->cl.n_keys_pad + b0;
     a.thresholds = box->thresholds;
-    a.n_cl_total = box->n_cl;
-    a.n_boxes = box->n_boxes;
+    a.n_boxes = n;
+    for (int b = b0; b < b0 + n; ++b) {
+        const BoxDev &bx = box->hb[b];
+        a.n_cl_total += box->cl_box_h[b].n_cl;
+        a.hist_cap = std::max(a.hist_cap, bx.n_types * bx.n_types * bx.n_bins);
+    }
     // at least four items per warp, so that the last ones to finish idle the chip little; more
     // shares repeat the box tests of a cluster
-    while (a.plog < 5 && (box->n_cl << a.plog) < 4LL * warps) ++a.plog;
-    for (const auto &b : box->hb) a.hist_cap = std::max(a.hist_cap, b.n_types * b.n_types * b.n_bins);
+    while (a.plog < 5 && (a.n_cl_total << a.plog) < 4LL * warps) ++a.plog;
     return a;
 }
 
@@ -1074,7 +1072,7 @@ static ClArgs cl_args(epsr_box *box, int warps)
 static int gr_all(epsr_box *box, uint64_t *hist, cudaStream_t s)
 {
     const int grid = box->sms * box->gr_ctas_per_sm;
-    ClArgs a = cl_args(box, grid * 8);
+    ClArgs a = cl_args(box, 0, box->n_boxes, grid * 8);
     if (gr_clusters_smem(a.hist_cap) > (size_t)kClMaxSmem) return gr_range(box, 0, (long long)box->tiles_h.size(), hist, s);
     int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, false, nullptr, s);
     if (rc) return rc;
@@ -1488,20 +1486,22 @@ extern "C" int epsr_ep_update(epsr_box *box, int32_t b, const float *dS, int32_t
 }
 
 // ---- differentiable form: smeared histogram, adjoints, chi^2 ----------------------------------
-// One traversal of the smeared form: on nodes when every box's node grid fits in shared memory,
-// pair by pair otherwise.
+// The smeared form: on nodes when every box's node grid fits in shared memory, pair by pair otherwise.
+// On nodes the boxes are taken in groups that the workspace holds, so that a handle keeps at most
+// kSmWorkspace (or one box's need) however many boxes it has, and the call allocates nothing.
 struct SmearPlan {
-    ClArgs c;
     SmearArgs a;
     bool table;
     size_t smem;
     int grid;
+    int group, offs;      // boxes per group; offsets of the weight table
+    double *W;
 };
 
 static int smear_plan(epsr_box *box, double sigma, bool forward, SmearPlan *p, cudaStream_t s)
 {
     if (!(sigma > 0) || sigma > 2.0) return set_error(EPSR_EINVAL, "smeared g: sigma must be in (0, 2] A");
-    memset(&p->a, 0, sizeof(p->a));
+    memset(p, 0, sizeof(*p));
     int np = 1, rows = 1;
     for (const auto &b : box->hb) {
         np = std::max(np, b.n_pairs);
@@ -1510,28 +1510,35 @@ static int smear_plan(epsr_box *box, double sigma, bool forward, SmearPlan *p, c
     const size_t lists = smear_smem(true, 0);
     p->a.nodes_cap = (int)(((size_t)kClMaxSmem - lists) / 16 / np);
     p->table = true;
-    long long most = 0;
     for (const auto &b : box->hb) {
         const SmearGrid g = smear_grid(b.n_bins, b.dr_A, sigma, p->a.nodes_cap);
         p->table = p->table && g.S > 0;
-        if (g.S > 0) most = std::max(most, (long long)b.n_pairs * g.nodes);
+        if (g.S == 0) break;
+        p->a.stride = std::max(p->a.stride, (long long)b.n_pairs * g.nodes);
+        p->offs = std::max(p->offs, g.n_off);
     }
-    p->smem = p->table ? smear_smem(true, most) : smear_smem(false, rows);
+    p->smem = p->table ? smear_smem(true, p->a.stride) : smear_smem(false, rows);
     if (p->smem > (size_t)kClMaxSmem) return set_error(EPSR_EINVAL, "smeared g: n_pairs*n_bins too large");
     p->grid = box->sms * (p->table ? 1 : 2);
-    p->c = cl_args(box, p->grid * smear_warps_per_cta());
+    p->group = box->n_boxes;
+    if (p->table) {
+        const size_t per_box = (size_t)p->a.stride * 32 + (size_t)p->offs * 5 * sizeof(double);
+        p->group = (int)std::min<size_t>({(size_t)box->n_boxes, box->sm_ws_bytes / per_box, (size_t)kSmMaxGroup});
+        p->a.moments = (long long *)box->sm_ws;
+        p->a.table = (const float4 *)box->sm_ws;
+        p->W = (double *)(box->sm_ws + (size_t)p->group * p->a.stride * 32);
+    }
     p->a.sigma = sigma;
-    p->a.node_off = box->node_off;
-    p->a.moments = box->moments;
-    p->a.table = box->sm_table;
     p->a.acc = box->smear_acc;
     p->a.lambda = box->lambda;
     // the forward repeats bit for bit, so its clusters must not depend on the timing of atomics: what is
     // rounded into the moments depends on the centre of the i-cluster
-    int rc = launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, forward, &p->a.index, s);
-    if (!rc && p->table)
-        rc = launch_smear_weights(box->boxes, box->n_boxes, sigma, p->a.nodes_cap, box->sm_weights, s);
-    return rc;
+    return launch_clusters(box->boxes, box->atom_box, box->coords, box->n_atoms, box->cl, forward, &p->a.index, s);
+}
+
+static int smear_traverse(epsr_box *box, const SmearPlan &p, int b0, int n, bool backward, cudaStream_t s)
+{
+    return launch_smear(cl_args(box, b0, n, p.grid * smear_warps_per_cta()), p.a, backward, p.table, p.smem, p.grid, s);
 }
 
 extern "C" int epsr_gr_smeared_fwd(epsr_box *box, double sigma, double *Ht, float *gt, epsr_stream_t stream)
@@ -1541,13 +1548,22 @@ extern "C" int epsr_gr_smeared_fwd(epsr_box *box, double sigma, double *Ht, floa
     SmearPlan p;
     int rc = smear_plan(box, sigma, true, &p, s);
     if (rc) return rc;
-    if (p.table) CK(cudaMemsetAsync(box->moments, 0, (size_t)4 * box->n_nodes * sizeof(long long), s));
-    else CK(cudaMemsetAsync(box->smear_acc, 0, (size_t)box->hist_len * sizeof(unsigned long long), s));
-    if ((rc = launch_smear(p.c, p.a, false, p.table, p.smem, p.grid, s))) return rc;
-    if (p.table)
-        return launch_smear_bins(box->boxes, box->n_boxes, sigma, p.a.nodes_cap, box->node_off, box->moments,
-                                 box->sm_weights, Ht, gt, box->hist_len, box->hist_box, s);
-    return launch_smear_norm(box->boxes, box->n_boxes, box->smear_acc, Ht, gt, box->hist_len, box->hist_box, s);
+    if (!p.table) {
+        CK(cudaMemsetAsync(box->smear_acc, 0, (size_t)box->hist_len * sizeof(unsigned long long), s));
+        if ((rc = smear_traverse(box, p, 0, box->n_boxes, false, s))) return rc;
+        return launch_smear_norm(box->boxes, box->n_boxes, box->smear_acc, Ht, gt, box->hist_len, box->hist_box, s);
+    }
+    for (int b0 = 0; b0 < box->n_boxes; b0 += p.group) {
+        const int n = std::min(p.group, box->n_boxes - b0);
+        const long long h0 = box->hist_box_h[b0], h1 = b0 + n < box->n_boxes ? box->hist_box_h[b0 + n] : box->hist_len;
+        if ((rc = launch_smear_weights(box->boxes + b0, n, sigma, p.a.nodes_cap, p.offs, p.W, s))) return rc;
+        CK(cudaMemsetAsync(p.a.moments, 0, (size_t)n * p.a.stride * 32, s));
+        if ((rc = smear_traverse(box, p, b0, n, false, s))) return rc;
+        if ((rc = launch_smear_bins(box->boxes + b0, n, sigma, p.a.nodes_cap, p.offs, p.a.stride, p.a.moments, p.W, Ht, gt, h0,
+                                    h1, box->hist_box + b0, s)))
+            return rc;
+    }
+    return EPSR_OK;
 }
 
 extern "C" int epsr_gr_smeared_bwd(epsr_box *box, double sigma, const float *dgt, float *grad,
@@ -1559,13 +1575,18 @@ extern "C" int epsr_gr_smeared_bwd(epsr_box *box, double sigma, const float *dgt
     int rc = smear_plan(box, sigma, false, &p, s);
     if (rc) return rc;
     rc = launch_smear_lambda(box->boxes, box->n_boxes, dgt, box->lambda, box->hist_len, box->hist_box, s);
-    if (!rc && p.table)
-        rc = launch_smear_table(box->boxes, box->n_boxes, sigma, p.a.nodes_cap, box->node_off, box->sm_weights,
-                                box->lambda, box->sm_table, s);
     if (rc) return rc;
     CK(cudaMemsetAsync(grad, 0, (size_t)box->n_atoms * 3 * sizeof(float), s));
     p.a.grad = grad;
-    return launch_smear(p.c, p.a, true, p.table, p.smem, p.grid, s);
+    for (int b0 = 0; b0 < box->n_boxes; b0 += p.group) {
+        const int n = std::min(p.group, box->n_boxes - b0);
+        if (p.table && ((rc = launch_smear_weights(box->boxes + b0, n, sigma, p.a.nodes_cap, p.offs, p.W, s)) ||
+                        (rc = launch_smear_table(box->boxes + b0, n, sigma, p.a.nodes_cap, p.offs, p.a.stride, p.W, box->lambda,
+                                                 (float4 *)box->sm_ws, s))))
+            return rc;
+        if ((rc = smear_traverse(box, p, b0, n, true, s))) return rc;
+    }
+    return EPSR_OK;
 }
 
 extern "C" int epsr_sq_exec_adjoint(epsr_sq_plan *plan, const float *dS_total, int32_t n_cols,

@@ -195,6 +195,10 @@ struct SmearGrid {
 };
 constexpr int kSmOffsets = 2048;      // offsets of the weight table, at most
 constexpr int kSmMaxS = 16;           // nodes per bin, at most
+// Workspace of a handle: per box moments or derivative table (4 x 8 bytes a node and type pair), then
+// weights (5 doubles an offset). Handles of many boxes take them in groups of as many as fit.
+constexpr size_t kSmWorkspace = 64u << 20;
+constexpr int kSmMaxGroup = 32768;    // boxes in grid.y
 // h = sigma / 12, or as fine as nodes_cap nodes allow; S = 0 when that leaves it above sigma / 8.
 inline
 #ifdef __CUDACC__
@@ -221,9 +225,9 @@ struct SmearArgs {
     const int *index;          // atom at each position in cluster order
     double sigma;
     int nodes_cap;             // nodes per type pair that fit in shared memory
-    const long long *node_off; // [n_boxes] first node of the box in the moments (x 4) and the table
-    long long *moments;        // forward, nodes: [4][n_pairs][nodes] per box, accumulated
-    const float4 *table;       // backward, nodes: [n_pairs][nodes] per box
+    long long stride;          // nodes x type pairs per box, at most
+    long long *moments;        // forward, nodes: [n_boxes][4 stride], per box [4][n_pairs][nodes], accumulated
+    const float4 *table;       // backward, nodes: [n_boxes][stride], per box [n_pairs][nodes]
     unsigned long long *acc;   // forward, direct: weights * 2^20, accumulated
     const float *lambda;       // backward, direct: dL/dHt [hist_len]
     float *grad;               // backward output [n_atoms_total][3] (accumulated)
@@ -231,11 +235,13 @@ struct SmearArgs {
 size_t smear_smem(bool table, long long rows);
 int smear_warps_per_cta();
 int launch_smear(const ClArgs &c, const SmearArgs &a, bool backward, bool table, size_t smem, int grid, cudaStream_t stream);
-int launch_smear_weights(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, double *W, cudaStream_t stream);
-int launch_smear_bins(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, const long long *node_off,
-                      const long long *moments, const double *W, double *Ht, float *gt, long long hist_len,
+// weights W [n_boxes][5][offs]; moments and table as in SmearArgs; hist_box the first rows of these boxes,
+// of which Ht and gt rows h0 .. h1 - 1 are formed
+int launch_smear_weights(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, int offs, double *W, cudaStream_t stream);
+int launch_smear_bins(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, int offs, long long stride,
+                      const long long *moments, const double *W, double *Ht, float *gt, long long h0, long long h1,
                       const long long *hist_box, cudaStream_t stream);
-int launch_smear_table(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, const long long *node_off,
+int launch_smear_table(const BoxDev *boxes, int n_boxes, double sigma, int nodes_cap, int offs, long long stride,
                        const double *W, const float *lam, float4 *table, cudaStream_t stream);
 int launch_smear_norm(const BoxDev *boxes, int n_boxes, const unsigned long long *acc, double *Ht,
                       float *gt, long long hist_len, const long long *hist_box, cudaStream_t stream);

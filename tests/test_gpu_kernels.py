@@ -176,3 +176,39 @@ def test_smeared_boxes_of_one_handle(types):
     for g in want:
         assert np.linalg.norm(grad[a0:a0 + len(g)].cpu().numpy() - g) <= 1e-4 * np.linalg.norm(g)
         a0 += len(g)
+
+
+def test_smeared_handles_of_many_boxes():
+    """A handle of 1,000 boxes holds no workspace of its own per box (it was 0.7 MB each); 400 boxes that
+    need more than the workspace are taken in groups: boxes at the groups' ends against the oracle with
+    the bars of test_smeared_edges."""
+    s = synth.uniform_gas(30, 20.0, seed=2, n_types=2)
+    s.bin_p, s.bin_q, s.n_bins = 1, 25, 200
+    free, held = [], []
+    for n in (100, 1000):
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+        held.append(epsr.Box([s] * n))
+    free.append(torch.cuda.mem_get_info()[0])
+    assert (free[1] - free[2]) - (free[0] - free[1]) < 200 << 20
+    for h in held:
+        h.close()
+    systems = []
+    for i in range(400):
+        s = synth.uniform_gas(900, 16.0, seed=i, n_types=2)
+        s.bin_p, s.bin_q, s.n_bins = 1, 25, 200
+        systems.append(s)
+    box = epsr.Box(systems)
+    Ht = torch.zeros(box.hist_len, dtype=torch.float64, device=DEV)
+    box.epsr_gr_smeared_fwd(0.05, Ht)
+    lam = np.cos(np.arange(600).reshape(3, -1) * 0.08)
+    ob = oracle.Box(systems[0])
+    _, factor = oracle.smeared_g(ob, ob.smeared_hist(0.05))
+    dgt = np.tile((lam / factor).astype(np.float32).reshape(-1), 400)
+    grad = torch.zeros((box.n_atoms, 3), dtype=torch.float32, device=DEV)
+    box.epsr_gr_smeared_bwd(0.05, torch.from_numpy(dgt).to(DEV), grad)
+    for b in [0, 1, *range(325, 333), 399]:
+        ob = oracle.Box(systems[b])
+        ref, gref = ob.smeared_hist(0.05), ob.smeared_grad(0.05, lam)
+        assert np.abs(Ht[600 * b:600 * b + 600].cpu().numpy().reshape(3, -1) - ref).max() <= 1e-5 * np.abs(ref).max()
+        assert np.linalg.norm(grad[900 * b:900 * b + 900].cpu().numpy() - gref) <= 1e-4 * np.linalg.norm(gref)
