@@ -212,3 +212,23 @@ def test_smeared_handles_of_many_boxes():
         ref, gref = ob.smeared_hist(0.05), ob.smeared_grad(0.05, lam)
         assert np.abs(Ht[600 * b:600 * b + 600].cpu().numpy().reshape(3, -1) - ref).max() <= 1e-5 * np.abs(ref).max()
         assert np.linalg.norm(grad[900 * b:900 * b + 900].cpu().numpy() - gref) <= 1e-4 * np.linalg.norm(gref)
+
+
+@pytest.mark.parametrize("n,L,boxes", [(60, 10.0, 300), (2, 9.0, 200)], ids=["few-pairs", "two-atoms"])
+def test_smeared_many_small_boxes(n, L, boxes):
+    """Handles of many boxes with few pairs each, which are smeared pair by pair: every box against the
+    oracle with the bars of test_smeared_edges (and one weight's rounding, 2^-21, for single pairs)."""
+    systems = []
+    for i in range(boxes):
+        s = synth.uniform_gas(n, L, seed=1000 + i, n_types=2)
+        s.bin_p, s.bin_q, s.n_bins = 3, 100, 140 + i % 3
+        systems.append(s)
+    box = epsr.Box(systems)
+    Ht = torch.zeros(box.hist_len, dtype=torch.float64, device=DEV)
+    box.epsr_gr_smeared_fwd(0.05, Ht)
+    h0 = 0
+    for s in systems:
+        ref = oracle.Box(s).smeared_hist(0.05)
+        got = Ht[h0:h0 + ref.size].cpu().numpy().reshape(ref.shape)
+        assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max() + 2.0 ** -21
+        h0 += ref.size
