@@ -479,10 +479,12 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
         op4 = op[kk];
         int nx, ny, nz;
         if (mr.kind == 1) {
-            // minimum-image offsets from atom 0 (below 2^25), summed over the molecule, and this atom's own
+            // minimum-image offsets from atom 0, summed over the molecule, and this atom's own (sums in 64
+            // bits: below 2^25 where a box is made, but atoms without springs may drift apart)
             const int4 b0 = op[0];
             const int hl = L >> 1;
-            int sx = 0, sy = 0, sz = 0, ox = 0, oy = 0, oz = 0;
+            long long sx = 0, sy = 0, sz = 0;
+            int ox = 0, oy = 0, oz = 0;
             for (int i = 0; i < m; ++i) {
                 const int4 c = op[i];
                 const int dx = mi_signed32(c.x - b0.x, L, hl), dy = mi_signed32(c.y - b0.y, L, hl),
@@ -490,16 +492,13 @@ __device__ __noinline__ void trial_moves(McBatch &b, const MoveRec *ring, long l
                 sx += dx; sy += dy; sz += dz;
                 if (i == kk) { ox = dx; oy = dy; oz = dz; }
             }
-            const int ux = m * ox - sx, uy = m * oy - sy, uz = m * oz - sz;
+            const long long ux = (long long)m * ox - sx, uy = (long long)m * oy - sy, uz = (long long)m * oz - sz;
             const int *R = mr.R;
             // per axis: s 2^30 + R (m o - s), then floor((. + m 2^29) / 2^30) (32 bits) and
             // floor division by m
-            const long long numx = (long long)sx * 1073741824LL + (long long)R[0] * ux + (long long)R[1] * uy +
-                                   (long long)R[2] * uz;
-            const long long numy = (long long)sy * 1073741824LL + (long long)R[3] * ux + (long long)R[4] * uy +
-                                   (long long)R[5] * uz;
-            const long long numz = (long long)sz * 1073741824LL + (long long)R[6] * ux + (long long)R[7] * uy +
-                                   (long long)R[8] * uz;
+            const long long numx = sx * 1073741824LL + R[0] * ux + R[1] * uy + R[2] * uz;
+            const long long numy = sy * 1073741824LL + R[3] * ux + R[4] * uy + R[5] * uz;
+            const long long numz = sz * 1073741824LL + R[6] * ux + R[7] * uy + R[8] * uz;
             const long long half = (long long)m * 536870912LL;
             nx = wrap_near(b0.x, floordiv32((int)((numx + half) >> 30), m) + mr.shift[0], L);
             ny = wrap_near(b0.y, floordiv32((int)((numy + half) >> 30), m) + mr.shift[1], L);

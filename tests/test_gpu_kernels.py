@@ -257,3 +257,25 @@ def test_energy_change_error_with_many_ctas():
         if e["accepted"]:
             ob.apply(mol, trial)
     assert np.sqrt(err / ref) <= 0.95e-7
+
+
+def test_rotation_of_a_wide_molecule():
+    """Trial coordinates of a molecule whose atoms lie 690 A to both sides of the first (three times the
+    offset is past 2^31 grid units), wherever the rotated sum fits 32 bits again."""
+    s = synth.uniform_gas(3, 100.0, seed=1, n_types=1)
+    s.L_fx, s.mol_start, s.rigid_molecules = 2147483646, np.array([0, 3]), True
+    s.max_translation, s.max_rotation_deg = 0.0, 60.0
+    s.xyz = np.array([[5, 6, 7], [25, 6, 7], [5, 9, 7]], np.int32)
+    box = epsr.Box(s)
+    a = 720000000
+    wide = np.array([[1000000000, 5, 3], [1000000000 + a, 5, 3], [1000000000 - a, 5, 3]], np.int32)
+    checked = 0
+    for t in range(40):
+        box.epsr_box_set_coords(wide)
+        _, log = run_logged(box, 1, seed=3, move0=t)
+        _, trial, _ = oracle.Box(s, xyz=wide).propose(3, t)
+        p = (trial.astype(np.int64) - wide[0] + s.L_fx // 2) % s.L_fx - s.L_fx // 2
+        if (np.abs(p) * 3 + 3 < 2 ** 31).all():
+            checked += 1
+            assert np.array_equal(log[0][0]["trial"][:3], trial)
+    assert checked > 20
