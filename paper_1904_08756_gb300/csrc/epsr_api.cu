@@ -311,13 +311,15 @@ static void plan_mc_groups(epsr_box *h)
     // gives each box one CTA, then the rest greedily to the largest slices. The sweep never got
     // slower with more CTAs (us a move, 64 a batch: 900-atom water 0.84 on 14 CTAs, 0.66 on 29;
     // 3,000 atoms 0.60 on 24, 0.50 on 94; 12,000-atom flexible water with an empirical potential
-    // 0.45 on 48, 0.36 on 152; 12,000-atom silica 0.29 on 48, 0.24 on 152).
+    // 0.45 on 48, 0.36 on 152; 12,000-atom silica 0.29 on 48, 0.24 on 152), except where the exchange
+    // outweighs two chunks: 60 atoms 1.01 on one CTA, 1.14 on two; 90 atoms as 30 molecules 1.88 and 1.82.
+    const int least = h->mc_ctas > 0 ? 32 : 64;      // atoms that one CTA takes alone
     const int nb = h->n_boxes;
     const int budget = h->mc_ctas > 0 ? h->mc_ctas : h->sms;
     h->total_mc_cells = 0;
     std::vector<int> G(nb, 1);
     if (nb == 1) {
-        const long long want = (h->hb[0].n_atoms + 31) / 32;
+        const long long want = h->hb[0].n_atoms <= least ? 1 : (h->hb[0].n_atoms + 31) / 32;
         G[0] = (int)std::max(1LL, std::min<long long>(want, budget));
     } else {
         // every box starts with one CTA; each further CTA goes to the box whose per-CTA
@@ -330,7 +332,7 @@ static void plan_mc_groups(epsr_box *h)
                 const long long c = (h->hb[i].n_atoms + G[i] - 1) / G[i];
                 if (c > worst) { worst = c; imax = i; }
             }
-            if (worst <= 32) break;
+            if (worst <= (G[imax] == 1 ? least : 32)) break;
             ++G[imax];
             ++used;
         }

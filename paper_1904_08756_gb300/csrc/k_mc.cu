@@ -771,7 +771,9 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         int nb_next = 0;
         // ---- A, B. the next batch, while the partials of the current one reach the other CTAs --------
         // Its current and trial coordinates (integer arithmetic). The decisions of the current batch are
-        // not known yet: the few molecules that they move are taken up again after them.
+        // not known yet: the few molecules that they move are taken up again after them. (A single CTA
+        // waits for nobody, and takes them once, after the decisions: 300 moves of 3 atoms 1275 -> 1105 us,
+        // of 60 atoms 343 -> 303, of one water molecule 2990 -> 2445.)
         if (tn < A.n_moves) {
             nb_next = min((int)min((long long)batch_k, A.n_moves - tn), sh.nb_min);
             if (tid == 0) nxt.nb = nb_next;
@@ -782,8 +784,10 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
                 nxt.spos[gk][gsub] = gp - (int)bx.atom0;
                 if (gsub == 0) nxt.mol[gk] = mol;
             }
-            __syncthreads();
-            if (prep_warp) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
+            if (G > 1) {
+                __syncthreads();
+                if (prep_warp) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
+            }
         }
         bool again = false;
         if (nb > 0) {
@@ -1012,7 +1016,7 @@ __global__ void __launch_bounds__(kMcThreads, 1) mc_sweep_kernel(McArgs A)
         par ^= 1;
         t0 = tn;
         nb = nb_next;
-        if (__syncthreads_or(again)) {
+        if (__syncthreads_or(again || G == 1)) {
             if (prep_warp) trial_moves<CUT>(nxt, sh.ring, tn, nb_next, bx);
             __syncthreads();
         }

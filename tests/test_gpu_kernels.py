@@ -279,3 +279,19 @@ def test_rotation_of_a_wide_molecule():
             checked += 1
             assert np.array_equal(log[0][0]["trial"][:3], trial)
     assert checked > 20
+
+
+def test_sweep_small_boxes_replay():
+    """Boxes around the size up to which one CTA sweeps alone (and prepares a batch after the decisions of the
+    one before), in one handle: every move of every box against the oracle."""
+    systems = [mixed_box([1], 12, 2, seed=1), mixed_box([1, 3], 32, 3, seed=2), mixed_box([1], 65, 2, seed=3),
+               mixed_box([3], 2, 2, seed=4), mixed_box([1, 2], 140, 2, seed=5)]
+    box = epsr.Box(systems)
+    _, log = run_logged(box, 500, seed=21)
+    xyz = box.epsr_box_get_coords()
+    a0 = 0
+    for b, s in enumerate(systems):
+        ob, _, _, flips = replay(s, s.xyz, log[b], 21, box_index=b)
+        assert flips <= 2
+        assert np.array_equal(xyz[a0:a0 + s.n_atoms], ob.xyz)
+        a0 += s.n_atoms
