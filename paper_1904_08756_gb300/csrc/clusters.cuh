@@ -12,9 +12,10 @@
 // Fast coordinates: relative to the centre c of the i-cluster's box, j' = wrap(x_j - c) and
 // i' = x_i - c as FP32. With h the half width of the box, |i'| <= h <= 2^23 is exact, and an
 // atom inside the range R of some i has |j'| <= R + h; where 2 (R + h) < L the difference j' - i'
-// is the minimum image of every pair in range, and where R + h <= 2^25 it is off by at most one
-// grid unit, and only when |j'| >= 2^24, where the pair is longer than 2^24 - 2^23 = 2^23 units:
-// the squared distance then carries a relative error below 2^-21.1 + 2^-22 (rounding of the
+// is the minimum image of every pair in range, and where R + h <= 2^25 it is off by the rounding of
+// j', at most one grid unit and only when |j'| >= 2^24, where the component is longer than 2^24 -
+// 2^23 = 2^23 units, and by its own, one more from 2^24 units on: either is at most 2^-23 of the
+// component, so the squared distance carries a relative error below 2^-21 + 2^-22 (rounding of the
 // squares), its root half of that. Clusters that do not meet the three conditions (boxes less
 // than about twice the range wide, sparse boxes, fine grids) keep integer coordinates in the
 // list and take the integer minimum image per pair.

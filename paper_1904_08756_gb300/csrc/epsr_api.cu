@@ -853,9 +853,7 @@ int box_summary(const epsr_box *box, int b, BoxSummary *out)
     out->n_boxes = box->n_boxes;
     out->n_pairs = bx.n_pairs;
     out->n_bins = bx.n_bins;
-    out->kT = bx.kT;
     out->rho = (double)bx.n_atoms / bx.volume;
-    out->dr = bx.dr_A;
     return EPSR_OK;
 }
 
@@ -930,7 +928,6 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     a.pos_of = box->pos_of;
     a.boxes = box->boxes;
     a.coords = box->coords;
-    a.mol_start = box->mol_start;
     a.thresholds = box->thresholds;
     a.ep = box->ep;
     a.cta_box = box->cta_box;
@@ -939,7 +936,6 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
     a.stats = box->stats;
     a.log = log;
     a.status = box->status;
-    a.seed = seed;
     a.log_stride = n_moves;
     a.max_spin = 1LL << 40;
     a.timeout_ns = (unsigned long long)(box->timeout_ms * 1e6);
@@ -964,7 +960,6 @@ static int mc_sweep_enqueue(epsr_box *box, int64_t n_moves, uint64_t seed, uint6
                                  move0 + (uint64_t)c0, box->moves, s);
         if (rc) return rc;
         a.n_moves = n;
-        a.move0 = move0 + (uint64_t)c0;
         a.log_off = c0;
         CK(cudaMemsetAsync(box->flags, 0, box->cta_box_len * sizeof(unsigned), s));
         rc = launch_mc_sweep(a, box->cta_box_len, smem, s);

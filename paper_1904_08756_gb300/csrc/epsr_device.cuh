@@ -47,7 +47,6 @@ struct BoxDev {
     double dr_A;          // bin width in Angstrom (bin_p / bin_q)
     float inv_s2;         // 2^(-2 scale_log2): grid units^2 -> A^2
     float inv_dr_fx;      // 1 / (bin width in grid units)
-    uint32_t pre_r;       // g(r) prefilter half width on the 2^32-periodic scaled grid
     uint32_t pre16_bias;  // all-pairs histogram prefilter on the 2^16-periodic grid: bias B = R16 + 1
     uint32_t pre16_t;     // threshold T = 2 R16 + 1 in both halfwords
     int32_t pre16_all;    // 1: the cube covers the whole period (every pair takes the exact path)
@@ -434,16 +433,13 @@ __device__ __forceinline__ int ld_relaxed_gpu(const int *p)
 }
 
 // Host side: prefilter half widths of the all-pairs histogram. Every counted pair has
-// |dx| < R = ceil(sqrt(tmax)) + 1 grid units on each axis. On the 2^32-periodic grid
-// (x' = floor(x 2^32 / L)) that is |dx'| < R' = ceil(R 2^32 / L) + 2; on the 2^16-periodic
-// grid (x16 = x' >> 16) |dx16| <= R16 = ceil(R 2^16 / L) + 1, tested as the biased value
+// |dx| < R = ceil(sqrt(tmax)) + 1 grid units on each axis. On the 2^16-periodic grid
+// (x16 = floor(x 2^32 / L) >> 16) that is |dx16| <= R16 = ceil(R 2^16 / L) + 1, tested as the biased value
 // (x16_i + R16 + 1 - x16_j) mod 2^16 <= 2 R16 + 1. A pair at exactly |dx16| = R16 has
 // |dx| > R and is never counted.
 inline void set_prefilter(BoxDev &bx)
 {
     const double R = std::ceil(std::sqrt((double)bx.tmax)) + 1.0;
-    const double Rs = std::ceil(R * 4294967296.0 / (double)bx.L) + 2.0;
-    bx.pre_r = Rs >= 2147483647.0 ? 2147483647u : (unsigned)Rs;
     const double R16 = std::ceil(R * 65536.0 / (double)bx.L) + 1.0;
     if (2.0 * R16 + 1.0 <= 65534.0) {
         const uint32_t r16 = (uint32_t)R16, t = 2u * r16 + 1u;

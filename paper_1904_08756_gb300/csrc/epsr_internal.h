@@ -25,7 +25,7 @@ void note_launch();
 std::string box_shape_key(const epsr_box *box);
 struct BoxSummary {
     int n_boxes, n_pairs, n_bins;
-    double kT, rho, dr;     // kJ/mol, atoms per A^3, A
+    double rho;             // atoms per A^3
 };
 int box_summary(const epsr_box *box, int b, BoxSummary *out);
 int box_sms(const epsr_box *box);
@@ -53,7 +53,6 @@ constexpr int kMcMaxWords = 24;           // chunk mask words per CTA of such a 
 struct McArgs {
     const BoxDev *boxes;
     int4 *coords;                 // [n_atoms_total] {x, y, z, type}
-    const int *mol_start;         // concatenated box-local molecule starts
     const long long *thresholds;  // concatenated [n_bins + 1] per box
     const float *ep;              // concatenated [n_pairs * n_bins] per box
     const int *cta_box;           // [grid]
@@ -69,7 +68,6 @@ struct McArgs {
     long long log_off;            // log index of this launch's first move
     int *status;                  // device status word
     long long n_moves;
-    unsigned long long seed, move0;
     long long log_stride;
     long long max_spin;           // iteration limit of one barrier wait
     unsigned long long timeout_ns;// time limit of one barrier wait
@@ -93,7 +91,6 @@ int launch_mc_moves(const BoxDev *boxes, const int *mol_start, int n_boxes, long
                     cudaStream_t stream);
 int launch_intra_energy(const BoxDev *boxes, int n_boxes, const int4 *coords, const int *mol_start, double *U,
                         cudaStream_t stream);
-int mc_threads();
 int mc_escapee_max();
 int mc_batch_max();
 
@@ -281,9 +278,5 @@ struct ChiParams {
 };
 int launch_chi2(const float *S, const float *target, const float *Q, int nQ, const ChiParams &prm,
                 const double *C, double *chi2, float *dS, double *dC, cudaStream_t stream);
-
-// ---- S(Q) --------------------------------------------------------------------------------
-int sq_build_kernel_matrix(const float *Q, int nQ, int n_bins, double dr, int mode, float *K32,
-                           void *Ksplit, int ld_split, cudaStream_t stream);
 
 }  // namespace epsr

@@ -27,7 +27,7 @@ struct epsr_refiner {
     epsr_box *box = nullptr;
     epsr_sq_plan *plan = nullptr;
     int n_data = 0, P = 0, n_bins = 0, nQ = 0;
-    double kT = 0, rho = 0, dr = 0;
+    double rho = 0;
     epsr_refine_params prm{};
     std::vector<double> w, w_cols, flat;
     std::vector<float> Q;
@@ -121,9 +121,7 @@ extern "C" int epsr_refiner_create(epsr_box *box, epsr_sq_plan *plan, const floa
     r->P = bs.n_pairs;
     r->n_bins = bs.n_bins;
     r->nQ = nQ;
-    r->kT = bs.kT;
     r->rho = bs.rho;
-    r->dr = bs.dr;
     r->prm = *params;
     r->w.assign(w, w + (size_t)n_data * r->P);
     r->flat.assign(flat, flat + n_data);

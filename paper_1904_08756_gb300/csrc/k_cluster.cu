@@ -173,7 +173,7 @@ int launch_clusters(const BoxDev *boxes, const int *atom_box, const int4 *coords
 // a value of i and one of j, whatever the number of types), folded into the caller's pairs when it
 // leaves a box. The bin comes from the FP32 squared distance; within its error of a bin edge
 // (x 2^-20 of the distance x in bins; the errors of clusters.cuh, of sqrt_approx and of the scale
-// add up to less than x 2^-21) the exact integer distance and the threshold table decide.
+// add up to less than x (2^-22 + 2^-23 + 2 2^-23)) the exact integer distance and the threshold table decide.
 constexpr int kClThreads = 256;
 constexpr int kClWarps = kClThreads / 32;
 

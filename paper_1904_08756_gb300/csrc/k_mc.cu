@@ -1320,7 +1320,6 @@ int launch_mc_sweep(const McArgs &args, int grid, size_t smem, cudaStream_t stre
     return EPSR_OK;
 }
 
-int mc_threads() { return kMcThreads; }
 int mc_escapee_max() { return kEscMax; }
 int mc_batch_max() { return kBatchMax; }
 
