@@ -355,7 +355,7 @@ static void plan_mc_groups(epsr_box *h)
 // copy on the 2^32-periodic grid); otherwise the slices live in global memory, a part of the copy is
 // staged, and chunks double until their masks take at most kMcMaxWords words and everything fits.
 // Large empirical potentials leave the thresholds in global memory and shrink the stage: tables of up
-// to about 110 KB have room beside the least stage and four mask words.
+// to about 120 KB have room beside the least stage and a few mask words.
 struct McLayout {
     int slice_cap = 0, words_cap = 1, chunk_log = 5, stage = kMcStageChunk, tbl_cap = 0;
     size_t smem = 0;
@@ -397,7 +397,7 @@ static int mc_layout(const epsr_box *h, McLayout *L)
             L->tbl_cap = 0;
             tables = sizes(5);
         }
-        if (too_large()) L->stage = kMcStageLeast;
+        while (too_large() && L->stage > kMcStageLeast) L->stage /= 2;
         while ((L->words_cap > kMcMaxWords || total() > kMcMaxDynSmem) && L->words_cap > 1) tables = sizes(L->chunk_log + 1);
         L->smem = total();
         if (L->smem > kMcMaxDynSmem)

@@ -35,7 +35,7 @@ void sq_plan_dims(const epsr_sq_plan *p, int *nQ, int *n_bins, int *max_cols);
 int sq_plan_stages(const epsr_sq_plan *p);
 
 // ---- Monte Carlo kernel ----------------------------------------------------------------------
-constexpr size_t kMcMaxDynSmem = 156 * 1024;   // with about 69 KB of static shared memory, under the 227 KB per CTA
+constexpr size_t kMcMaxDynSmem = 161 * 1024;   // with 66 KB of static shared memory, under the 227 KB per CTA
 // exchange buffer of the sweep, per parity: the partial dU of every move of a batch from every
 // CTA ([kMcBatchMax][grid]), then kMcSlotStride - kMcBatchMax = kMcCorrPerCta floats per CTA of
 // which a box group uses its first CTA's share onwards for the batch-pair corrections
@@ -47,7 +47,7 @@ constexpr int kMcSlotStride = kMcBatchMax + kMcCorrPerCta;
 constexpr int kMcCorrItems = 4096;
 // partners staged at once in shared memory when the slices live in global memory, and with
 // empirical-potential tables that leave no room for as many
-constexpr int kMcStageChunk = 2048, kMcStageLeast = 512;
+constexpr int kMcStageChunk = 2048, kMcStageLeast = 256;
 constexpr int kMcMaxWords = 24;           // chunk mask words per CTA of such a slice, at most
 
 struct McArgs {

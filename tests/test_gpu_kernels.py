@@ -295,3 +295,18 @@ def test_sweep_small_boxes_replay():
         assert flips <= 2
         assert np.array_equal(xyz[a0:a0 + s.n_atoms], ob.xyz)
         a0 += s.n_atoms
+
+
+@pytest.mark.parametrize("types,bins,n", [(8, 848, 60), (7, 1080, 60), (6, 1440, 40), (8, 700, 3000)])
+def test_sweep_largest_tables_replay(types, bins, n):
+    """The largest empirical potentials that boxes were made with (122 KB at 8 types), in small boxes and with
+    slices in global memory: every move against the oracle."""
+    s = mixed_box([1], n, types, seed=types, n_bins=bins)
+    P = types * (types + 1) // 2
+    table = (np.random.default_rng(6).normal(size=(P, bins)) * 0.3).astype(np.float32)
+    box = epsr.Box(s)
+    box.epsr_box_set_ep(0, table)
+    _, log = run_logged(box, 400, seed=22)
+    ob, _, _, flips = replay(s, s.xyz, log[0], 22, ep=table.astype(np.float64))
+    assert flips <= 2
+    assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
