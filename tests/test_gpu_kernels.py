@@ -310,3 +310,39 @@ def test_sweep_largest_tables_replay(types, bins, n):
     ob, _, _, flips = replay(s, s.xyz, log[0], 22, ep=table.astype(np.float64))
     assert flips <= 2
     assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
+
+
+def test_histogram_of_a_mixed_handle():
+    """Both histogram entries on boxes of 900 to 12,000 atoms of one to three types, against the all-pairs kernel
+    over every tile and, box by box, the oracle."""
+    systems = [synth.water_box(300, seed=72, L_A=20.8), synth.water_box(3000, seed=73), synth.silica_box(600, seed=74),
+               synth.silica_box(4000, seed=75), synth.uniform_gas(1057, 24.0, seed=76, n_types=3),
+               synth.uniform_gas(40, 30.0, seed=77, n_types=1)]
+    box = epsr.Box(systems)
+    H = torch.zeros((3, box.hist_len), dtype=torch.int64, device=DEV)
+    box.epsr_partial_gr(H[0])
+    box.epsr_partial_gr_cells(H[1])
+    box.epsr_partial_gr_range(0, box.epsr_partial_gr_tiles(), H[2])
+    assert torch.equal(H[0], H[2]) and torch.equal(H[1], H[2])
+    h0 = 0
+    for s in systems:
+        ref = oracle.Box(s).histogram(threads=8)
+        assert np.array_equal(H[0, h0:h0 + ref.size].cpu().numpy().astype(np.uint64).reshape(ref.shape), ref)
+        h0 += ref.size
+
+
+@pytest.mark.parametrize("near_all,r_lj,ctas", [(True, 0.0, 0), (True, 6.0, 3), (False, 6.0, 1), (False, 0.0, 1)],
+                         ids=["near-all", "near-all-cut", "global-cut", "global"])
+def test_sweep_paths_replay(near_all, r_lj, ctas):
+    """Every chunk near, and slices in global memory (22,500 atoms on one CTA), with Lennard-Jones cut and not."""
+    n_mol = 1500 if near_all else 15000
+    s = mixed_box([1, 2], n_mol, 3, seed=31, n_bins=150, r_lj=r_lj)
+    box = epsr.Box(s)
+    if near_all:
+        box.epsr_mc_set_cells(0, 0)
+    if ctas:
+        box.epsr_mc_set_ctas(ctas)
+    _, log = run_logged(box, 500, seed=23)
+    ob, _, _, flips = replay(s, s.xyz, log[0], 23)
+    assert flips <= 2
+    assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
