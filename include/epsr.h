@@ -330,7 +330,8 @@ int epsr_sq_weights(const epsr_box *box, int32_t b, double *w, double *flat);
  * adds to bin k the mass of a Gaussian of width sigma centred on r, truncated at +-5 sigma,
  *   w_k(r) = Phi(clip((r_{k+1} - r)/sigma)) - Phi(clip((r_k - r)/sigma)),  clip to [-5, 5].
  * epsr_gr_smeared_fwd: Ht device double [hist_len] (overwritten); gt device float [hist_len]
- *   or NULL: the smeared g~ = Ht V / (P_ab shell_k), normalised like epsr_partial_gr's g.
+ *   or NULL: the smeared g~ = Ht V / (P_ab shell_k), normalised like epsr_partial_gr's g. The
+ *   result is the same bits in every call on the same coordinates.
  * epsr_gr_smeared_bwd: given dL/dg~ (device float [hist_len]) writes dL/dx, device float
  *   [n_atoms_total][3] per Angstrom (overwritten). Pair distances are recomputed.
  * epsr_sq_exec_adjoint: dg[c][k] = w_c sum_i K[i][k] dS_total[set(c)][i], the adjoint of
