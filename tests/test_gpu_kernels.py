@@ -346,3 +346,19 @@ def test_sweep_paths_replay(near_all, r_lj, ctas):
     ob, _, _, flips = replay(s, s.xyz, log[0], 23)
     assert flips <= 2
     assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
+
+
+@pytest.mark.parametrize("sizes,n_mol,ctas,r_lj,moves", [([1], 700, 0, 4.0, 6000), ([1], 700, 1, 0.0, 4000), ([2, 3], 250, 5, 0.0, 4000),
+                                                         ([1], 3000, 0, 4.0, 6000)])
+def test_large_steps_replay(sizes, n_mol, ctas, r_lj, moves):
+    """Steps of 2 A in a dense box: trials land on top of molecules that an earlier move of the batch takes away,
+    so a dU of a few kJ/mol is what is left of 10^4 and more. Every move against the oracle, with the bars of all replays."""
+    s = mixed_box(sizes, n_mol, 2, seed=n_mol, n_bins=100, spacing=3.2, r_lj=r_lj)
+    s.r_coul, s.eps, s.max_translation = 0.0, [0.4, 0.4], 2.0
+    box = epsr.Box(s)
+    if ctas:
+        box.epsr_mc_set_ctas(ctas)
+    _, log = run_logged(box, moves, seed=24)
+    ob, _, _, flips = replay(s, s.xyz, log[0], 24)
+    assert flips <= 2
+    assert np.array_equal(box.epsr_box_get_coords(), ob.xyz)
