@@ -217,9 +217,9 @@ __device__ __forceinline__ bool metropolis(float d, float thr) { return (d <= 0.
 
 // True when the corrections of the accepted moves, of magnitude w in all, cancel the batch-start value d
 // of a move down to f: what the FP32 sums of d lost below 2^-24 of it would then show in f. The bar is
-// a rounding of 6e-5 kJ/mol, and 4e-6 of f: below that f is as good as any FP32 sum. Steps of 2 A in dense
-// boxes: worst error over the bar of 1e-5 of the condition scale + 1e-4, 15 -> 0.2 (10 and more without
-// the cut at 16 moves a batch too, 260 at 64); 99,999-atom water 751 -> 754 us for 3,000 moves.
+// a rounding of 6e-5 kJ/mol, and 4e-6 of f: below that f is as good as any FP32 sum. Random boxes with
+// steps up to 2 A, worst error against 1e-5 of the condition scale + 1e-4 kJ/mol: 260 times without the cut
+// (15 times with batches of 16), 0.2 with it. 99,999-atom water 751 -> 754 us for 3,000 moves.
 constexpr float kCancelled = 512.f;
 __device__ __forceinline__ bool cancelled(float d, float w, float f)
 {
